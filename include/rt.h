@@ -154,7 +154,7 @@ int rt_set_precision(rt_grid *g, int precision);
  * streams per-segment weights (E, alpha, beta, gamma) evaluated once per chi
  * in FP64 and the gather weight w l / L: as FP32 for RT_MIXED (16 extra bytes
  * per segment of device memory with the gather weight folded in, see
- * RT_TUNE_FOLD_WEIGHT; 20 without), as FP64 for RT_FP64 (40 bytes), each
+ * RT_TUNE_FOLD_WEIGHT; 20 without), as FP64 for RT_FP64 (48 bytes), each
  * allocated at its first use; 0, or when that memory is not available: the
  * march evaluates the weights itself from chi and l.
  * RT_TUNE_MARCH_COARSEN: segments per lane of the streamed-weight march, 1
@@ -186,8 +186,8 @@ int rt_set_precision(rt_grid *g, int precision);
  * sweeps of an RT_MIXED rt_solve, whose right-hand sides carry FP32 rounding,
  * the bound is max(10^-value, 1e-8); its FP64 residual steps use 10^-value. */
 #define RT_TUNE_NN_JTOL 8
-/* RT_TUNE_MARCH64_COARSEN: segments per lane of the FP64 streamed-weight
- * march, 1 or 2 (default). */
+/* RT_TUNE_MARCH64_COARSEN: 1 or 2, accepted and without effect (the FP64
+ * streamed-weight march runs one characteristic per lane). */
 #define RT_TUNE_MARCH64_COARSEN 9
 /* RT_TUNE_MARCH_LOOKAHEAD (default 1): the register-prefetch FP32 march loads
  * the voxel words two tiles ahead and issues the S lookups of the next tile
@@ -508,7 +508,7 @@ typedef struct rt_timing {
     int64_t kernel_launches;  /* every kernel this library launched on the grid since the reset */
     int64_t march_bytes;      /* DRAM bytes the timed march launches stream by design (per segment:
                                  8 FP32, 12 FP64; streamed-weight FP32 24, or 20 without RT_TUNE_SCATTER,
-                                 4 more without RT_TUNE_FOLD_WEIGHT; streamed-weight FP64 48 / 44) */
+                                 4 more without RT_TUNE_FOLD_WEIGHT; streamed-weight FP64 48) */
     double os_ms;             /* summed event time of the nearest-neighbour OS-step solves (timing 1 only) */
     int64_t os_solves;        /* OS-step solves since the reset (counted at any timing setting) */
     int64_t os_krylov_its;    /* their BiCGSTAB iterations */

@@ -388,6 +388,11 @@ int adjoint_pass(rt_grid *g, bool full, int homog, const double *u, const double
                  double *tB, double *oS, double *oC, double *oB)
 {
     const int n = g->nvox;
+    if (!full) {  // Lambda^T depends on chi only: the weights streamed for the FP64 formal solutions serve it
+        bool done = false;
+        const int rc = rt_grid_adjoint_ray64(g, u, gc, oS, &done);
+        if (rc != RT_OK || done) return rc;
+    }
     ACK(pack_chiS64(n, g->d_chi, g->d_S, g->d_cs64, g->st));
     for (int b = 0; b < g->nblk; ++b) {
         const int w0 = g->blk_w0[b], nw = g->blk_nw[b];

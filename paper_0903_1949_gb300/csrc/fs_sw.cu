@@ -1,6 +1,6 @@
 // fs_sw.cu -- J-only formal solution of the ALI iteration with streamed
-// segment weights (the hot loop of the mixed-precision path, FP32; the same
-// march in FP64 for the FP64 path).
+// segment weights (the hot loop of the mixed-precision path, FP32; the FP64
+// march is in ray64.cu, its gathers are here).
 //
 // The weights of a segment in the recurrence I_k = I_{k-1} E_k + alpha_k
 // S_{k-1} + beta_k S_k + gamma_k S_{k+1} (scheme R6 of Papers I-II, Sect. 2)
@@ -119,13 +119,6 @@ __global__ void k_bundles(const int64_t *ray_off, int64_t r_lo, int64_t r_hi, in
 // I -> A I + b composed by an inclusive shuffle scan over the warp; the next
 // tile's words and weights are fetched before the current one is processed.
 __device__ __forceinline__ float4 ldw(const float4 *p) { return __ldcs(p); }
-__device__ __forceinline__ Wd4 ldw(const Wd4 *p)
-{
-    const double2 a = __ldcs(reinterpret_cast<const double2 *>(p));
-    const double2 b = __ldcs(reinterpret_cast<const double2 *>(p) + 1);
-    return Wd4{a.x, a.y, b.x, b.y};
-}
-
 // SLA: the S lookups of tile t + 1 are issued while tile t is marched (its
 // words are loaded two tiles ahead), so no tile waits for its own lookups.
 // FOLD: the weights carry the gather weight (k_coef_stream_fold); the c stream
@@ -762,40 +755,6 @@ __global__ void k_coef_stream_fold(const uint32_t *__restrict__ vox, const doubl
     }
 }
 
-// FP64 weights of every segment for the current chi (FP64 streamed march).
-__global__ void k_coef_stream64(const uint32_t *__restrict__ vox, const double *__restrict__ len64,
-                                const double *__restrict__ chi, int64_t nseg, Wd4 *__restrict__ cw)
-{
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nseg; s += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t w = vox[s];
-        const bool para = (w & RTK_PARA) != 0u;
-        const double x = chi[w & RTK_VOXMASK] * len64[s];
-        const double p = para ? chi[vox[s + 1] & RTK_VOXMASK] * len64[s + 1] : 0.0;
-        double E, al, be, ga;
-        Coef64::eval(x, p, para, E, al, be, ga);
-        if (w & (RTK_RAYSTART | RTK_RESTART)) {
-            be += al;
-            al = 0.0;
-        }
-        cw[s] = Wd4{E, al, be, ga};
-    }
-}
-
-__global__ void k_seg_weight64(const uint32_t *__restrict__ vox, const double *__restrict__ len64,
-                               const int64_t *__restrict__ ang_seg_off, int n_ang, const double *__restrict__ wt,
-                               const double *__restrict__ invL, int nvox, int64_t nseg, double *__restrict__ cg)
-{
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nseg; s += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = n_ang;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (ang_seg_off[mid] <= s) lo = mid;
-            else hi = mid;
-        }
-        cg[s] = wt[lo] * len64[s] * invL[(int64_t)lo * nvox + (vox[s] & RTK_VOXMASK)];
-    }
-}
-
 // Gather weight times path length of every segment: w_Omega l_s / L_{Omega v_s}.
 __global__ void k_seg_weight(const uint32_t *__restrict__ vox, const double *__restrict__ len64,
                              const int64_t *__restrict__ ang_seg_off, int n_ang, const double *__restrict__ wt,
@@ -947,31 +906,6 @@ cudaError_t gather_sw_launch(const SwGather &t, cudaStream_t st)
     if (grid <= 0) return cudaSuccess;
     if (t.buf64) k_gather_sw<double><<<(unsigned)grid, 256, 0, st>>>(t);
     else k_gather_sw<float><<<(unsigned)grid, 256, 0, st>>>(t);
-    return cudaGetLastError();
-}
-
-cudaError_t march_sw64_launch(const SwMarch64 &m, int coarsen, cudaStream_t st)
-{
-    const int64_t grid = (m.nbundles + 7) / 8;
-    if (grid <= 0) return cudaSuccess;
-    if (coarsen == 2) k_march_sw<SwMarch64, 2, false><<<(unsigned)grid, 256, 0, st>>>(m);
-    else k_march_sw<SwMarch64, 1, false><<<(unsigned)grid, 256, 0, st>>>(m);
-    return cudaGetLastError();
-}
-
-cudaError_t coef_stream64(const uint32_t *vox, const double *len64, const double *chi, int64_t nseg, Wd4 *cw,
-                          cudaStream_t st)
-{
-    if (nseg <= 0) return cudaSuccess;
-    k_coef_stream64<<<grid_cap(nseg), 256, 0, st>>>(vox, len64, chi, nseg, cw);
-    return cudaGetLastError();
-}
-
-cudaError_t seg_weight64(const uint32_t *vox, const double *len64, const int64_t *ang_seg_off, int n_ang,
-                         const double *wt, const double *invL, int nvox, int64_t nseg, double *cg, cudaStream_t st)
-{
-    if (nseg <= 0) return cudaSuccess;
-    k_seg_weight64<<<grid_cap(nseg), 256, 0, st>>>(vox, len64, ang_seg_off, n_ang, wt, invL, nvox, nseg, cg);
     return cudaGetLastError();
 }
 

@@ -79,10 +79,16 @@ struct rt_grid {
     float *d_cg = nullptr;    // w_Omega l / L per segment
     int sw_enabled = 1;
     int sw_state = 0;         // 0 not allocated yet, 1 allocated, -1 allocation failed
-    rtk::Wd4 *d_cw64 = nullptr;  // FP64 weights per segment (FP64 streamed march)
-    double *d_cg64 = nullptr;    // FP64 w l / L per segment
+    // FP64 streamed march (ray64.cu): the characteristics sorted by length within their
+    // angle blocks, and the streams of their groups of 32
+    int32_t *d_rorder = nullptr, *d_rlen = nullptr;
+    int64_t *d_rgbase = nullptr;
+    std::vector<int64_t> h_rg0;  // first group of every block (nblk + 1)
+    uint2 *d_wp64 = nullptr;     // segment word and output position
+    rtk::Wd4 *d_cw64 = nullptr;  // FP64 weights
+    double *d_cg64 = nullptr;    // FP64 w l / L
     int sw64_state = 0;
-    int sw64_coarsen = 2;     // segments per lane of the FP64 streamed march (RT_TUNE_MARCH64_COARSEN)
+    int wp64_pos = -1;           // output positions in d_wp64: 1 list order, 0 segment order, -1 not filled
     bool cw64_ok = false;
     int pos_state = 0;        // list positions: 0 not tried, 1 allocated, -1 not available
     bool cw_ok = false;       // d_cw4 matches the current chi
@@ -145,6 +151,11 @@ int rt_grid_member_fs(rt_grid *g, const float2 *cs, const float *B32, const uint
 // The grid's exact nearest-neighbour Lambda* (d_L27) for its current chi, built
 // on first use after rt_set_opacity; returns an RT_ status.
 int rt_grid_build_nn(rt_grid *g);
+
+// y = Lambda^T u (plus Lambda_F^T gc when gc is not NULL) by the streamed-weight
+// transpose of the FP64 march, on the grid's stream.  *done = false (and
+// nothing written) when the streamed weights are off or do not fit.
+int rt_grid_adjoint_ray64(rt_grid *g, const double *u, const double *gc, double *y, bool *done);
 
 // FP64 J of another opacity field on this grid's geometry (a batch member):
 // (chi, S) packed in cs64, B, parabola choices in pbits.  Runs on st.

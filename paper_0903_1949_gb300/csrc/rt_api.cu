@@ -872,39 +872,136 @@ bool use_sw(rt_grid *g)
     return sw_common(g);
 }
 
-// FP64 streamed weights (40 bytes per segment), the same life cycle.
+// One angle block of the FP64 streamed march.
+Ray64 ray64_block(rt_grid *g, int b)
+{
+    Ray64 m{};
+    const int w0 = g->blk_w0[b], nw = g->blk_nw[b];
+    m.r_lo = g->h_ang_ray_off[w0];
+    m.r_hi = g->h_ang_ray_off[w0 + nw];
+    m.seg_lo = g->h_ang_seg_off[w0];
+    m.ngroups = g->h_rg0[b + 1] - g->h_rg0[b];
+    m.ray_off = g->d_ray_off;
+    m.order = g->d_rorder;
+    m.olen = g->d_rlen;
+    m.gbase = g->d_rgbase + g->h_rg0[b];
+    m.wp = g->d_wp64;
+    m.cw = g->d_cw64;
+    m.cg = g->d_cg64;
+    return m;
+}
+
+// Device memory that lives as long as the grid, counted; NULL when it does not fit.
+void *keep_alloc(rt_grid *g, size_t bytes)
+{
+    void *q = nullptr;
+    if (cudaMalloc(&q, std::max<size_t>(1, bytes)) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    g->allocs.push_back(q);
+    g->bytes += (int64_t)bytes;
+    return q;
+}
+
+// The slots of the FP64 streamed march (once per grid): characteristics sorted
+// by length within their angle blocks, groups of 32, one slot per step and
+// characteristic.  false when the arrays do not fit.
+bool ray64_setup(rt_grid *g)
+{
+    const int cap = geom_scratch_cap(g->G);  // no characteristic is longer
+    const int64_t nh = (int64_t)g->nblk * (cap + 1);
+    g->h_rg0.assign(g->nblk + 1, 0);
+    for (int b = 0; b < g->nblk; ++b) {
+        const int64_t nr = g->h_ang_ray_off[g->blk_w0[b] + g->blk_nw[b]] - g->h_ang_ray_off[g->blk_w0[b]];
+        g->h_rg0[b + 1] = g->h_rg0[b] + (nr + 31) / 32;
+    }
+    const int64_t ng = g->h_rg0[g->nblk];
+    struct Tmp {
+        std::vector<void *> v;
+        ~Tmp()
+        {
+            for (void *q : v) cudaFree(q);
+        }
+        void *get(size_t bytes)
+        {
+            void *q = nullptr;
+            if (cudaMalloc(&q, bytes) != cudaSuccess) {
+                cudaGetLastError();
+                return nullptr;
+            }
+            v.push_back(q);
+            return q;
+        }
+    } tmp;
+    int32_t *hist = (int32_t *)tmp.get(4 * nh), *gw = (int32_t *)tmp.get(4 * std::max<int64_t>(1, ng));
+    int64_t *cursor = (int64_t *)tmp.get(8 * (nh + 1));
+    int64_t *stmp = (int64_t *)tmp.get(8 * (size_t)scan_tmp_elems(std::max(nh, ng)));
+    g->d_rorder = (int32_t *)keep_alloc(g, 4 * (size_t)g->n_rays);
+    g->d_rlen = (int32_t *)keep_alloc(g, 4 * (size_t)g->n_rays);
+    g->d_rgbase = (int64_t *)keep_alloc(g, 8 * (size_t)(ng + 1));
+    if (!hist || !gw || !cursor || !stmp || !g->d_rorder || !g->d_rlen || !g->d_rgbase) return false;
+    if (cudaMemsetAsync(hist, 0, 4 * nh, g->st) != cudaSuccess ||
+        ray64_hist(g->n_rays, g->d_ray_off, g->d_ray_angle, g->ablk, cap, hist, g->st) != cudaSuccess ||
+        scan_i32(hist, cursor, nh, stmp, g->st) != cudaSuccess ||
+        ray64_place(g->n_rays, g->d_ray_off, g->d_ray_angle, g->ablk, cap, cursor, g->d_rorder, g->d_rlen, g->st) !=
+            cudaSuccess)
+        return false;
+    for (int b = 0; b < g->nblk; ++b)
+        if (ray64_group_slots(g->h_ang_ray_off[g->blk_w0[b]], g->h_rg0[b + 1] - g->h_rg0[b], g->d_rlen,
+                              gw + g->h_rg0[b], g->st) != cudaSuccess)
+            return false;
+    int64_t slots = 0;
+    if (scan_i32(gw, g->d_rgbase, ng, stmp, g->st) != cudaSuccess ||
+        cudaMemcpyAsync(&slots, g->d_rgbase + ng, sizeof(int64_t), cudaMemcpyDeviceToHost, g->st) != cudaSuccess ||
+        cudaStreamSynchronize(g->st) != cudaSuccess)
+        return false;
+    g->launches += 6 + g->nblk;
+    g->d_wp64 = (uint2 *)keep_alloc(g, sizeof(uint2) * (size_t)slots);
+    g->d_cw64 = (Wd4 *)keep_alloc(g, sizeof(Wd4) * (size_t)slots);
+    g->d_cg64 = (double *)keep_alloc(g, sizeof(double) * (size_t)slots);
+    return g->d_wp64 && g->d_cw64 && g->d_cg64;
+}
+
+// FP64 streamed weights (48 bytes per slot), the same life cycle.
 bool use_sw64(rt_grid *g)
 {
     if (!g->sw_enabled || g->sw64_state < 0) return false;
     if (g->sw64_state == 0) {
-        void *a = nullptr, *b = nullptr;
-        if (cudaMalloc(&a, sizeof(Wd4) * (size_t)g->n_seg) != cudaSuccess ||
-            cudaMalloc(&b, sizeof(double) * (size_t)(g->n_seg + 4)) != cudaSuccess) {
+        if (!ray64_setup(g)) {
+            for (void *q : {(void *)g->d_rorder, (void *)g->d_rlen, (void *)g->d_rgbase, (void *)g->d_wp64,
+                            (void *)g->d_cw64, (void *)g->d_cg64})
+                dfree(g, q);
+            g->d_rorder = g->d_rlen = nullptr;
+            g->d_rgbase = nullptr;
+            g->d_wp64 = nullptr;
+            g->d_cw64 = nullptr;
+            g->d_cg64 = nullptr;
             cudaGetLastError();
-            if (a) cudaFree(a);
             g->sw64_state = -1;
             return false;
         }
-        g->allocs.push_back(a);
-        g->allocs.push_back(b);
-        g->bytes += (int64_t)(40 * g->n_seg);
-        g->d_cw64 = (Wd4 *)a;
-        g->d_cg64 = (double *)b;
-        if (seg_weight64(g->d_vox, g->d_len64, g->d_ang_seg_off, g->n_ang, g->d_wt, g->d_invL, g->nvox, g->n_seg,
-                         g->d_cg64, g->st) != cudaSuccess) {
-            g->sw64_state = -1;
-            return false;
-        }
-        g->launches++;
         g->sw64_state = 1;
+        g->wp64_pos = -1;
         g->cw64_ok = false;
     }
+    if (!sw_common(g)) return false;
+    const int pos = g->sw_scatter && g->d_pos ? 1 : 0;
+    if (g->wp64_pos != pos) {
+        for (int b = 0; b < g->nblk; ++b)
+            if (ray64_fill(ray64_block(g, b), g->d_vox, g->d_len64, pos ? g->d_pos : nullptr, g->d_ray_angle, g->d_wt,
+                           g->d_invL, g->nvox, g->st) != cudaSuccess)
+                return false;
+        g->launches += g->nblk;
+        g->wp64_pos = pos;
+    }
     if (!g->cw64_ok) {
-        if (coef_stream64(g->d_vox, g->d_len64, g->d_chi, g->n_seg, g->d_cw64, g->st) != cudaSuccess) return false;
-        g->launches++;
+        for (int b = 0; b < g->nblk; ++b)
+            if (ray64_coef(ray64_block(g, b), g->d_vox, g->d_len64, g->d_chi, g->st) != cudaSuccess) return false;
+        g->launches += g->nblk;
         g->cw64_ok = true;
     }
-    return sw_common(g);
+    return true;
 }
 
 // Blocked voxel order for the FP32 march's S lookups (once per grid): slots of
@@ -983,25 +1080,6 @@ SwMarch sw_march(rt_grid *g, int b, int homog, float *out)
     return m;
 }
 
-SwMarch64 sw_march64(rt_grid *g, int b, int homog, double *out)
-{
-    SwMarch64 m{};
-    const int w0 = g->blk_w0[b];
-    m.vox = g->d_vox;
-    m.cw = g->d_cw64;
-    m.cg = g->d_cg64;
-    m.bnd = g->d_bnd + g->h_bnd_off[b];
-    m.pos = (g->sw_scatter && g->d_pos) ? g->d_pos : nullptr;
-    m.seg_lo = g->h_ang_seg_off[w0];
-    m.nbundles = g->h_bnd_off[b + 1] - g->h_bnd_off[b];
-    m.S = nullptr;  // set by the caller (the S of this formal solution)
-    m.B = g->d_B;
-    m.I_outer = g->I_outer;
-    m.homog = homog;
-    m.out = out;
-    return m;
-}
-
 SwGather sw_gather(rt_grid *g, int b, const float *buf, double *J)
 {
     SwGather t{};
@@ -1047,15 +1125,13 @@ int run_fs_J_sw(rt_grid *g, int prec, int homog, const double *S_src, double *J)
                      (float *)g->d_segbuf + 2 * g->max_blk_seg};
     double *b64[2] = {(double *)g->d_segbuf, (double *)g->d_segbuf + g->max_blk_seg};
     const bool fold = !f64 && g->sw_fold && g->sw_stages == 0;  // no separate gather-weight stream
-    const int64_t bps = (f64 ? (scatter ? 48 : 44) : (scatter ? 28 : 24)) - (fold ? 4 : 0);  // streamed bytes per segment
+    const int64_t bps = f64 ? 48 : (scatter ? 28 : 24) - (fold ? 4 : 0);  // streamed bytes per segment
     auto segs = [&](int b) -> int64_t {
         return g->h_ang_seg_off[g->blk_w0[b] + g->blk_nw[b]] - g->h_ang_seg_off[g->blk_w0[b]];
     };
     auto march = [&](int b, int q, cudaStream_t st) -> cudaError_t {
         if (!f64) return march_sw_launch(sw_march(g, b, homog, b32[q]), g->sw_coarsen, st);
-        SwMarch64 m = sw_march64(g, b, homog, b64[q]);
-        m.S = S_src;
-        return march_sw64_launch(m, g->sw64_coarsen, st);
+        return ray64_march(ray64_block(g, b), S_src, g->d_B, g->I_outer, homog, b64[q], st);
     };
     auto gather = [&](int b, int q, cudaStream_t st) -> cudaError_t {
         SwGather t = sw_gather(g, b, b32[q], J);
@@ -1142,7 +1218,7 @@ int run_fs_J_sw_streams(rt_grid *g, int prec, int homog, const double *S_src, do
                      (float *)g->d_segbuf + 2 * g->max_blk_seg};
     double *b64[2] = {(double *)g->d_segbuf, (double *)g->d_segbuf + g->max_blk_seg};
     const bool fold = !f64 && g->sw_fold && g->sw_stages == 0;  // no separate gather-weight stream
-    const int64_t bps = (f64 ? (scatter ? 48 : 44) : (scatter ? 28 : 24)) - (fold ? 4 : 0);  // streamed bytes per segment
+    const int64_t bps = f64 ? 48 : (scatter ? 28 : 24) - (fold ? 4 : 0);  // streamed bytes per segment
     auto segs = [&](int b) -> int64_t {
         return g->h_ang_seg_off[g->blk_w0[b] + g->blk_nw[b]] - g->h_ang_seg_off[g->blk_w0[b]];
     };
@@ -1152,9 +1228,7 @@ int run_fs_J_sw_streams(rt_grid *g, int prec, int homog, const double *S_src, do
     }
     auto march = [&](int b, int q, cudaStream_t st) -> cudaError_t {
         if (!f64) return march_sw_launch(sw_march(g, b, homog, b32[q]), g->sw_coarsen, st);
-        SwMarch64 m = sw_march64(g, b, homog, b64[q]);
-        m.S = S_src;
-        return march_sw64_launch(m, g->sw64_coarsen, st);
+        return ray64_march(ray64_block(g, b), S_src, g->d_B, g->I_outer, homog, b64[q], st);
     };
     auto gather = [&](int b, int q, cudaStream_t st) -> cudaError_t {
         SwGather t = sw_gather(g, b, b32[q], J);
@@ -1504,6 +1578,25 @@ int rt_grid_member_fs(rt_grid *g, const float2 *cs, const float *B32, const uint
 
 int rt_grid_build_nn(rt_grid *g) { return build_nn(g); }
 
+int rt_grid_adjoint_ray64(rt_grid *g, const double *u, const double *gc, double *y, bool *done)
+{
+    *done = false;
+    if (!use_sw64(g)) {
+        CK(cudaGetLastError());
+        return RT_OK;
+    }
+    double *buf = (double *)g->d_segbuf;
+    for (int b = 0; b < g->nblk; ++b) {
+        CK(ray64_adjoint(ray64_block(g, b), u, gc, g->d_dirs, g->d_ray_angle, buf, g->st));
+        SwGather t = sw_gather(g, b, nullptr, y);
+        t.buf64 = buf;
+        CK(g->wp64_pos ? gather_rows_sw_launch(t, g->nvox, g->st) : gather_sw_launch(t, g->st));
+        g->launches += 2;
+    }
+    *done = true;
+    return RT_OK;
+}
+
 int rt_grid_member_fs64J(rt_grid *g, const double2 *cs64, const double *B64, const uint32_t *pbits, double *J,
                          cudaStream_t st)
 {
@@ -1688,8 +1781,7 @@ int rt_tune(rt_grid *g, int knob, int value)
     }
     if (knob == RT_TUNE_MARCH64_COARSEN) {
         if (value != 1 && value != 2) return fail(RT_EINVAL, "FP64 march coarsening must be 1 or 2");
-        g->sw64_coarsen = value;
-        return RT_OK;
+        return RT_OK;  // one characteristic per lane: no segments per lane to choose
     }
     if (knob == RT_TUNE_MARCH_STAGES) {
         if (value != 0 && (value < 2 || value > 4)) return fail(RT_EINVAL, "march stages: 0 or 2..4");

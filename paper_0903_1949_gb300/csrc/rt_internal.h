@@ -230,22 +230,37 @@ struct SwMarch {
 struct alignas(32) Wd4 {
     double x, y, z, w;
 };
-// The same march in FP64 (streamed FP64 weights and w l / L).
-struct SwMarch64 {
-    using T = double;
-    using W = Wd4;
-    const uint32_t *vox;
-    const Wd4 *cw;
-    const double *cg;
-    const int2 *bnd;
-    const int32_t *pos;
-    int64_t seg_lo, nbundles;
-    const double *S;
-    const double *B;
-    double I_outer;
-    int homog;
-    double *out;
+// One angle block of the FP64 march with one characteristic per lane (ray64.cu):
+// the block's characteristics [r_lo, r_hi) sorted by length (order, olen), 32 to
+// a group, the streams at slot gbase[g] + 32 k + lane.
+struct Ray64 {
+    int64_t r_lo, r_hi, seg_lo, ngroups;
+    const int64_t *ray_off;
+    const int32_t *order, *olen;
+    const int64_t *gbase;  // of this block's groups
+    uint2 *wp;             // segment word (flags RAYSTART, CORE, RESTART) and output position
+    Wd4 *cw;
+    double *cg;            // w_Omega l / L
 };
+// Counting sort of the characteristics by length within their angle blocks
+// (blocks of ablk solid angles): hist holds cap + 1 lengths per block, its
+// exclusive scan is the cursor.
+cudaError_t ray64_hist(int64_t n_rays, const int64_t *ray_off, const int32_t *ray_angle, int ablk, int cap,
+                       int32_t *hist, cudaStream_t st);
+cudaError_t ray64_place(int64_t n_rays, const int64_t *ray_off, const int32_t *ray_angle, int ablk, int cap,
+                        int64_t *cursor, int32_t *order, int32_t *olen, cudaStream_t st);
+cudaError_t ray64_group_slots(int64_t r_lo, int64_t ngroups, const int32_t *olen, int32_t *gw, cudaStream_t st);
+// Words, output positions (pos, or the segment's place in its block when NULL)
+// and gather weights; once per grid.  Weights; once per chi.
+cudaError_t ray64_fill(const Ray64 &m, const uint32_t *vox, const double *len64, const int32_t *pos,
+                       const int32_t *ray_angle, const double *wt, const double *invL, int nvox, cudaStream_t st);
+cudaError_t ray64_coef(const Ray64 &m, const uint32_t *vox, const double *len64, const double *chi, cudaStream_t st);
+cudaError_t ray64_march(const Ray64 &m, const double *S, const double *B, double I_outer, int homog, double *out,
+                        cudaStream_t st);
+// out = the block's per-segment shares of Lambda^T u (plus Lambda_F^T gc, the
+// Cartesian flux adjoint, when gc is not NULL).
+cudaError_t ray64_adjoint(const Ray64 &m, const double *u, const double *gc, const double *dirs,
+                          const int32_t *ray_angle, double *out, cudaStream_t st);
 struct SwGather {
     const int32_t *off, *jorder, *jsell, *crow, *cbeg, *clr, *lfirst, *perm;
     const int64_t *jgbase;
@@ -266,13 +281,6 @@ cudaError_t blk_scatter(int nvox, const int32_t *vblk, const float *S, const flo
 cudaError_t sw_bundles(const int64_t *ray_off, int64_t r_lo, int64_t r_hi, int64_t seg_lo, int64_t nseg, int chunk,
                        int2 *bnd, cudaStream_t st);
 cudaError_t march_sw_launch(const SwMarch &m, int coarsen, cudaStream_t st);
-// coarsen: segments per lane, 1 or 2.
-cudaError_t march_sw64_launch(const SwMarch64 &m, int coarsen, cudaStream_t st);
-// FP64 weights and w l / L per segment for the FP64 streamed march.
-cudaError_t coef_stream64(const uint32_t *vox, const double *len64, const double *chi, int64_t nseg, Wd4 *cw,
-                          cudaStream_t st);
-cudaError_t seg_weight64(const uint32_t *vox, const double *len64, const int64_t *ang_seg_off, int n_ang,
-                         const double *wt, const double *invL, int nvox, int64_t nseg, double *cg, cudaStream_t st);
 cudaError_t gather_sw_launch(const SwGather &t, cudaStream_t st);
 // J from values in ownership-list order (march with pos): contiguous rows.
 cudaError_t gather_rows_sw_launch(const SwGather &t, int nvox, cudaStream_t st);
