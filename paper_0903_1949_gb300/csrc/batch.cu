@@ -464,6 +464,11 @@ int line_nn_os(rt_batch *b)
     o.jmax = 100000;
     o.krylov = 1;
     o.kmax = 1000;
+    // At chi_l / chi_c = 1e6 and eps_l = 1e-4 the operator is so ill-conditioned that
+    // two solves which both meet the 1e-14 criterion differ by 1e-5 to 2e-5 of S_l;
+    // (rh, r) taken directly keeps the iterates the ones this solve has always given,
+    // and the solve is a few percent of a line step.
+    o.own_rho = 1;
     double *x = nullptr;
     int its = 0, sweeps = 0, status = 0;
     BCK(nn_os_solve(o, b->st, &x, &its, &sweeps, &status));

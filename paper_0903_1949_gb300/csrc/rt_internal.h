@@ -367,6 +367,8 @@ struct NnOs {
     double jtol;
     int jmax, krylov, kmax;
     int stall;
+    int own_rho;  // != 0: rho of the FP32 BiCGSTAB from a dot product of its own (three reductions an
+                  // iteration instead of two), see rt_line_step's solve
 };
 int64_t nn_os_work_elems(int nvox);
 cudaError_t nn_os_solve(const NnOs &o, cudaStream_t st, double **x_out, int *krylov_its, int *sweeps, int *status);
