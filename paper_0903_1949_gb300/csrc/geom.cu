@@ -358,6 +358,8 @@ __device__ int walk(const GeomDev &G, double x0, double y0, double z0, double dx
     return RTK_END_LOST;
 }
 
+#include "geom_fast.cuh"
+
 __device__ __forceinline__ void ijk_of(const GeomDev &G, int v, int &i, int &j, int &k)
 {
     k = v % G.n3;
@@ -393,7 +395,7 @@ __device__ __forceinline__ bool core_launch(const GeomDev &G, int i, int j, int 
 struct MarkVisit {
     uint32_t *H;
     int n;
-    __device__ void cell(int v, double, double, int)
+    __device__ void cell(int v)
     {
         atomicOr(H + (v >> 5), 1u << (v & 31));
         n++;
@@ -479,14 +481,41 @@ struct FwdWrite {
     }
 };
 
-__global__ void k_mark_boundary(GeomDev G, const double *dirs, int w0, int nw, uint32_t *hit, int words, int *lost,
-                                uint32_t *cnt)
+// Voxels that may start a characteristic, without repeats: the outermost shell
+// (or cylinder), the innermost one, and on the cylindrical grid the two end
+// planes of the shells between.
+__device__ __forceinline__ int n_boundary(const GeomDev &G)
 {
-    int64_t total = (int64_t)nw * G.nvox;
+    const int face = G.n2 * G.n3, inner = G.n1 > 1 ? face : 0;
+    const int between = G.coord == RT_SPHERICAL || G.n1 <= 2 ? 0 : (G.n1 - 2) * G.n2 * (G.n3 > 1 ? 2 : 1);
+    return face + inner + between;
+}
+
+__device__ __forceinline__ int boundary_voxel(const GeomDev &G, int q)
+{
+    const int face = G.n2 * G.n3;
+    if (q < face) return (G.n1 - 1) * face + q;
+    q -= face;
+    if (q < face) return q;  // i = 0 (n1 > 1)
+    q -= face;
+    const int ends = G.n3 > 1 ? 2 : 1;  // one shell's voxels in the end planes
+    const int i = 1 + q / (G.n2 * ends), r = q % (G.n2 * ends);
+    return vid(G, i, r / ends, (r % ends) ? G.n3 - 1 : 0);
+}
+
+// Marks the voxels of the characteristics of the boundary and core voxels: a
+// thread per voxel that may start one.  The walk is the FP32 one with exact
+// fallback: on 65 x 33 x 65 voxels and 1024 directions the kernel took 113 ms
+// with the FP64 walk and a thread for every voxel of the grid.
+__global__ void __launch_bounds__(128) k_mark_boundary(GeomDev G, GeomF F, const double *dirs, int w0, int nw,
+                                                       uint32_t *hit, int words, int *lost, uint32_t *cnt)
+{
+    const int nb = n_boundary(G);
+    const int64_t total = (int64_t)nw * nb;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
-        int wl = (int)(idx / G.nvox);
-        int v = (int)(idx - (int64_t)wl * G.nvox);
+        const int wl = (int)(idx / nb);
+        const int v = boundary_voxel(G, (int)(idx - (int64_t)wl * nb));
         int w = w0 + wl;
         int i, j, k;
         ijk_of(G, v, i, j, k);
@@ -495,124 +524,192 @@ __global__ void k_mark_boundary(GeomDev G, const double *dirs, int w0, int nw, u
         double x, y, z;
         centre_of(G, i, j, k, x, y, z);
         MarkVisit mv{hit + (int64_t)wl * words, 0};
-        int eb = walk(G, x, y, z, -dx, -dy, -dz, i, j, k, mv);
-        const int nb = mv.n;
-        int ef = walk(G, x, y, z, dx, dy, dz, i, j, k, mv);
-        const bool bad = eb == RTK_END_LOST || ef == RTK_END_LOST;
+        int e[2], n[2];
+        for (int h = 0; h < 2; ++h) {  // backward, forward
+            const double sg = h ? 1.0 : -1.0;
+            mv.n = 0;
+            e[h] = fast_walk(G, F, x, y, z, sg * dx, sg * dy, sg * dz, i, j, k, mv);
+            n[h] = mv.n;
+        }
+        const bool bad = e[0] == RTK_END_LOST || e[1] == RTK_END_LOST;
         if (bad) atomicAdd(lost, 1);
-        cnt[(int64_t)w * G.nvox + v] = pack_counts(nb, mv.n - nb, bad);
+        cnt[(int64_t)w * G.nvox + v] = pack_counts(n[0], n[1], bad);
     }
 }
 
 __device__ __forceinline__ uint32_t read_word(uint32_t *p) { return atomicOr(p, 0u); }
 
-// One warp per solid angle.  The warp takes the next (up to) 32 voxels that
-// are not yet hit, traces the 32 characteristics through their centres in
-// parallel, then accepts them in voxel order: candidate m is kept only if no
-// accepted characteristic of a lower voxel has hit it, exactly as a serial
-// pass in increasing voxel index would decide.
-// One warp per CTA: the CTAs, one per solid angle, spread over every SM (the
-// walks are FP64-bound, so SMs with more solid angles than others finish last).
-constexpr int CPL_WARPS = 1;
+// Coverage completion, one CTA per solid angle at a time.  A round takes the
+// next COVER_C voxels that are not yet hit, traces the characteristics through
+// their centres in parallel (backward halves in the first COVER_C threads,
+// forward halves in the others) and decides them in voxel order exactly as a
+// serial pass would: candidate m is launched unless a launched candidate of a
+// lower voxel hits it.  A traced voxel that is itself a later candidate sets a
+// bit in the tracing candidate's row, so the decision is COVER_C steps on a
+// 256-bit mask; the voxels of the launched ones are then marked together.
+// The walks take most of the time, so a round is as wide as keeps their waste
+// low: on two sph65 directions 1.5 to 2.5 candidates are traced per launched
+// one at 32 a round, 2.9 to 3.7 at 128, 4.3 to 4.8 at 512.  With FP64 walks
+// and one warp per solid angle this took 575 ms for 64 of them and 912 ms for
+// 1024 on 65 x 33 x 65 voxels.
+constexpr int COVER_C = 256;
+constexpr int COVER_T = 2 * COVER_C;
+constexpr int COVER_W = COVER_C / 32;
+constexpr int COVER_CTAS = 152;             // one resident CTA (16 warps of 128 registers) an SM
+constexpr size_t COVER_SMEM = 160 * 1024;  // hit words kept in shared memory at most
 
-__global__ void __launch_bounds__(32 * CPL_WARPS) k_complete(GeomDev G, const double *dirs, int w0, int nw, uint32_t *hit,
-                                                  uint32_t *comp, int words, int32_t *scratch, int cap, int *lost,
-                                                  uint32_t *cnt)
+struct CoverVisit {
+    int32_t *list;       // every COVER_T-th entry is this thread's
+    const uint32_t *H;   // hit words at the start of the round
+    const int *cand;
+    uint32_t *row;       // later candidates this one hits
+    int n, v0, vlast, ncand;
+    __device__ __forceinline__ void cell(int v)
+    {
+        list[(int64_t)n * COVER_T] = v;
+        ++n;
+        // (volatile: earlier rounds changed the words by atomics, past L1)
+        if (v > v0 && v <= vlast && !((*(volatile const uint32_t *)(H + (v >> 5)) >> (v & 31)) & 1u)) {
+            int lo = 0, hi = ncand;  // cand[lo] == v: every unhit voxel up to vlast is a candidate
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (cand[mid] <= v) lo = mid;
+                else hi = mid;
+            }
+            if (cand[lo] == v) atomicOr(row + (lo >> 5), 1u << (lo & 31));
+        }
+    }
+};
+
+__global__ void __launch_bounds__(COVER_T) k_cover(GeomDev G, GeomF F, const double *dirs, int w0, int nw,
+                                                   uint32_t *hit, uint32_t *comp, int words, int in_smem,
+                                                   int32_t *scratch, int half_cap, int *lost, uint32_t *cnt)
 {
-    __shared__ int cand_s[CPL_WARPS][32];
-    const int wib = threadIdx.x >> 5;
-    const int lane = threadIdx.x & 31;
-    const int wl = blockIdx.x * CPL_WARPS + wib;
-    if (wl >= nw) return;
-    const int w = w0 + wl;
-    const double dx = dirs[3 * w], dy = dirs[3 * w + 1], dz = dirs[3 * w + 2];
-    uint32_t *H = hit + (int64_t)wl * words;
-    uint32_t *C = comp + (int64_t)wl * words;
-    int32_t *mylist = scratch + ((int64_t)wl * 32 + lane) * cap;
-    int *cand = cand_s[wib];
-    int pos = 0;
-    while (pos < G.nvox) {
-        // collect up to 32 unhit voxels in increasing order
-        int ncand = 0;
-        int scan = pos;
-        while (ncand < 32 && scan < G.nvox) {
-            uint32_t w0w = 0, w1w = 0;
-            if (lane == 0) {
-                w0w = read_word(H + (scan >> 5));
-                if ((scan >> 5) + 1 < words) w1w = read_word(H + (scan >> 5) + 1);
+    extern __shared__ uint32_t hsm[];
+    __shared__ int cand[COVER_C];
+    __shared__ uint32_t conf[COVER_C][COVER_W];
+    __shared__ uint32_t take[COVER_W];
+    __shared__ int len[COVER_T];
+    __shared__ unsigned char isbad[COVER_T];
+    __shared__ int wsum[COVER_T / 32], s_next;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int m = tid & (COVER_C - 1), fwd = tid / COVER_C;
+    int32_t *const list = scratch + (int64_t)blockIdx.x * half_cap * COVER_T + tid;
+    for (int wl = blockIdx.x; wl < nw; wl += gridDim.x) {
+        const int w = w0 + wl;
+        const double sg = fwd ? 1.0 : -1.0;
+        const double dx = sg * dirs[3 * w], dy = sg * dirs[3 * w + 1], dz = sg * dirs[3 * w + 2];
+        uint32_t *const Hg = hit + (int64_t)wl * words;
+        uint32_t *const C = comp + (int64_t)wl * words;
+        uint32_t *const H = in_smem ? hsm : Hg;
+        if (in_smem)
+            for (int q = tid; q < words; q += COVER_T) hsm[q] = Hg[q];
+        __syncthreads();
+        int pos = 0;
+        while (pos < G.nvox) {
+            // the next COVER_C unhit voxels in increasing order
+            int ncand = 0, scan = pos;
+            while (ncand < COVER_C && scan < G.nvox) {
+                const int q = (scan >> 5) + tid;
+                uint32_t free = 0;
+                if (q < words) {
+                    free = ~*(volatile uint32_t *)(H + q);
+                    if (q == (scan >> 5)) free &= 0xffffffffu << (scan & 31);
+                    if (32 * q + 32 > G.nvox) free &= (1u << (G.nvox & 31)) - 1u;  // the last, partial word
+                }
+                const int mine = __popc(free);
+                int incl = mine;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += u;
+                }
+                if (lane == 31) wsum[wid] = incl;
+                if (tid == 0) s_next = min(G.nvox, 32 * ((scan >> 5) + COVER_T));
+                __syncthreads();
+                int before = incl - mine, total = 0;
+                for (int u = 0; u < COVER_T / 32; ++u) {
+                    if (u < wid) before += wsum[u];
+                    total += wsum[u];
+                }
+                int at = ncand + before;
+                while (free && at < COVER_C) {
+                    const int b = __ffs(free) - 1;
+                    free &= free - 1;
+                    cand[at] = 32 * q + b;
+                    if (at == COVER_C - 1) s_next = 32 * q + b + 1;
+                    ++at;
+                }
+                __syncthreads();
+                ncand = min(COVER_C, ncand + total);
+                scan = s_next;
+                __syncthreads();
             }
-            w0w = __shfl_sync(0xffffffffu, w0w, 0);
-            w1w = __shfl_sync(0xffffffffu, w1w, 0);
-            int v = scan + lane;
-            uint32_t word = ((v >> 5) == (scan >> 5)) ? w0w : w1w;
-            bool unhit = (v < G.nvox) && !((word >> (v & 31)) & 1u);
-            uint32_t m = __ballot_sync(0xffffffffu, unhit);
-            int need = 32 - ncand;
-            int cnt = __popc(m);
-            int last_taken_lane = 31;
-            if (cnt > need) {
-                // keep the first `need` set bits
-                uint32_t mm = m;
-                for (int q = 0; q < need; ++q) mm &= mm - 1;
-                m &= ~mm;
-                last_taken_lane = 31 - __clz(m);
+            pos = scan;
+            if (ncand == 0) break;
+            // trace them
+            for (int q = tid; q < COVER_C * COVER_W; q += COVER_T) (&conf[0][0])[q] = 0u;
+            __syncthreads();
+            int n = 0, end = RTK_END_EXIT;
+            if (m < ncand) {
+                const int v = cand[m];
+                int i, j, k;
+                ijk_of(G, v, i, j, k);
+                double x, y, z;
+                centre_of(G, i, j, k, x, y, z);
+                CoverVisit cv{list, H, cand, conf[m], 0, v, cand[ncand - 1], ncand};
+                end = fast_walk(G, F, x, y, z, dx, dy, dz, i, j, k, cv);
+                n = cv.n;
             }
-            if (unhit && ((m >> lane) & 1u)) {
-                int rank = __popc(m & ((1u << lane) - 1u));
-                cand[ncand + rank] = v;
+            len[tid] = n;
+            isbad[tid] = end == RTK_END_LOST;
+            __syncthreads();
+            // decide them in voxel order
+            if (tid == 0) {
+                uint32_t dead[COVER_W], t[COVER_W];
+#pragma unroll
+                for (int u = 0; u < COVER_W; ++u) dead[u] = t[u] = 0u;
+                int nlost = 0;
+#pragma unroll
+                for (int u = 0; u < COVER_W; ++u)
+                    for (int b = 0; b < 32; ++b) {
+                        const int c = 32 * u + b;
+                        if (c >= ncand) break;
+                        const bool bad = isbad[c] || isbad[COVER_C + c];
+                        uint32_t r[COVER_W];
+#pragma unroll
+                        for (int h = 0; h < COVER_W; ++h) r[h] = conf[c][h];
+                        if ((dead[u] >> b) & 1u) continue;
+                        if (bad) {  // not launched, and not tried again
+                            ++nlost;
+                            continue;
+                        }
+                        t[u] |= 1u << b;
+#pragma unroll
+                        for (int h = 0; h < COVER_W; ++h) dead[h] |= r[h];
+                    }
+#pragma unroll
+                for (int u = 0; u < COVER_W; ++u) take[u] = t[u];
+                if (nlost) atomicAdd(lost, nlost);
             }
-            ncand += __popc(m);
-            scan += (cnt > need) ? last_taken_lane + 1 : 32;
-            __syncwarp();
-        }
-        pos = scan;
-        // trace the candidates
-        int nl = 0, bad = 0;
-        uint32_t pc = 0;  // packed walk counts of this lane's candidate
-        if (lane < ncand) {
-            int v = cand[lane];
-            int i, j, k;
-            ijk_of(G, v, i, j, k);
-            double x, y, z;
-            centre_of(G, i, j, k, x, y, z);
-            ListVisit lv{mylist, cap, 0};
-            int eb = walk(G, x, y, z, -dx, -dy, -dz, i, j, k, lv);
-            const int nbk = lv.n;
-            int ef = walk(G, x, y, z, dx, dy, dz, i, j, k, lv);
-            nl = lv.n < cap ? lv.n : cap;
-            bad = (eb == RTK_END_LOST || ef == RTK_END_LOST || lv.n > cap) ? 1 : 0;
-            pc = pack_counts(nbk, lv.n - nbk, eb == RTK_END_LOST || ef == RTK_END_LOST);
-        }
-        __syncwarp();
-        // accept in voxel order
-        for (int m = 0; m < ncand; ++m) {
-            int v = cand[m];
-            int n_m = __shfl_sync(0xffffffffu, nl, m);
-            int bad_m = __shfl_sync(0xffffffffu, bad, m);
-            const uint32_t pc_m = __shfl_sync(0xffffffffu, pc, m);
-            uint32_t word = 0;
-            if (lane == 0) word = read_word(H + (v >> 5));
-            word = __shfl_sync(0xffffffffu, word, 0);
-            if (!((word >> (v & 31)) & 1u)) {
-                if (bad_m) {
-                    if (lane == 0) {
-                        atomicOr(H + (v >> 5), 1u << (v & 31));
-                        atomicAdd(lost, 1);
-                    }
-                } else {
-                    if (lane == 0) {
-                        atomicOr(C + (v >> 5), 1u << (v & 31));
-                        cnt[(int64_t)w * G.nvox + v] = pc_m;
-                    }
-                    const int32_t *lst = scratch + ((int64_t)wl * 32 + m) * cap;
-                    for (int e = lane; e < n_m; e += 32) {
-                        int u = lst[e];
-                        atomicOr(H + (u >> 5), 1u << (u & 31));
-                    }
+            __syncthreads();
+            // mark the voxels of the launched ones
+            if (m < ncand && ((take[m >> 5] >> (m & 31)) & 1u)) {
+                for (int q0 = 0; q0 < n; q0 += 8) {  // eight reads in flight
+                    int v[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) v[u] = list[(int64_t)min(q0 + u, n - 1) * COVER_T];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) atomicOr(H + (v[u] >> 5), 1u << (v[u] & 31));
+                }
+                if (!fwd) {
+                    const int v = cand[m];
+                    atomicOr(C + (v >> 5), 1u << (v & 31));
+                    cnt[(int64_t)w * G.nvox + v] = pack_counts(n, len[COVER_C + m], false);
                 }
             }
-            __syncwarp();
+            __syncthreads();
         }
+        __syncthreads();
     }
 }
 
@@ -912,19 +1009,32 @@ int blocks_for(int64_t n, int threads)
 
 int geom_scratch_cap(const GeomDev &G) { return 2 * (4 * (G.n1 + G.n2 + G.n3) + 16) + 8; }
 
-cudaError_t geom_mark_boundary(const GeomDev &G, const double *dirs, int w0, int nw, uint32_t *hit, int words,
-                               int *lost, uint32_t *cnt, cudaStream_t st)
+cudaError_t geom_mark_boundary(const GeomDev &G, const GeomF &F, const double *dirs, int w0, int nw, uint32_t *hit,
+                               int words, int *lost, uint32_t *cnt, cudaStream_t st)
 {
-    int64_t total = (int64_t)nw * G.nvox;
-    k_mark_boundary<<<blocks_for(total, 256), 256, 0, st>>>(G, dirs, w0, nw, hit, words, lost, cnt);
+    const int face = G.n2 * G.n3;
+    const int64_t nb = 2 * (int64_t)face + (G.coord == RT_SPHERICAL ? 0 : 2 * (int64_t)G.n1 * G.n2);
+    k_mark_boundary<<<blocks_for(nw * nb, 128), 128, 0, st>>>(G, F, dirs, w0, nw, hit, words, lost, cnt);
     return cudaGetLastError();
 }
 
-cudaError_t geom_complete(const GeomDev &G, const double *dirs, int w0, int nw, uint32_t *hit, uint32_t *comp,
-                          int words, int32_t *scratch, int cap, int *lost, uint32_t *cnt, cudaStream_t st)
+// CTAs of the completion and the list entries each needs.
+int geom_cover_blocks(int nw) { return nw < COVER_CTAS ? nw : COVER_CTAS; }
+int64_t geom_cover_scratch(const GeomDev &G) { return (int64_t)(4 * (G.n1 + G.n2 + G.n3) + 16) * COVER_T; }
+
+cudaError_t geom_complete(const GeomDev &G, const GeomF &F, const double *dirs, int w0, int nw, uint32_t *hit,
+                          uint32_t *comp, int words, int32_t *scratch, int blocks, int *lost, uint32_t *cnt,
+                          cudaStream_t st)
 {
-    k_complete<<<(nw + CPL_WARPS - 1) / CPL_WARPS, 32 * CPL_WARPS, 0, st>>>(G, dirs, w0, nw, hit, comp, words, scratch,
-                                                                           cap, lost, cnt);
+    // the hit words in shared memory where they fit
+    const size_t bytes = sizeof(uint32_t) * (size_t)words;
+    const int in_smem = bytes <= COVER_SMEM;
+    if (in_smem && bytes > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_cover, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)COVER_SMEM);
+        if (e != cudaSuccess) return e;
+    }
+    k_cover<<<blocks, COVER_T, in_smem ? bytes : 0, st>>>(G, F, dirs, w0, nw, hit, comp, words, in_smem, scratch,
+                                                          4 * (G.n1 + G.n2 + G.n3) + 16, lost, cnt);
     return cudaGetLastError();
 }
 

@@ -32,10 +32,11 @@ namespace rtk {
 struct GeomF {
     int coord, n1, n2, n3, nphi, inner_bc, nvox;
     const float *e1, *e3;     // radial (or R) edges; z edges (cylindrical)
-    const float *ct;          // cos(theta_j), j = 0..n2 (spherical)
+    const float *ct;          // cos(theta_j), j = 0..n2 (spherical), 0 for the plane z = 0
     const float *ctm, *stm;   // cos/sin of theta mid-points (spherical)
     const float *cp, *sp;     // cos/sin of phi_k
     const float *cpm, *spm;   // cos/sin of phi mid-points
+    int r0_zero;              // the innermost edge is 0 (cylindrical)
 };
 
 enum { PRED_EXIT = 0, PRED_CORE = 1, PRED_LOST = 2 };

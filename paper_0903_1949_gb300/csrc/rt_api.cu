@@ -272,7 +272,7 @@ int upload_tables(rt_grid *g)
 // float-guided completion (RT_TUNE_GEOM_PREDICT on a NULL grid).
 int g_geom_predict = 0;
 
-// Float copies of the geometry tables for the guided completion, on the device
+// Float copies of the geometry tables for the launch set, on the device
 // (freed by the caller through dfree).
 int upload_tables_f(rt_grid *g, GeomF &F, std::vector<void *> &owned)
 {
@@ -291,7 +291,10 @@ int upload_tables_f(rt_grid *g, GeomF &F, std::vector<void *> &owned)
         ct.resize(g->n2 + 1);
         ctm.resize(g->n2);
         stm.resize(g->n2);
-        for (int j = 0; j <= g->n2; ++j) ct[j] = (float)std::cos(g->h_e[1][j]);
+        for (int j = 0; j <= g->n2; ++j) {
+            const double c = std::cos(g->h_e[1][j]);
+            ct[j] = std::fabs(c) < 1e-12 ? 0.0f : (float)c;  // the plane z = 0
+        }
         for (int j = 0; j < g->n2; ++j) {
             const double tm = 0.5 * (g->h_e[1][j] + g->h_e[1][j + 1]);
             ctm[j] = (float)std::cos(tm);
@@ -323,6 +326,7 @@ int upload_tables_f(rt_grid *g, GeomF &F, std::vector<void *> &owned)
     F.nphi = g->nphi;
     F.inner_bc = g->inner_bc;
     F.nvox = g->nvox;
+    F.r0_zero = g->h_e[0][0] == 0.0;
     return RT_OK;
 }
 
@@ -339,19 +343,24 @@ int build_geometry(rt_grid *g)
     // launch set: boundary marks, then serial-order coverage completion, in angle chunks
     const int cap = geom_scratch_cap(g->G);
     const bool guided = g_geom_predict != 0;
+    // solid angles at a time: hit words, and the completion's lists (per CTA; per
+    // solid angle with guesses), within 2 GB
+    const int64_t per_cta = 4 * geom_cover_scratch(g->G);
     const int64_t per_angle =
-        (int64_t)words * 4 + (int64_t)32 * cap * 4 + (guided ? (int64_t)32 * cap * 4 + (int64_t)nvox * 4 : 0);
-    int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(n_ang, ((int64_t)1 << 31) / per_angle));
+        (int64_t)words * 4 + (guided ? (int64_t)64 * cap * 4 + (int64_t)nvox * 4 : 0);
+    const int64_t room = (int64_t)1 << 31;
+    const int ctas = (int)std::max<int64_t>(1, std::min<int64_t>(geom_cover_blocks(n_ang), room / 2 / per_cta));
+    int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(n_ang, (room - (guided ? 0 : ctas * per_cta)) / per_angle));
     uint32_t *hit = nullptr;
     int32_t *scratch = nullptr, *pscr = nullptr, *stamp = nullptr;
     RCK(dalloc(g, &hit, (size_t)chunk * words));
-    RCK(dalloc(g, &scratch, (size_t)chunk * 32 * cap));
+    RCK(dalloc(g, &scratch, guided ? (size_t)chunk * 32 * cap : (size_t)(ctas * geom_cover_scratch(g->G))));
     GeomF F{};
     std::vector<void *> ftab;
+    RCK(upload_tables_f(g, F, ftab));
     if (guided) {
         RCK(dalloc(g, &pscr, (size_t)chunk * 32 * cap));
         RCK(dalloc(g, &stamp, (size_t)chunk * nvox));
-        RCK(upload_tables_f(g, F, ftab));
     }
     // walk counts of every launched characteristic (n_ang x n_vox), recorded by the launch-set passes
     uint32_t *wcnt = nullptr;
@@ -359,14 +368,14 @@ int build_geometry(rt_grid *g)
     for (int w0 = 0; w0 < n_ang; w0 += chunk) {
         int nw = std::min(chunk, n_ang - w0);
         CK(cudaMemsetAsync(hit, 0, sizeof(uint32_t) * (size_t)nw * words, g->st));
-        CK(geom_mark_boundary(g->G, g->d_dirs, w0, nw, hit, words, g->d_lost, wcnt, g->st));
+        CK(geom_mark_boundary(g->G, F, g->d_dirs, w0, nw, hit, words, g->d_lost, wcnt, g->st));
         if (guided) {
             CK(cudaMemsetAsync(stamp, 0, sizeof(int32_t) * (size_t)nw * nvox, g->st));
             CK(geom_complete_pred(g->G, F, g->d_dirs, w0, nw, hit, comp + (size_t)w0 * words, words, scratch, pscr,
                                   stamp, cap, g->d_lost, wcnt, g->st));
         } else {
-            CK(geom_complete(g->G, g->d_dirs, w0, nw, hit, comp + (size_t)w0 * words, words, scratch, cap, g->d_lost,
-                             wcnt, g->st));
+            CK(geom_complete(g->G, F, g->d_dirs, w0, nw, hit, comp + (size_t)w0 * words, words, scratch,
+                             std::min(ctas, nw), g->d_lost, wcnt, g->st));
         }
     }
     dfree(g, hit);

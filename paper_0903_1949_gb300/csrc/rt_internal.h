@@ -41,12 +41,17 @@ struct GeomDev {
 };
 
 // ---- geometry (geom.cu, compiled without FMA contraction) ----
+struct GeomF;
 // Marks every voxel hit by the characteristics of the boundary and core voxels.
-cudaError_t geom_mark_boundary(const GeomDev &G, const double *dirs, int w0, int nw, uint32_t *hit, int words,
-                               int *lost, uint32_t *cnt, cudaStream_t st);
-// Coverage completion in increasing voxel order, one warp per solid angle.
-cudaError_t geom_complete(const GeomDev &G, const double *dirs, int w0, int nw, uint32_t *hit, uint32_t *comp,
-                          int words, int32_t *scratch, int cap, int *lost, uint32_t *cnt, cudaStream_t st);
+cudaError_t geom_mark_boundary(const GeomDev &G, const GeomF &F, const double *dirs, int w0, int nw, uint32_t *hit,
+                               int words, int *lost, uint32_t *cnt, cudaStream_t st);
+// Coverage completion in increasing voxel order: `blocks` CTAs (at most
+// geom_cover_blocks(nw)) with geom_cover_scratch int32 entries each.
+cudaError_t geom_complete(const GeomDev &G, const GeomF &F, const double *dirs, int w0, int nw, uint32_t *hit,
+                          uint32_t *comp, int words, int32_t *scratch, int blocks, int *lost, uint32_t *cnt,
+                          cudaStream_t st);
+int geom_cover_blocks(int nw);
+int64_t geom_cover_scratch(const GeomDev &G);
 // cnt[w n_vox + v]: cells of the backward (high 16 bits) and forward walk of the
 // characteristic launched at voxel v for solid angle w, recorded by the two
 // launch-set passes; the segment counts then need no walk of their own.
@@ -60,7 +65,6 @@ cudaError_t geom_write_segs(const GeomDev &G, const double *dirs, int64_t n_rays
                             const int32_t *ray_angle, const int64_t *ray_off, const int32_t *nback, uint32_t *vox,
                             double *len64, float *len32, int *lost, cudaStream_t st);
 int geom_scratch_cap(const GeomDev &G);
-struct GeomF;
 // Coverage completion guided by a float guess of each candidate's line (same
 // launch set as geom_complete); pscr: 32 lists of cap per solid angle, stamp:
 // n_vox per solid angle, zeroed before the call.
