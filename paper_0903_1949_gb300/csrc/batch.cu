@@ -6,9 +6,9 @@
 // parabola choices (a bit per crossing segment, from its chi in FP64); the
 // crossing lists and ownership lists are those of the member's grid.  One
 // ALI iteration of all members is: pack (chi, S) in FP32, then for each wave
-// k (angle block k of every member that has one) a persistent FP32 J-only
-// march over the bundles of all the wave's items and a persistent J gather
-// over their lists, then the FP64 ALI update of every member.  Each member
+// k (angle block k of members that have one, up to WAVE_SEG segments) a persistent
+// FP32 J-only march over the bundles of all the wave's items and a persistent J
+// gather over their lists beside the next wave's march, then the FP64 ALI update of every member.  Each member
 // appears at most once per wave, so its J accumulates over its angle blocks
 // in a fixed order.  The whole iteration is captured once as a CUDA graph and
 // replayed; rt_batch_autotune picks the bundle size and the persistent grid.
@@ -60,22 +60,47 @@ __global__ void k_bpack(int64_t n, const double *chi, const double *S, const dou
     }
 }
 
+// maxrel[m] <- max over the block of rel, a non-negative double or NaN (their bit
+// patterns order like the values), for blocks whose threads may belong to several
+// members: one atomic per warp and member.  (One per voxel took 588 us for twelve
+// members of 1.4e5 and 1.9e4 voxels, all waiting on the same few words.)
+__device__ __forceinline__ void member_max(bool valid, int m, double rel, unsigned long long *maxrel)
+{
+    const unsigned FULL = 0xffffffffu;
+    unsigned long long x = valid ? (unsigned long long)__double_as_longlong(rel) : 0ull;
+    const int m0 = __shfl_sync(FULL, valid ? m : -1, 0);
+    if (__all_sync(FULL, !valid || m == m0)) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long y = __shfl_xor_sync(FULL, x, o);
+            x = y > x ? y : x;
+        }
+        if ((threadIdx.x & 31) == 0 && m0 >= 0) atomicMax(maxrel + m0, x);
+    } else if (valid) {  // the warp straddles two members
+        atomicMax(maxrel + m, x);
+    }
+}
+
 // ALI update of every member's voxels; per-member max |dS| / |S_new|.
 __global__ void k_bali(int64_t n, const int64_t *voff, int nm, double *S, const double *J, const double *L,
                        const double *eps, const double *B, unsigned long long *maxrel)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nm;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        const bool valid = i < n;
+        int lo = 0, hi = valid ? nm : 0;
         while (hi - lo > 1) {
             int mid = (lo + hi) >> 1;
             if (voff[mid] <= i) lo = mid;
             else hi = mid;
         }
-        const double e = eps[i], s = S[i];
-        const double sn = s + ((1.0 - e) * J[i] + e * B[i] - s) / (1.0 - (1.0 - e) * L[i]);
-        const double rel = fabs(sn - s) / fabs(sn);
-        S[i] = sn;
-        atomicMax(maxrel + lo, (unsigned long long)__double_as_longlong(rel));
+        double rel = 0.0;
+        if (valid) {
+            const double e = eps[i], s = S[i];
+            const double sn = s + ((1.0 - e) * J[i] + e * B[i] - s) / (1.0 - (1.0 - e) * L[i]);
+            rel = fabs(sn - s) / fabs(sn);
+            S[i] = sn;
+        }
+        member_max(valid, lo, rel, maxrel);
     }
 }
 
@@ -85,22 +110,27 @@ __global__ void k_bali(int64_t n, const int64_t *voff, int nm, double *S, const 
 __global__ void k_bresid(int64_t n, const int64_t *voff, int nm, const int *active, const double *S, const double *J,
                          const double *L, const double *eps, const double *B, double *R, unsigned long long *maxrel)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nm;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        const bool valid = i < n;
+        int lo = 0, hi = valid ? nm : 0;
         while (hi - lo > 1) {
             int mid = (lo + hi) >> 1;
             if (voff[mid] <= i) lo = mid;
             else hi = mid;
         }
-        if (!active[lo]) {
+        const bool on = valid && active[lo];
+        double rel = 0.0;
+        if (on) {
+            const double e = eps[i], s = S[i];
+            const double r = (1.0 - e) * J[i] + e * B[i] - s;
+            R[i] = r;
+            const double d = r / (1.0 - (1.0 - e) * L[i]);
+            rel = fabs(d) / fabs(s + d);
+        } else if (valid) {
             R[i] = 0.0;
-            continue;
         }
-        const double e = eps[i], s = S[i];
-        const double r = (1.0 - e) * J[i] + e * B[i] - s;
-        R[i] = r;
-        const double d = r / (1.0 - (1.0 - e) * L[i]);
-        atomicMax(maxrel + lo, (unsigned long long)__double_as_longlong(fabs(d) / fabs(s + d)));
+        member_max(on, lo, rel, maxrel);
     }
 }
 
@@ -110,17 +140,23 @@ __global__ void k_bresid(int64_t n, const int64_t *voff, int nm, const int *acti
 __global__ void k_bcorr(int64_t n, const int64_t *voff, int nm, double *D, const double *J, const double *R,
                         const double *L, const double *eps, const double *S, unsigned long long *maxrel)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nm;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        const bool valid = i < n;
+        int lo = 0, hi = valid ? nm : 0;
         while (hi - lo > 1) {
             int mid = (lo + hi) >> 1;
             if (voff[mid] <= i) lo = mid;
             else hi = mid;
         }
-        const double e = eps[i], d = D[i];
-        const double dn = d + ((1.0 - e) * J[i] + R[i] - d) / (1.0 - (1.0 - e) * L[i]);
-        D[i] = dn;
-        atomicMax(maxrel + lo, (unsigned long long)__double_as_longlong(fabs(dn - d) / fabs(S[i] + dn)));
+        double rel = 0.0;
+        if (valid) {
+            const double e = eps[i], d = D[i];
+            const double dn = d + ((1.0 - e) * J[i] + R[i] - d) / (1.0 - (1.0 - e) * L[i]);
+            D[i] = dn;
+            rel = fabs(dn - d) / fabs(S[i] + dn);
+        }
+        member_max(valid, lo, rel, maxrel);
     }
 }
 
@@ -224,6 +260,11 @@ __global__ void k_line_rhs(int nvox, int nf, const double *J, const double *phi,
     y[v] = (1.0 - eps_l[v]) * jb + eps_l[v] * B[v] - S_l[v];
 }
 
+// Segments of a wave at most (unless one item alone has more): 48 MB of FP32
+// values, so that with the next wave's in its other buffer they stay in L2 from
+// the march to the gather, and two bundles for every resident warp of the march.
+constexpr int64_t WAVE_SEG = 12000000;
+
 struct Wave {
     int n = 0;            // items
     int64_t mi0 = 0;      // first item in the concatenated item arrays
@@ -258,7 +299,9 @@ struct rt_batch {
     MarchItem *d_mi = nullptr;
     GatherItem *d_gi = nullptr;
     int64_t *d_bpfx = nullptr, *d_wpfx = nullptr;
-    float *wbuf = nullptr;
+    float *wbuf = nullptr;  // per-segment values of the waves, two buffers in turn
+    cudaStream_t st2 = nullptr;           // the gathers' stream, and the events between it and st
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_m[2] = {}, ev_g[2] = {};
     double *wpart = nullptr;
     int *wcnt = nullptr;
     unsigned long long *counters = nullptr;
@@ -312,6 +355,10 @@ void bfree_all(rt_batch *b)
     b->graph_corr = nullptr;
     for (void *p : b->allocs) cudaFree(p);
     b->allocs.clear();
+    for (cudaEvent_t *e : {&b->ev_fork, &b->ev_join, &b->ev_m[0], &b->ev_m[1], &b->ev_g[0], &b->ev_g[1]})
+        if (*e) cudaEventDestroy(*e), *e = nullptr;
+    if (b->st2) cudaStreamDestroy(b->st2);
+    b->st2 = nullptr;
     if (b->own_stream && b->st) cudaStreamDestroy(b->st);
     b->st = nullptr;
 }
@@ -346,6 +393,31 @@ int build_prefixes(rt_batch *b)
     return RT_OK;
 }
 
+// March and gather of every wave (captured): the gathers run in order on the
+// second stream, each beside the next wave's march; a march waits for the gather
+// that read its buffer two waves before.
+int enqueue_waves(rt_batch *b, int homog)
+{
+    BCK(cudaMemsetAsync(b->counters, 0, 2 * sizeof(unsigned long long) * b->waves.size(), b->st));
+    BCK(cudaEventRecord(b->ev_fork, b->st));
+    BCK(cudaStreamWaitEvent(b->st2, b->ev_fork, 0));
+    for (size_t i = 0; i < b->waves.size(); ++i) {
+        const Wave &w = b->waves[i];
+        const int q = (int)(i & 1);
+        if (i >= 2) BCK(cudaStreamWaitEvent(b->st, b->ev_g[q], 0));
+        BCK(march_batch(b->d_mi + w.mi0, b->d_bpfx + w.pf0, w.n, w.bundles, b->chunk, homog, b->counters + 2 * i,
+                        b->grid_march, b->st));
+        BCK(cudaEventRecord(b->ev_m[q], b->st));
+        BCK(cudaStreamWaitEvent(b->st2, b->ev_m[q], 0));
+        BCK(gather_J_batch(b->d_gi + w.mi0, b->d_wpfx + w.pf0, w.n, w.work, b->counters + 2 * i + 1, b->grid_gather,
+                           b->st2));
+        BCK(cudaEventRecord(b->ev_g[q], b->st2));
+    }
+    BCK(cudaEventRecord(b->ev_join, b->st2));
+    BCK(cudaStreamWaitEvent(b->st, b->ev_join, 0));
+    return RT_OK;
+}
+
 // The kernels of one ALI iteration of all members (captured into the graph).
 int enqueue_iteration(rt_batch *b)
 {
@@ -356,12 +428,7 @@ int enqueue_iteration(rt_batch *b)
     }
     k_bpack<<<152 * 8, 256, 0, b->st>>>(b->ntot, b->chi, b->S, b->B, b->cs, b->B32);
     BCK(cudaGetLastError());
-    for (const Wave &w : b->waves) {
-        BCK(cudaMemsetAsync(b->counters, 0, 2 * sizeof(unsigned long long), b->st));
-        BCK(march_batch(b->d_mi + w.mi0, b->d_bpfx + w.pf0, w.n, w.bundles, b->chunk, 0, b->counters, b->grid_march,
-                        b->st));
-        BCK(gather_J_batch(b->d_gi + w.mi0, b->d_wpfx + w.pf0, w.n, w.work, b->counters + 1, b->grid_gather, b->st));
-    }
+    BRCK(enqueue_waves(b, 0));
     BCK(cudaMemsetAsync(b->maxrel, 0, sizeof(unsigned long long) * b->nm, b->st));
     if (b->line && b->lstar == RT_LSTAR_NN) {  // the OS solve follows the graph (line_nn_os)
         k_line_rhs<<<(b->lnvox + 255) / 256, 256, 0, b->st>>>(b->lnvox, b->nf, b->J, b->phi, b->wq, b->eps_l, b->Bl,
@@ -381,12 +448,7 @@ int enqueue_correction(rt_batch *b)
 {
     k_bpack<<<152 * 8, 256, 0, b->st>>>(b->ntot, b->chi, b->D, b->B, b->cs, b->B32);
     BCK(cudaGetLastError());
-    for (const Wave &w : b->waves) {
-        BCK(cudaMemsetAsync(b->counters, 0, 2 * sizeof(unsigned long long), b->st));
-        BCK(march_batch(b->d_mi + w.mi0, b->d_bpfx + w.pf0, w.n, w.bundles, b->chunk, 1, b->counters, b->grid_march,
-                        b->st));
-        BCK(gather_J_batch(b->d_gi + w.mi0, b->d_wpfx + w.pf0, w.n, w.work, b->counters + 1, b->grid_gather, b->st));
-    }
+    BRCK(enqueue_waves(b, 1));
     BCK(cudaMemsetAsync(b->maxrel, 0, sizeof(unsigned long long) * b->nm, b->st));
     k_bcorr<<<152 * 8, 256, 0, b->st>>>(b->ntot, b->d_voff, b->nm, b->D, b->J, b->R, b->L, b->eps, b->S, b->maxrel);
     BCK(cudaGetLastError());
@@ -591,7 +653,6 @@ int rt_batch_create(rt_batch **out, rt_grid *const *grids, int n_grids, int n_me
     TRY(balloc(b, &b->B32, b->ntot));
     TRY(balloc(b, &b->d_voff, n_members + 1));
     TRY(balloc(b, &b->maxrel, n_members));
-    TRY(balloc(b, &b->counters, 2));
     TRY(balloc(b, &b->R, b->ntot));
     TRY(balloc(b, &b->D, b->ntot));
     TRY(balloc(b, &b->cs64, max_vox));
@@ -602,7 +663,7 @@ int rt_batch_create(rt_batch **out, rt_grid *const *grids, int n_grids, int n_me
     b->pbits.assign(n_members, nullptr);
     for (int m = 0; m < n_members; ++m)
         TRY(balloc(b, &b->pbits[m], (grids[member_grid[m]]->n_seg + 31) / 32));
-    // waves: wave k holds angle block k of every member whose grid has one
+    // waves: angle block k of every member whose grid has one, cut where WAVE_SEG is reached
     int maxblk = 0;
     for (rt_grid *g : b->grids) maxblk = std::max(maxblk, g->nblk);
     int64_t max_buf = 0, max_part = 0, max_cnt = 0;
@@ -610,11 +671,21 @@ int rt_batch_create(rt_batch **out, rt_grid *const *grids, int n_grids, int n_me
         Wave w;
         w.mi0 = (int64_t)b->h_mi.size();
         int64_t buf = 0, part = 0, cnt = 0;
+        auto push = [&]() {  // the wave is complete
+            b->waves.push_back(w);
+            max_buf = std::max(max_buf, buf);
+            max_part = std::max(max_part, part);
+            max_cnt = std::max(max_cnt, cnt);
+            w = Wave();
+            w.mi0 = (int64_t)b->h_mi.size();
+            buf = part = cnt = 0;
+        };
         for (int m = 0; m < n_members; ++m) {
             rt_grid *g = b->grids[b->mgrid[m]];
             if (k >= g->nblk) continue;
             const int w0 = g->blk_w0[k], nw = g->blk_nw[k];
             const int64_t lo = g->h_ang_seg_off[w0], ns = g->h_ang_seg_off[w0 + nw] - lo;
+            if (w.n > 0 && buf + ns > WAVE_SEG) push();
             MarchItem mi;
             mi.vox = g->d_vox;
             mi.len = g->d_len32;
@@ -654,22 +725,28 @@ int rt_batch_create(rt_batch **out, rt_grid *const *grids, int n_grids, int n_me
             cnt += std::max(1, gi.t.nlong);
             w.n++;
         }
-        b->waves.push_back(w);
-        max_buf = std::max(max_buf, buf);
-        max_part = std::max(max_part, part);
-        max_cnt = std::max(max_cnt, cnt);
+        if (w.n > 0) push();
     }
-    TRY(balloc(b, &b->wbuf, max_buf));
+    max_buf = (max_buf + 3) & ~(int64_t)3;
+    TRY(balloc(b, &b->wbuf, 2 * max_buf));
+    TRY(balloc(b, &b->counters, 2 * b->waves.size()));
+    if (cudaStreamCreateWithFlags(&b->st2, cudaStreamNonBlocking) != cudaSuccess)
+        return fail_and_free(bfail(RT_ECUDA, "stream creation failed"));
+    for (cudaEvent_t *e : {&b->ev_fork, &b->ev_join, &b->ev_m[0], &b->ev_m[1], &b->ev_g[0], &b->ev_g[1]})
+        if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess)
+            return fail_and_free(bfail(RT_ECUDA, "event creation failed"));
     TRY(balloc(b, &b->wpart, max_part));
     TRY(balloc(b, &b->wcnt, max_cnt));
     if (cudaMemsetAsync(b->wcnt, 0, sizeof(int) * max_cnt, b->st) != cudaSuccess)
         return fail_and_free(bfail(RT_ECUDA, "memset failed"));
-    for (size_t i = 0; i < b->h_mi.size(); ++i) {  // turn offsets into pointers
-        b->h_mi[i].out = b->wbuf + (intptr_t)b->h_mi[i].out;
-        b->h_gi[i].buf = b->wbuf + (intptr_t)b->h_gi[i].buf;
-        b->h_gi[i].part = b->wpart + (intptr_t)b->h_gi[i].part;
-        b->h_gi[i].t.cnt = b->wcnt + (intptr_t)b->h_gi[i].t.cnt;
-    }
+    for (size_t q = 0; q < b->waves.size(); ++q)  // turn offsets into pointers
+        for (int64_t i = b->waves[q].mi0; i < b->waves[q].mi0 + b->waves[q].n; ++i) {
+            float *const base = b->wbuf + (q & 1) * max_buf;
+            b->h_mi[i].out = base + (intptr_t)b->h_mi[i].out;
+            b->h_gi[i].buf = base + (intptr_t)b->h_gi[i].buf;
+            b->h_gi[i].part = b->wpart + (intptr_t)b->h_gi[i].part;
+            b->h_gi[i].t.cnt = b->wcnt + (intptr_t)b->h_gi[i].t.cnt;
+        }
     TRY(balloc(b, &b->d_mi, b->h_mi.size()));
     TRY(balloc(b, &b->d_gi, b->h_gi.size()));
     if (cudaMemcpyAsync(b->d_mi, b->h_mi.data(), sizeof(MarchItem) * b->h_mi.size(), cudaMemcpyHostToDevice, b->st) !=

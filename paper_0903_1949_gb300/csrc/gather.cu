@@ -110,8 +110,8 @@ __global__ void __launch_bounds__(256) k_rs_scatter(const uint32_t *__restrict__
 // Inverse path lengths of one block, a thread per (solid angle, voxel): its
 // entries are a run of the voxel's list (six on average), found by bisection.
 // The few runs of more than INVL_SHORT entries (an outer voxel on the lines
-// through the core has thousands) are each summed by a warp, the lanes taking
-// entries in turn and adding in a fixed tree.  A thread per voxel over its whole
+// through the core has thousands) are each read by a warp, 32 entries at a time,
+// and added in the same order, so every sum is the one of a serial pass.  A thread per voxel over its whole
 // list took 1.1 ms a block on 65 x 33 x 65 voxels, waiting for the longest.
 constexpr int INVL_SHORT = 64;
 
@@ -159,8 +159,13 @@ __global__ void __launch_bounds__(256) k_invL(int nvox, const int32_t *off, cons
     const int lane = threadIdx.x & 31;
     for (int i = threadIdx.x >> 5; i < nlong; i += blockDim.x >> 5) {
         double acc = 0.0;
-        for (int e = lbeg[i] + lane; e < lend[i]; e += 32) acc += len[perm[e]];
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        double l = lbeg[i] + lane < lend[i] ? len[perm[lbeg[i] + lane]] : 0.0;
+        for (int e = lbeg[i]; e < lend[i]; e += 32) {
+            const double next = e + 32 + lane < lend[i] ? len[perm[e + 32 + lane]] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 32; ++u) acc += __shfl_sync(0xffffffffu, l, u);  // past the end: + 0
+            l = next;
+        }
         if (lane == 0) out[longv[i]] = (acc > 0.0) ? 1.0 / acc : 0.0;
     }
 }
@@ -388,30 +393,31 @@ __global__ void k_make_wL32(int64_t n, int nvox, const double *invL, const doubl
         wL[i] = (float)(wt[i / nvox] * invL[i]);
 }
 
-// One thread per voxel with more than one unit: add its unit sums in order.
-__global__ void k_gather_rows(int nmulti, const int32_t *__restrict__ multi, const int64_t *__restrict__ ufirst,
-                              const double *__restrict__ part, double *J, double *Lst, double *Fc, int first)
+// Voxels with more than one unit: their unit sums added in order, eight lanes to
+// a voxel of which five take a component each, eight sums in flight (a thread per
+// voxel and component after component took 50 us a block of 65 x 33 x 65 voxels,
+// waiting for the voxels with hundreds of units).
+__global__ void __launch_bounds__(256) k_gather_rows(int nmulti, const int32_t *__restrict__ multi,
+                                                     const int64_t *__restrict__ ufirst,
+                                                     const double *__restrict__ part, double *J, double *Lst, double *Fc,
+                                                     int first)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nmulti) return;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = t >> 3, c = t & 7;
+    if (i >= nmulti || c > 4) return;
     const int v = multi[i];
-    double j = 0.0, l = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
-    for (int64_t u = ufirst[v]; u < ufirst[v + 1]; ++u) {
-        const double *o = part + 5 * u;
-        j += o[0]; l += o[1]; fx += o[2]; fy += o[3]; fz += o[4];
+    const int64_t u0 = ufirst[v], u1 = ufirst[v + 1];
+    double a = 0.0;
+    for (int64_t u = u0; u < u1; u += 8) {
+        double x[8];
+#pragma unroll
+        for (int h = 0; h < 8; ++h) x[h] = u + h < u1 ? part[5 * (u + h) + c] : 0.0;
+#pragma unroll
+        for (int h = 0; h < 8; ++h)
+            if (u + h < u1) a += x[h];
     }
-    if (!first) {
-        j += J[v];
-        l += Lst[v];
-        fx += Fc[3 * (int64_t)v];
-        fy += Fc[3 * (int64_t)v + 1];
-        fz += Fc[3 * (int64_t)v + 2];
-    }
-    J[v] = j;
-    Lst[v] = l;
-    Fc[3 * (int64_t)v] = fx;
-    Fc[3 * (int64_t)v + 1] = fy;
-    Fc[3 * (int64_t)v + 2] = fz;
+    double *o = c == 0 ? J + v : c == 1 ? Lst + v : Fc + 3 * (int64_t)v + (c - 2);
+    *o = first ? a : a + *o;
 }
 
 // Voxels whose ownership list needs more than one unit (compacted in voxel order).
@@ -892,7 +898,7 @@ cudaError_t gather_block(int nvox, const int32_t *csr_off, const int32_t *perm_b
     else
         k_gather_units64<<<blocks, 256, 0, st>>>(nvox, nunits, urow, order, ulen, gbase, sell, (const double2 *)buf,
                                                  ang_seg_off, w0, nw, seg_lo, invL, wt, dirs, part, J, Lst, Fc, first);
-    if (nmulti > 0) k_gather_rows<<<(nmulti + 255) / 256, 256, 0, st>>>(nmulti, multi, ufirst, part, J, Lst, Fc, first);
+    if (nmulti > 0) k_gather_rows<<<(nmulti * 8 + 255) / 256, 256, 0, st>>>(nmulti, multi, ufirst, part, J, Lst, Fc, first);
     return cudaGetLastError();
 }
 
