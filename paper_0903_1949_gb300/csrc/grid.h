@@ -148,6 +148,17 @@ struct rt_grid {
 int rt_grid_member_fs(rt_grid *g, const float2 *cs, const float *B32, const uint32_t *pbits, double *J, double *L,
                       double *Fc, cudaStream_t st);
 
+// Work arrays of the nearest-neighbour operator's build on a grid: allocated at
+// the first build that uses them, freed with the object (after its stream).
+struct NnScratch {
+    int8_t *slot = nullptr;
+    double *val = nullptr, *part = nullptr;
+    rtk::Wd4 *cw = nullptr;
+    cudaStream_t st = nullptr;
+    bool get(const rt_grid *g);  // false: no memory
+    ~NnScratch();
+};
+
 // The grid's exact nearest-neighbour Lambda* (d_L27) for its current chi, built
 // on first use after rt_set_opacity; returns an RT_ status.
 int rt_grid_build_nn(rt_grid *g);
@@ -165,5 +176,6 @@ int rt_grid_member_fs64J(rt_grid *g, const double2 *cs64, const double *B64, con
 // The exact nearest-neighbour Lambda* (27 entries per voxel, slot q = 9 (di+1) +
 // 3 (dj+1) + (dk+1), phi periodic) of another opacity field chi, with its
 // parabola choices pbits (bit per segment, as para_bits), on this grid's
-// geometry, into L27; runs on st and returns after it has drained.
-int rt_grid_nn_lstar(rt_grid *g, const double *chi, const uint32_t *pbits, double *L27, cudaStream_t st);
+// geometry, into L27; queued on st, with `work` kept until st has drained.
+int rt_grid_nn_lstar(rt_grid *g, const double *chi, const uint32_t *pbits, double *L27, NnScratch &work,
+                     cudaStream_t st);

@@ -1393,34 +1393,14 @@ int ng_maybe(rt_grid *g, double *out, const double *wref)
 // order; the diagonal is copied to d_L.
 // The exact nearest-neighbour Lambda* of opacity chi (device, n_vox) with the
 // parabola choices pbits (NULL: those marked in the crossing words for the
-// grid's own chi) into L27 (device, 27 n_vox), on stream st; returns after the
-// stream has drained.
-int nn_lstar_into(rt_grid *g, const double *chi, const uint32_t *pbits, double *L27, cudaStream_t st)
+// grid's own chi) into L27 (device, 27 n_vox), queued on stream st.
+int nn_lstar_into(rt_grid *g, const double *chi, const uint32_t *pbits, double *L27, NnScratch &work, cudaStream_t st)
 {
     const int n = g->nvox;
-    int8_t *slot = nullptr;
-    double *val = nullptr, *part = nullptr;
-    int64_t max_units = 1;
-    for (int b = 0; b < g->nblk; ++b) max_units = std::max(max_units, g->h_nunits[b]);
-    if (cudaMalloc(&slot, (size_t)RTK_NNW * std::max<int64_t>(1, g->max_blk_seg)) != cudaSuccess ||
-        cudaMalloc(&val, sizeof(double) * RTK_NNW * std::max<int64_t>(1, g->max_blk_seg)) != cudaSuccess ||
-        cudaMalloc(&part, sizeof(double) * 27 * (size_t)max_units) != cudaSuccess) {
-        cudaGetLastError();
-        if (slot) cudaFree(slot);
-        if (val) cudaFree(val);
-        return fail(RT_ENOMEM, "NN Lambda* work arrays could not be allocated");
-    }
-    struct Free {
-        void *a, *b, *c;
-        cudaStream_t st;
-        ~Free()
-        {
-            cudaStreamSynchronize(st);  // no launch may still use them
-            cudaFree(a);
-            cudaFree(b);
-            cudaFree(c);
-        }
-    } fr{slot, val, part, st};
+    work.st = st;
+    if (!work.get(g)) return fail(RT_ENOMEM, "NN Lambda* work arrays could not be allocated");
+    int8_t *slot = work.slot;
+    double *val = work.val, *part = work.part;
     for (int b = 0; b < g->nblk; ++b) {
         const int w0 = g->blk_w0[b], nw = g->blk_nw[b];
         NnWalk a{};
@@ -1441,7 +1421,8 @@ int nn_lstar_into(rt_grid *g, const double *chi, const uint32_t *pbits, double *
         a.sph = g->coord == RT_SPHERICAL;
         a.slot = slot;
         a.val = val;
-        CK(nn_walk(a, st));
+        a.cw = work.cw;
+        CK(nn_walk(a, g->h_ang_seg_off[w0 + nw] - a.seg_lo, st));
         NnUnits un{};
         un.urow = g->d_urow + g->h_ubase[b];
         un.ubeg = g->d_ubeg + g->h_ubase[b];
@@ -1450,16 +1431,16 @@ int nn_lstar_into(rt_grid *g, const double *chi, const uint32_t *pbits, double *
         un.multi = g->d_multi + g->h_mbase[b];
         un.nmulti = g->h_mbase[b + 1] - g->h_mbase[b];
         CK(nn_gather(n, g->d_csr_off + (size_t)b * (n + 1), g->d_perm + a.seg_lo, slot, val, un, part, L27, b == 0, st));
-        g->launches += 3;
+        g->launches += 4;
     }
-    CK(cudaStreamSynchronize(st));
     return RT_OK;
 }
 
 int build_nn(rt_grid *g)
 {
     if (g->nn_ok) return RT_OK;
-    RCK(nn_lstar_into(g, g->d_chi, nullptr, g->d_L27, g->st));
+    NnScratch work;
+    RCK(nn_lstar_into(g, g->d_chi, nullptr, g->d_L27, work, g->st));
     CK(nn_diag(g->nvox, g->d_L27, g->d_L, g->st));
     g->launches++;
     RCK(sync(g));
@@ -1556,11 +1537,36 @@ int check_lost(rt_grid *g)
 
 }  // namespace
 
-int rt_grid_nn_lstar(rt_grid *g, const double *chi, const uint32_t *pbits, double *L27, cudaStream_t st)
+bool NnScratch::get(const rt_grid *g)
+{
+    if (cw) return true;
+    int64_t units = 1;
+    for (int64_t u : g->h_nunits) units = std::max(units, u);
+    const size_t seg = (size_t)std::max<int64_t>(1, g->max_blk_seg);
+    if (cudaMalloc(&slot, RTK_NNW * seg) != cudaSuccess || cudaMalloc(&val, sizeof(double) * RTK_NNW * seg) != cudaSuccess ||
+        cudaMalloc(&part, sizeof(double) * 27 * (size_t)units) != cudaSuccess ||
+        cudaMalloc(&cw, sizeof(Wd4) * seg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
+NnScratch::~NnScratch()
+{
+    if (slot || val || part || cw) cudaStreamSynchronize(st);  // no launch may still use them
+    cudaFree(slot);
+    cudaFree(val);
+    cudaFree(part);
+    cudaFree(cw);
+}
+
+int rt_grid_nn_lstar(rt_grid *g, const double *chi, const uint32_t *pbits, double *L27, NnScratch &work,
+                     cudaStream_t st)
 {
     if (g->nphi < 3) return fail(RT_EINVAL, "the nearest-neighbour Lambda* needs n_phi >= 3");
     if (!pbits) return fail(RT_EINVAL, "parabola choices of chi required");
-    return nn_lstar_into(g, chi, pbits, L27, st);
+    return nn_lstar_into(g, chi, pbits, L27, work, st);
 }
 
 int rt_grid_member_fs(rt_grid *g, const float2 *cs, const float *B32, const uint32_t *pbits, double *J, double *L,

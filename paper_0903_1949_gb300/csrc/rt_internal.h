@@ -338,8 +338,10 @@ struct NnWalk {
     int nvox, n2, n3, sph;
     int8_t *slot;                // RTK_NNW per segment: neighbour slot of v_s or -1
     double *val;                 // RTK_NNW per segment: w l / L times dI_s/dS_u
+    Wd4 *cw;                     // work: the weights of the block's segments
 };
-cudaError_t nn_walk(const NnWalk &a, cudaStream_t st);
+// The block's nseg segments: their weights, then the walk.
+cudaError_t nn_walk(const NnWalk &a, int64_t nseg, cudaStream_t st);
 // An angle block's gather work units (its ownership lists cut into pieces of
 // at most a fixed number of entries): unit voxel and first entry, per-voxel
 // unit offsets, and the voxels with more than one unit.
