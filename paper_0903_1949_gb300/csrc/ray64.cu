@@ -29,26 +29,21 @@ namespace {
 constexpr double FOUR_PI_R = 12.566370614359172953850573533118;
 constexpr int STEPS_PER_WARP = 8;  // steps of a group that one warp of the set-up kernels takes at a time
 
-// Characteristics per length, longest first (key = cap - length), per angle block.
-__global__ void k_ray_hist(int64_t n_rays, const int64_t *__restrict__ ray_off, const int32_t *__restrict__ ray_angle,
-                           int ablk, int cap, int32_t *__restrict__ hist)
+// Sort keys of the characteristics, longest first: cap - length.
+__global__ void k_ray_keys(int64_t n_rays, const int64_t *__restrict__ ray_off, int cap, uint32_t *__restrict__ key)
 {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x) {
-        const int len = (int)(ray_off[r + 1] - ray_off[r]);
-        atomicAdd(hist + (int64_t)(ray_angle[r] / ablk) * (cap + 1) + (cap - len), 1);
-    }
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x)
+        key[r] = (uint32_t)(cap - (int)(ray_off[r + 1] - ray_off[r]));
 }
 
-// order: the block's characteristics, longest first; olen: their lengths.
-__global__ void k_ray_place(int64_t n_rays, const int64_t *__restrict__ ray_off, const int32_t *__restrict__ ray_angle,
-                            int ablk, int cap, unsigned long long *__restrict__ cursor, int32_t *__restrict__ order,
+// order holds a block's characteristics relative to r_lo: make them global, and note their lengths.
+__global__ void k_ray_order(int64_t r_lo, int64_t n, const int64_t *__restrict__ ray_off, int32_t *__restrict__ order,
                             int32_t *__restrict__ olen)
 {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n_rays; r += (int64_t)gridDim.x * blockDim.x) {
-        const int len = (int)(ray_off[r + 1] - ray_off[r]);
-        const int64_t p = (int64_t)atomicAdd(cursor + (int64_t)(ray_angle[r] / ablk) * (cap + 1) + (cap - len), 1ull);
-        order[p] = (int32_t)r;
-        olen[p] = len;
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = r_lo + order[r_lo + p];
+        order[r_lo + p] = (int32_t)r;
+        olen[r_lo + p] = (int32_t)(ray_off[r + 1] - ray_off[r]);
     }
 }
 
@@ -247,18 +242,16 @@ dim3 slot_grid(const Ray64 &m) { return dim3(rblocks(32 * m.ngroups, 128), 8); }
 
 }  // namespace
 
-cudaError_t ray64_hist(int64_t n_rays, const int64_t *ray_off, const int32_t *ray_angle, int ablk, int cap,
-                       int32_t *hist, cudaStream_t st)
+cudaError_t ray64_keys(int64_t n_rays, const int64_t *ray_off, int cap, uint32_t *key, cudaStream_t st)
 {
-    k_ray_hist<<<rcap(n_rays), 256, 0, st>>>(n_rays, ray_off, ray_angle, ablk, cap, hist);
+    k_ray_keys<<<rcap(n_rays), 256, 0, st>>>(n_rays, ray_off, cap, key);
     return cudaGetLastError();
 }
 
-cudaError_t ray64_place(int64_t n_rays, const int64_t *ray_off, const int32_t *ray_angle, int ablk, int cap,
-                        int64_t *cursor, int32_t *order, int32_t *olen, cudaStream_t st)
+cudaError_t ray64_order(int64_t r_lo, int64_t n, const int64_t *ray_off, int32_t *order, int32_t *olen, cudaStream_t st)
 {
-    k_ray_place<<<rcap(n_rays), 256, 0, st>>>(n_rays, ray_off, ray_angle, ablk, cap,
-                                              reinterpret_cast<unsigned long long *>(cursor), order, olen);
+    if (n <= 0) return cudaSuccess;
+    k_ray_order<<<rcap(n), 256, 0, st>>>(r_lo, n, ray_off, order, olen);
     return cudaGetLastError();
 }
 

@@ -919,11 +919,13 @@ void *keep_alloc(rt_grid *g, size_t bytes)
 bool ray64_setup(rt_grid *g)
 {
     const int cap = geom_scratch_cap(g->G);  // no characteristic is longer
-    const int64_t nh = (int64_t)g->nblk * (cap + 1);
     g->h_rg0.assign(g->nblk + 1, 0);
+    auto r_lo = [&](int b) { return g->h_ang_ray_off[g->blk_w0[b]]; };
+    auto nrays = [&](int b) { return g->h_ang_ray_off[g->blk_w0[b] + g->blk_nw[b]] - r_lo(b); };
+    RadixScratch rs{};
     for (int b = 0; b < g->nblk; ++b) {
-        const int64_t nr = g->h_ang_ray_off[g->blk_w0[b] + g->blk_nw[b]] - g->h_ang_ray_off[g->blk_w0[b]];
-        g->h_rg0[b + 1] = g->h_rg0[b] + (nr + 31) / 32;
+        g->h_rg0[b + 1] = g->h_rg0[b] + (nrays(b) + 31) / 32;
+        rs.cap = std::max(rs.cap, nrays(b));
     }
     const int64_t ng = g->h_rg0[g->nblk];
     struct Tmp {
@@ -943,29 +945,39 @@ bool ray64_setup(rt_grid *g)
             return q;
         }
     } tmp;
-    int32_t *hist = (int32_t *)tmp.get(4 * nh), *gw = (int32_t *)tmp.get(4 * std::max<int64_t>(1, ng));
-    int64_t *cursor = (int64_t *)tmp.get(8 * (nh + 1));
-    int64_t *stmp = (int64_t *)tmp.get(8 * (size_t)scan_tmp_elems(std::max(nh, ng)));
+    const int64_t nhist = 256 * radix_tiles(rs.cap);
+    rs.kA = (uint32_t *)tmp.get(4 * (size_t)rs.cap);
+    rs.kB = (uint32_t *)tmp.get(4 * (size_t)rs.cap);
+    rs.vA = (int32_t *)tmp.get(4 * (size_t)rs.cap);
+    rs.vB = (int32_t *)tmp.get(4 * (size_t)rs.cap);
+    rs.hist = (int32_t *)tmp.get(4 * (size_t)nhist);
+    rs.off = (int64_t *)tmp.get(8 * (size_t)(nhist + 1));
+    rs.tmp = (int64_t *)tmp.get(8 * (size_t)scan_tmp_elems(nhist));
+    uint32_t *key = (uint32_t *)tmp.get(4 * (size_t)g->n_rays);
+    int32_t *cnt = (int32_t *)tmp.get(4 * (size_t)(cap + 1)), *coff = (int32_t *)tmp.get(4 * (size_t)(cap + 2));
+    int64_t *ctmp = (int64_t *)tmp.get(8 * (size_t)(cap + 2 + scan_tmp_elems(cap + 1)));
+    int32_t *gw = (int32_t *)tmp.get(4 * std::max<int64_t>(1, ng));
+    int64_t *stmp = (int64_t *)tmp.get(8 * (size_t)scan_tmp_elems(ng));
     g->d_rorder = (int32_t *)keep_alloc(g, 4 * (size_t)g->n_rays);
     g->d_rlen = (int32_t *)keep_alloc(g, 4 * (size_t)g->n_rays);
     g->d_rgbase = (int64_t *)keep_alloc(g, 8 * (size_t)(ng + 1));
-    if (!hist || !gw || !cursor || !stmp || !g->d_rorder || !g->d_rlen || !g->d_rgbase) return false;
-    if (cudaMemsetAsync(hist, 0, 4 * nh, g->st) != cudaSuccess ||
-        ray64_hist(g->n_rays, g->d_ray_off, g->d_ray_angle, g->ablk, cap, hist, g->st) != cudaSuccess ||
-        scan_i32(hist, cursor, nh, stmp, g->st) != cudaSuccess ||
-        ray64_place(g->n_rays, g->d_ray_off, g->d_ray_angle, g->ablk, cap, cursor, g->d_rorder, g->d_rlen, g->st) !=
-            cudaSuccess)
+    if (!rs.kA || !rs.kB || !rs.vA || !rs.vB || !rs.hist || !rs.off || !rs.tmp || !key || !cnt || !coff || !ctmp || !gw ||
+        !stmp || !g->d_rorder || !g->d_rlen || !g->d_rgbase)
         return false;
+    // stable: characteristics of one length stay in launch order, so that the lanes
+    // of a group have neighbouring origins and look up neighbouring voxels
+    if (ray64_keys(g->n_rays, g->d_ray_off, cap, key, g->st) != cudaSuccess) return false;
     for (int b = 0; b < g->nblk; ++b)
-        if (ray64_group_slots(g->h_ang_ray_off[g->blk_w0[b]], g->h_rg0[b + 1] - g->h_rg0[b], g->d_rlen,
-                              gw + g->h_rg0[b], g->st) != cudaSuccess)
+        if (csr_build(cap + 1, key + r_lo(b), nrays(b), cnt, coff, g->d_rorder + r_lo(b), ctmp, rs, g->st) != cudaSuccess ||
+            ray64_order(r_lo(b), nrays(b), g->d_ray_off, g->d_rorder, g->d_rlen, g->st) != cudaSuccess ||
+            ray64_group_slots(r_lo(b), g->h_rg0[b + 1] - g->h_rg0[b], g->d_rlen, gw + g->h_rg0[b], g->st) != cudaSuccess)
             return false;
     int64_t slots = 0;
     if (scan_i32(gw, g->d_rgbase, ng, stmp, g->st) != cudaSuccess ||
         cudaMemcpyAsync(&slots, g->d_rgbase + ng, sizeof(int64_t), cudaMemcpyDeviceToHost, g->st) != cudaSuccess ||
         cudaStreamSynchronize(g->st) != cudaSuccess)
         return false;
-    g->launches += 6 + g->nblk;
+    g->launches += 4 + 12 * g->nblk;
     g->d_wp64 = (uint2 *)keep_alloc(g, sizeof(uint2) * (size_t)slots);
     g->d_cw64 = (Wd4 *)keep_alloc(g, sizeof(Wd4) * (size_t)slots);
     g->d_cg64 = (double *)keep_alloc(g, sizeof(double) * (size_t)slots);

@@ -246,13 +246,11 @@ struct Ray64 {
     Wd4 *cw;
     double *cg;            // w_Omega l / L
 };
-// Counting sort of the characteristics by length within their angle blocks
-// (blocks of ablk solid angles): hist holds cap + 1 lengths per block, its
-// exclusive scan is the cursor.
-cudaError_t ray64_hist(int64_t n_rays, const int64_t *ray_off, const int32_t *ray_angle, int ablk, int cap,
-                       int32_t *hist, cudaStream_t st);
-cudaError_t ray64_place(int64_t n_rays, const int64_t *ray_off, const int32_t *ray_angle, int ablk, int cap,
-                        int64_t *cursor, int32_t *order, int32_t *olen, cudaStream_t st);
+// Sort keys cap - length of all characteristics; after the block's stable sort
+// by key (csr_build with order as its list) ray64_order makes its entries global
+// and notes the lengths.
+cudaError_t ray64_keys(int64_t n_rays, const int64_t *ray_off, int cap, uint32_t *key, cudaStream_t st);
+cudaError_t ray64_order(int64_t r_lo, int64_t n, const int64_t *ray_off, int32_t *order, int32_t *olen, cudaStream_t st);
 cudaError_t ray64_group_slots(int64_t r_lo, int64_t ngroups, const int32_t *olen, int32_t *gw, cudaStream_t st);
 // Words, output positions (pos, or the segment's place in its block when NULL)
 // and gather weights; once per grid.  Weights; once per chi.
