@@ -404,7 +404,7 @@ int adjoint_pass(rt_grid *g, bool full, int homog, const double *u, const double
         if (ns <= 0) continue;
         if (full) {
             ACK(march_block_I(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64, g->d_B, g->I_outer,
-                              homog, (double *)g->d_segbuf, g->march_chunk, g->st));
+                              homog, (double *)g->d_segbuf, g->chunk(), g->st));
             k_adjoint<true><<<(unsigned)blocks, 256, 0, g->st>>>(
                 g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64, g->d_B, g->I_outer, homog, u, gc,
                 g->d_invL, g->d_wt, g->d_dirs, g->d_ang_seg_off, w0, nw, n, (const double *)g->d_segbuf, nullptr, tC,

@@ -47,10 +47,18 @@ __global__ void k_pack32(int n, const double *chi, const double *S, const double
     }
 }
 
+// S in FP32 for the streamed-weight march, in the order of vblk (NULL: the grid's).
+__global__ void k_prep32(int n, const double *S, const int32_t *vblk, float *S32)
+{
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < n) S32[vblk ? vblk[v] : v] = (float)S[v];
+}
+
 __global__ void k_ali(int n, double *S, const double *J, const double *L, const double *eps, const double *B,
-                      int use_lstar, double *slot, unsigned long long *maxrel)
+                      int use_lstar, double *slot, unsigned long long *maxrel, unsigned long long *zero)
 {
     int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v == 0) *zero = 0ull;  // the next update's maximum
     double rel = 0.0;
     if (v < n) {
         double e = eps[v];
@@ -113,7 +121,9 @@ __global__ void k_fill(int n, double *x, double val)
 
 // Ng normal-equation sums over voxels with weights 1/wref^2 (wref = y0 if null).
 __global__ void __launch_bounds__(NG_THREADS) k_ng_dots(int n, const double *y0, const double *y1, const double *y2,
-                                                        const double *y3, const double *wref, double *partial)
+                                                        const double *y3, const double *wref, double *partial,
+                                                        unsigned *ticket, const unsigned long long *rel, double tol,
+                                                        double *coef)
 {
     __shared__ double sh[5][NG_THREADS];
     double a11 = 0, a12 = 0, a22 = 0, b1 = 0, b2 = 0;
@@ -136,15 +146,22 @@ __global__ void __launch_bounds__(NG_THREADS) k_ng_dots(int n, const double *y0,
             for (int c = 0; c < 5; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x < 5) partial[blockIdx.x * 5 + threadIdx.x] = sh[threadIdx.x][0];
-}
-
-__global__ void __launch_bounds__(NG_THREADS) k_ng_solve(const double *partial, double *coef)
-{
-    __shared__ double sh[5][NG_THREADS];
+    __shared__ bool last;
+    if (threadIdx.x < 5) __stcg(partial + blockIdx.x * 5 + threadIdx.x, sh[threadIdx.x][0]);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == (unsigned)gridDim.x - 1u;
+    }
+    __syncthreads();
+    if (!last) return;
+    // the block that finishes last adds the partials, in one fixed order, and solves
+    __threadfence();
+    if (threadIdx.x == 0) *ticket = 0u;
     double acc[5] = {0, 0, 0, 0, 0};
     for (int b = threadIdx.x; b < NG_BLOCKS; b += NG_THREADS)
-        for (int c = 0; c < 5; ++c) acc[c] += partial[b * 5 + c];
+        for (int c = 0; c < 5; ++c) acc[c] += __ldcg(partial + b * 5 + c);
+    __syncthreads();
     for (int c = 0; c < 5; ++c) sh[c][threadIdx.x] = acc[c];
     __syncthreads();
     for (int s = NG_THREADS / 2; s > 0; s >>= 1) {
@@ -156,6 +173,7 @@ __global__ void __launch_bounds__(NG_THREADS) k_ng_solve(const double *partial, 
         double A11 = sh[0][0], A12 = sh[1][0], A22 = sh[2][0], b1 = sh[3][0], b2 = sh[4][0];
         double det = A11 * A22 - A12 * A12;
         bool ok = (fabs(det) > 1e-14 * (A11 * A22)) && (det == det);
+        if (rel && __longlong_as_double((long long)*rel) < tol) ok = false;  // converged: the iterate stays
         coef[0] = ok ? (b1 * A22 - b2 * A12) / det : 0.0;
         coef[1] = ok ? (A11 * b2 - A12 * b1) / det : 0.0;
         coef[2] = ok ? 1.0 : 0.0;
@@ -176,7 +194,7 @@ inline unsigned nb(int n) { return (unsigned)((n + 255) / 256); }
 
 }  // namespace
 
-int ng_partial_elems(int) { return NG_BLOCKS * 5; }
+int ng_partial_elems(int) { return NG_BLOCKS * 5 + 1; }  // and the ticket, zero before the first use
 
 cudaError_t pack_chiS64(int nvox, const double *chi, const double *S, double2 *cs, cudaStream_t st)
 {
@@ -226,17 +244,25 @@ cudaError_t pack_preload()
 }
 
 cudaError_t ali_update(int nvox, double *S, const double *J, const double *Lst, const double *eps, const double *B,
-                       int use_lstar, double *hist_slot, unsigned long long *maxrel, cudaStream_t st)
+                       int use_lstar, double *hist_slot, unsigned long long *maxrel, unsigned long long *zero,
+                       cudaStream_t st)
 {
-    k_ali<<<nb(nvox), 256, 0, st>>>(nvox, S, J, Lst, eps, B, use_lstar, hist_slot, maxrel);
+    k_ali<<<nb(nvox), 256, 0, st>>>(nvox, S, J, Lst, eps, B, use_lstar, hist_slot, maxrel, zero);
+    return cudaGetLastError();
+}
+
+cudaError_t prep_S32(int nvox, const double *S, const int32_t *vblk, float *S32, cudaStream_t st)
+{
+    k_prep32<<<nb(nvox), 256, 0, st>>>(nvox, S, vblk, S32);
     return cudaGetLastError();
 }
 
 cudaError_t ng_extrapolate(int nvox, const double *y0, const double *y1, const double *y2, const double *y3,
-                           const double *wref, double *partial, double *coef, double *out, cudaStream_t st)
+                           const double *wref, double *partial, double *coef, double *out, cudaStream_t st,
+                           const unsigned long long *rel, double tol)
 {
-    k_ng_dots<<<NG_BLOCKS, NG_THREADS, 0, st>>>(nvox, y0, y1, y2, y3, wref, partial);
-    k_ng_solve<<<1, NG_THREADS, 0, st>>>(partial, coef);
+    k_ng_dots<<<NG_BLOCKS, NG_THREADS, 0, st>>>(nvox, y0, y1, y2, y3, wref, partial,
+                                                reinterpret_cast<unsigned *>(partial + NG_BLOCKS * 5), rel, tol, coef);
     k_ng_apply<<<nb(nvox), 256, 0, st>>>(nvox, y0, y1, y2, coef, out);
     return cudaGetLastError();
 }

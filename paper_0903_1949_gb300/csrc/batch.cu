@@ -1016,7 +1016,8 @@ int rt_line_create(rt_batch **out, rt_grid *g, int n_freq, const double *phi, co
         set_last_error(keep.c_str());
         return rc;
     }
-    if (cudaMemcpyAsync(b->phi, phi, sizeof(double) * n_freq, cudaMemcpyHostToDevice, b->st) != cudaSuccess ||
+    if ((ng && cudaMemsetAsync(b->ng_part, 0, sizeof(double) * ng_partial_elems(n), b->st) != cudaSuccess) ||
+        cudaMemcpyAsync(b->phi, phi, sizeof(double) * n_freq, cudaMemcpyHostToDevice, b->st) != cudaSuccess ||
         cudaMemcpyAsync(b->wq, wq, sizeof(double) * n_freq, cudaMemcpyHostToDevice, b->st) != cudaSuccess ||
         fill_const(n, b->ones, 1.0, b->st) != cudaSuccess || cudaStreamSynchronize(b->st) != cudaSuccess) {
         rt_batch_destroy(b);

@@ -797,17 +797,6 @@ __global__ void k_make_voxb(const uint32_t *__restrict__ vox, int64_t nseg, cons
     }
 }
 
-__global__ void k_blk_scatter(int nvox, const int32_t *__restrict__ vblk, const float *__restrict__ S,
-                              const float *__restrict__ B, float *__restrict__ Sb, float *__restrict__ Bb)
-{
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < nvox) {
-        const int q = vblk[v];
-        Sb[q] = S[v];
-        Bb[q] = B[v];
-    }
-}
-
 unsigned grid_cap(int64_t n)
 {
     int64_t b = (n + 255) / 256;
@@ -821,13 +810,6 @@ cudaError_t make_voxb(const uint32_t *vox, int64_t nseg, const int32_t *vblk, ui
 {
     if (nseg <= 0) return cudaSuccess;
     k_make_voxb<<<grid_cap(nseg), 256, 0, st>>>(vox, nseg, vblk, voxb);
-    return cudaGetLastError();
-}
-
-cudaError_t blk_scatter(int nvox, const int32_t *vblk, const float *S, const float *B, float *Sb, float *Bb,
-                        cudaStream_t st)
-{
-    k_blk_scatter<<<(nvox + 255) / 256, 256, 0, st>>>(nvox, vblk, S, B, Sb, Bb);
     return cudaGetLastError();
 }
 

@@ -56,7 +56,11 @@ struct rt_grid {
     double *d_H = nullptr, *d_ng_part = nullptr, *d_ng_coef = nullptr;
     unsigned long long *d_maxrel = nullptr;
     double *d_r = nullptr, *d_delta = nullptr, *d_Jd = nullptr, *d_Ld = nullptr, *d_Fcd = nullptr, *d_Lkeep = nullptr;
-    double *h_pin = nullptr;  // pinned scalars read back by the iteration control
+    // scalars of the iteration control, read back in one copy: [0] a maximum, [2] the error
+    // flag, [3..5] the Ng coefficients and whether they were applied, [6] and [7] the ALI
+    // updates' maxima in turn (an update clears the other one's)
+    double *d_stat = nullptr, *h_pin = nullptr;
+    int mr = 0;
     int *d_lost = nullptr;
     int lost = 0;
     double geom_ms = 0.0, geom_trace_ms = 0.0, geom_lists_ms = 0.0;
@@ -73,6 +77,15 @@ struct rt_grid {
     std::vector<int64_t> ev_segs;
     int64_t launches = 0;
     int march_chunk = 512;  // segments per warp bundle (RT_TUNE_MARCH_CHUNK)
+    // The bundle size in use: the default is lowered on small grids until the
+    // largest angle block has 16 bundles an SM (a warp takes its bundle 32 segments
+    // after 32: 16 us for 2.7e4 segments in bundles of 512).
+    int chunk() const
+    {
+        int c = march_chunk;
+        while (march_chunk == 512 && c > 64 && max_blk_seg < (int64_t)c * 152 * 16) c /= 2;
+        return c;
+    }
     std::vector<int64_t> ev_bytes;  // streamed DRAM bytes of each timed march launch
     // streamed-weight FP32 march (RT_TUNE_STREAMED_WEIGHTS)
     float4 *d_cw4 = nullptr;  // (E, alpha, beta, gamma) per segment for the current chi
@@ -92,6 +105,7 @@ struct rt_grid {
     bool cw64_ok = false;
     int pos_state = 0;        // list positions: 0 not tried, 1 allocated, -1 not available
     bool cw_ok = false;       // d_cw4 matches the current chi
+    bool b32_ok = false, b32b_ok = false;  // d_B32 and d_B32b match the current B
     int sw_coarsen = 1;       // segments per lane (RT_TUNE_MARCH_COARSEN)
     int sw_overlap = 1;       // gather of block b on st2 while block b + 1 is marched (RT_TUNE_OVERLAP)
     int sw_scatter = 1;       // march stores in ownership-list order (RT_TUNE_SCATTER)

@@ -114,12 +114,12 @@ int rt_fs_angle_noalloc(rt_grid *g, int omega, int precision, double *Ibar, doub
         if ((e = rtk::pack_chiS64(n, g->d_chi, g->d_S, g->d_cs64, g->st)) != cudaSuccess)
             return nofail(RT_ECUDA, cudaGetErrorString(e));
         e = rtk::march_block<double, double2>(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, s_lo, nseg, g->d_cs64,
-                                              g->d_B, g->I_outer, 0, para, (double2 *)scratch, g->march_chunk, g->st);
+                                              g->d_B, g->I_outer, 0, para, (double2 *)scratch, g->chunk(), g->st);
     } else {
         if ((e = rtk::pack_chiS32(n, g->d_chi, g->d_S, g->d_B, g->d_cs32, g->d_B32, nullptr, g->st)) != cudaSuccess)
             return nofail(RT_ECUDA, cudaGetErrorString(e));
         e = rtk::march_block<float, float2>(g->d_vox, g->d_len32, g->d_ray_off, r_lo, r_hi, s_lo, nseg, g->d_cs32,
-                                            g->d_B32, (float)g->I_outer, 0, para, (float2 *)scratch, g->march_chunk,
+                                            g->d_B32, (float)g->I_outer, 0, para, (float2 *)scratch, g->chunk(),
                                             g->st);
     }
     if (e != cudaSuccess) return nofail(RT_ECUDA, cudaGetErrorString(e));

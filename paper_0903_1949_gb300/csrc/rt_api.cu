@@ -691,10 +691,12 @@ int alloc_fields(rt_grid *g)
     RCK(dalloc(g, &g->d_S32, n));
     RCK(dalloc(g, &g->d_H, 4 * (size_t)n));
     RCK(dalloc(g, &g->d_ng_part, ng_partial_elems(n)));
-    RCK(dalloc(g, &g->d_ng_coef, 4));
-    RCK(dalloc(g, &g->d_maxrel, 1));
-    RCK(dalloc(g, &g->d_err, 1));
-    CK(cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st));
+    CK(cudaMemsetAsync(g->d_ng_part, 0, sizeof(double) * ng_partial_elems(n), g->st));
+    RCK(dalloc(g, &g->d_stat, 8));
+    CK(cudaMemsetAsync(g->d_stat, 0, 8 * sizeof(double), g->st));
+    g->d_maxrel = (unsigned long long *)g->d_stat;
+    g->d_err = (int *)(g->d_stat + 2);
+    g->d_ng_coef = g->d_stat + 3;
     RCK(dalloc(g, &g->d_r, n));
     RCK(dalloc(g, &g->d_delta, n));
     RCK(dalloc(g, &g->d_Jd, n));
@@ -740,7 +742,7 @@ int run_fs(rt_grid *g, int prec, int homog, const double *S_src, double *J, doub
             double2 *buf = (double2 *)g->d_segbuf;
             t0 = tstart(g, 0);
             CK(march_block<double, double2>(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64, g->d_B,
-                                            g->I_outer, homog, para, buf, g->march_chunk, g->st));
+                                            g->I_outer, homog, para, buf, g->chunk(), g->st));
             tstop(g, t0, 0, ns, 12 * ns);
             t1 = tstart(g, 1);
             CK(gather_block<double2>(n, off, g->d_perm + lo, buf, g->d_ang_seg_off, w0, nw, lo, g->d_invL, g->d_wL32,
@@ -754,7 +756,7 @@ int run_fs(rt_grid *g, int prec, int homog, const double *S_src, double *J, doub
             float2 *buf = (float2 *)g->d_segbuf;
             t0 = tstart(g, 0);
             CK(march_block<float, float2>(g->d_vox, g->d_len32, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs32, g->d_B32,
-                                          (float)g->I_outer, homog, para, buf, g->march_chunk, g->st));
+                                          (float)g->I_outer, homog, para, buf, g->chunk(), g->st));
             tstop(g, t0, 0, ns, 8 * ns);
             t1 = tstart(g, 1);
             CK(gather_block<float2>(n, off, g->d_perm + lo, buf, g->d_ang_seg_off, w0, nw, lo, g->d_invL, g->d_wL32,
@@ -801,12 +803,12 @@ bool sw_common(rt_grid *g)
             g->pos_state = -1;
         }
     }
-    if (g->bnd_chunk != g->march_chunk) {  // bundle bounds for the current chunk
+    if (g->bnd_chunk != g->chunk()) {  // bundle bounds for the current chunk
         std::vector<int64_t> off(g->nblk + 1, 0);
         for (int b = 0; b < g->nblk; ++b) {
             const int w0 = g->blk_w0[b], nw = g->blk_nw[b];
             const int64_t ns = g->h_ang_seg_off[w0 + nw] - g->h_ang_seg_off[w0];
-            off[b + 1] = off[b] + (ns + g->march_chunk - 1) / g->march_chunk;
+            off[b + 1] = off[b] + (ns + g->chunk() - 1) / g->chunk();
         }
         if (g->d_bnd) {
             cudaFree(g->d_bnd);
@@ -824,13 +826,13 @@ bool sw_common(rt_grid *g)
         for (int b = 0; b < g->nblk; ++b) {
             const int w0 = g->blk_w0[b], nw = g->blk_nw[b];
             const int64_t lo = g->h_ang_seg_off[w0], ns = g->h_ang_seg_off[w0 + nw] - lo;
-            if (sw_bundles(g->d_ray_off, g->h_ang_ray_off[w0], g->h_ang_ray_off[w0 + nw], lo, ns, g->march_chunk,
+            if (sw_bundles(g->d_ray_off, g->h_ang_ray_off[w0], g->h_ang_ray_off[w0 + nw], lo, ns, g->chunk(),
                            g->d_bnd + off[b], g->st) != cudaSuccess)
                 return false;
             g->launches++;
         }
         g->h_bnd_off = off;
-        g->bnd_chunk = g->march_chunk;
+        g->bnd_chunk = g->chunk();
     }
     return true;
 }
@@ -1042,6 +1044,7 @@ bool build_sblk(rt_grid *g)
                 const int64_t blk = ((int64_t)(i / 4) * nbj + j / 2) * nbk + k / 4;
                 h[((int64_t)i * n2 + j) * n3 + k] = (int32_t)(blk * 32 + ((i % 4) * 2 + j % 2) * 4 + k % 4);
             }
+    g->b32b_ok = false;
     void *a = nullptr, *b = nullptr, *c = nullptr, *d = nullptr;
     auto al = [&](void **q, size_t bytes) {
         if (cudaMalloc(q, bytes) != cudaSuccess) {
@@ -1069,6 +1072,21 @@ bool build_sblk(rt_grid *g)
     g->launches++;
     g->sblk_state = 1;
     return true;
+}
+
+// S_src (and, when it changed, B) in FP32 for the streamed-weight march.
+int prep32(rt_grid *g, const double *S_src, cudaStream_t st)
+{
+    const bool blk = g->sblk && build_sblk(g);
+    CK(prep_S32(g->nvox, S_src, blk ? g->d_vblk : nullptr, blk ? g->d_S32b : g->d_S32, st));
+    g->launches++;
+    bool &ok = blk ? g->b32b_ok : g->b32_ok;
+    if (!ok) {
+        CK(prep_S32(g->nvox, g->d_B, blk ? g->d_vblk : nullptr, blk ? g->d_B32b : g->d_B32, st));
+        g->launches++;
+        ok = true;
+    }
+    return RT_OK;
 }
 
 SwMarch sw_march(rt_grid *g, int b, int homog, float *out)
@@ -1163,10 +1181,7 @@ int run_fs_J_sw(rt_grid *g, int prec, int homog, const double *S_src, double *J)
         return scatter ? gather_rows_sw_launch(t, g->nvox, st) : gather_sw_launch(t, st);
     };
     if (!g->sw_overlap) {
-        if (!f64 && g->sblk && build_sblk(g)) {  // this step's FP32 S and B in the blocked order
-            CK(blk_scatter(g->nvox, g->d_vblk, g->d_S32, g->d_B32, g->d_S32b, g->d_B32b, g->st));
-            g->launches++;
-        }
+        if (!f64) RCK(prep32(g, S_src, g->st));
         for (int b = 0; b < g->nblk; ++b) {
             int t0 = tstart(g, 0);
             CK(march(b, 0, g->st));
@@ -1243,10 +1258,7 @@ int run_fs_J_sw_streams(rt_grid *g, int prec, int homog, const double *S_src, do
     auto segs = [&](int b) -> int64_t {
         return g->h_ang_seg_off[g->blk_w0[b] + g->blk_nw[b]] - g->h_ang_seg_off[g->blk_w0[b]];
     };
-    if (!f64 && g->sblk && build_sblk(g)) {  // this step's FP32 S and B in the blocked order
-        CK(blk_scatter(g->nvox, g->d_vblk, g->d_S32, g->d_B32, g->d_S32b, g->d_B32b, base));
-        g->launches++;
-    }
+    if (!f64) RCK(prep32(g, S_src, base));
     auto march = [&](int b, int q, cudaStream_t st) -> cudaError_t {
         if (!f64) return march_sw_launch(sw_march(g, b, homog, b32[q]), g->sw_coarsen, st);
         return ray64_march(ray64_block(g, b), S_src, g->d_B, g->I_outer, homog, b64[q], st);
@@ -1301,12 +1313,12 @@ int run_fs_J_sw_streams(rt_grid *g, int prec, int homog, const double *S_src, do
 int run_fs_J(rt_grid *g, int prec, int homog, const double *S_src, double *J)
 {
     const int n = g->nvox;
-    if (prec == RT_FP64) CK(pack_chiS64(n, g->d_chi, S_src, g->d_cs64, g->st));
-    else CK(pack_chiS32(n, g->d_chi, S_src, g->d_B, g->d_cs32, g->d_B32, g->d_S32, g->st));
-    g->launches++;
     if (prec == RT_MIXED && use_sw(g)) return run_fs_J_sw(g, prec, homog, S_src, J);
     if (prec == RT_FP64 && use_sw64(g)) return run_fs_J_sw(g, prec, homog, S_src, J);
     CK(cudaGetLastError());
+    if (prec == RT_FP64) CK(pack_chiS64(n, g->d_chi, S_src, g->d_cs64, g->st));
+    else CK(pack_chiS32(n, g->d_chi, S_src, g->d_B, g->d_cs32, g->d_B32, g->d_S32, g->st));
+    g->launches++;
     for (int b = 0; b < g->nblk; ++b) {
         int w0 = g->blk_w0[b], nw = g->blk_nw[b];
         int64_t r_lo = g->h_ang_ray_off[w0], r_hi = g->h_ang_ray_off[w0 + nw];
@@ -1317,7 +1329,7 @@ int run_fs_J(rt_grid *g, int prec, int homog, const double *S_src, double *J)
             double *buf = (double *)g->d_segbuf;
             t0 = tstart(g, 0);
             CK(march_block_J<double, double2>(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64, g->d_B,
-                                              g->I_outer, homog, buf, g->march_chunk, g->st));
+                                              g->I_outer, homog, buf, g->chunk(), g->st));
             tstop(g, t0, 0, ns, 12 * ns);
             t1 = tstart(g, 1);
             CK(gather_J<double>(n, off, g->jt[b], g->d_perm + lo, buf, g->d_ang_seg_off, w0, nw, lo, g->d_wL32,
@@ -1327,7 +1339,7 @@ int run_fs_J(rt_grid *g, int prec, int homog, const double *S_src, double *J)
             float *buf = (float *)g->d_segbuf;
             t0 = tstart(g, 0);
             CK(march_block_J<float, float2>(g->d_vox, g->d_len32, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs32,
-                                            g->d_B32, (float)g->I_outer, homog, buf, g->march_chunk, g->st));
+                                            g->d_B32, (float)g->I_outer, homog, buf, g->chunk(), g->st));
             tstop(g, t0, 0, ns, 8 * ns);
             t1 = tstart(g, 1);
             CK(gather_J<float>(n, off, g->jt[b], g->d_perm + lo, buf, g->d_ang_seg_off, w0, nw, lo, g->d_wL32,
@@ -1350,12 +1362,12 @@ int fs_iteration(rt_grid *g, int prec, const double *S_src, double *J)
     return RT_OK;
 }
 
-int read_maxrel(rt_grid *g, double *rel)
+// The iteration's scalars, read in one copy; *rel is the maximum at word `at`.
+int read_maxrel(rt_grid *g, double *rel, int at = 0)
 {
-    CK(cudaMemcpyAsync(g->h_pin, g->d_maxrel, sizeof(double), cudaMemcpyDeviceToHost, g->st));
-    CK(cudaMemcpyAsync(g->h_pin + 2, g->d_err, sizeof(int), cudaMemcpyDeviceToHost, g->st));
+    CK(cudaMemcpyAsync(g->h_pin, g->d_stat, 8 * sizeof(double), cudaMemcpyDeviceToHost, g->st));
     RCK(sync(g));
-    *rel = g->h_pin[0];  // the device word holds the bits of a non-negative double
+    *rel = g->h_pin[at];  // the device word holds the bits of a non-negative double
     int err = 0;
     std::memcpy(&err, g->h_pin + 2, sizeof(int));
     if (err) {
@@ -1384,20 +1396,27 @@ double *ng_append_slot(rt_grid *g)
     return g->d_H + (size_t)g->hs[g->nh] * g->nvox;
 }
 
-// After an iterate was written to the slot from ng_append_slot: extrapolate
-// into `out` once four iterates are stored; clears the history if applied.
-int ng_maybe(rt_grid *g, double *out, const double *wref)
+// After an iterate was written to the slot from ng_append_slot: queue the
+// extrapolation into `out` once four iterates are stored, unless the maximum at
+// rel (device) is below tol; the next read_maxrel says whether it was applied.
+int ng_queue(rt_grid *g, double *out, const double *wref, const unsigned long long *rel, double tol, bool *queued)
 {
-    g->nh++;
-    if (g->nh < 4) return RT_OK;
+    *queued = g->ng && g->nh == 3;
+    if (!*queued) return RT_OK;
     const size_t n = g->nvox;
     CK(ng_extrapolate(g->nvox, g->d_H + g->hs[3] * n, g->d_H + g->hs[2] * n, g->d_H + g->hs[1] * n,
-                      g->d_H + g->hs[0] * n, wref, g->d_ng_part, g->d_ng_coef, out, g->st));
-    g->launches += 3;
-    CK(cudaMemcpyAsync(g->h_pin + 1, g->d_ng_coef + 2, sizeof(double), cudaMemcpyDeviceToHost, g->st));
-    RCK(sync(g));
-    if (g->h_pin[1] != 0.0) g->nh = 0;
+                      g->d_H + g->hs[0] * n, wref, g->d_ng_part, g->d_ng_coef, out, g->st, rel, tol));
+    g->launches += 2;
     return RT_OK;
+}
+
+// The iterate counts (it did not meet the tolerance): the history is spent when
+// the extrapolation was applied.
+void ng_count(rt_grid *g, bool queued)
+{
+    if (!g->ng) return;
+    g->nh++;
+    if (queued && g->h_pin[5] != 0.0) g->nh = 0;
 }
 
 // Nearest-neighbour Lambda* of the current chi (FP64, once per chi): per
@@ -1501,8 +1520,11 @@ int nn_solve(rt_grid *g, const double *y, double **x_out, double jtol = 0.0)
     return RT_OK;
 }
 
-int ali_step_impl(rt_grid *g, int prec, double *rel_out)
+// One iteration and, unless its change is below tol, the Ng step that is due.
+int ali_step_impl(rt_grid *g, int prec, double tol, double *rel_out)
 {
+    bool queued = false;
+    int at = 0;
     if (g->use_lstar == RT_LSTAR_NN) {
         RCK(build_nn(g));
         RCK(run_fs_J(g, prec, 0, g->d_S, g->d_J));
@@ -1513,21 +1535,21 @@ int ali_step_impl(rt_grid *g, int prec, double *rel_out)
         double *slot = g->ng ? ng_append_slot(g) : nullptr;
         CK(nn_apply(g->nvox, g->d_S, x, nullptr, slot, g->d_maxrel, g->st));
         g->launches += 2;
-        double rel = 0.0;
-        RCK(read_maxrel(g, &rel));
-        *rel_out = rel;
-        g->history.push_back(rel);
-        return RT_OK;
+    } else {
+        RCK(fs_iteration(g, prec, g->d_S, g->d_J));
+        at = 6 + g->mr;
+        g->mr ^= 1;
+        double *slot = g->ng ? ng_append_slot(g) : nullptr;
+        CK(ali_update(g->nvox, g->d_S, g->d_J, g->d_L, g->d_eps, g->d_B, g->use_lstar, slot, g->d_maxrel + at,
+                      g->d_maxrel + 6 + g->mr, g->st));
+        g->launches++;
     }
-    RCK(fs_iteration(g, prec, g->d_S, g->d_J));
-    CK(cudaMemsetAsync(g->d_maxrel, 0, sizeof(unsigned long long), g->st));
-    double *slot = g->ng ? ng_append_slot(g) : nullptr;
-    CK(ali_update(g->nvox, g->d_S, g->d_J, g->d_L, g->d_eps, g->d_B, g->use_lstar, slot, g->d_maxrel, g->st));
-    g->launches++;
+    RCK(ng_queue(g, g->d_S, nullptr, g->d_maxrel + at, tol, &queued));
     double rel = 0.0;
-    RCK(read_maxrel(g, &rel));
+    RCK(read_maxrel(g, &rel, at));
     *rel_out = rel;
     g->history.push_back(rel);
+    if (!(rel < tol)) ng_count(g, queued);
     return RT_OK;
 }
 
@@ -1592,7 +1614,7 @@ int rt_grid_member_fs(rt_grid *g, const float2 *cs, const float *B32, const uint
         const int32_t *off = g->d_csr_off + (size_t)b * (n + 1);
         float2 *buf = (float2 *)g->d_segbuf;
         CK(march_block_bits(g->d_vox, g->d_len32, g->d_ray_off, r_lo, r_hi, lo, ns, cs, B32, (float)g->I_outer, buf,
-                            g->march_chunk, pbits, st));
+                            g->chunk(), pbits, st));
         CK(gather_block<float2>(n, off, g->d_perm + lo, buf, g->d_ang_seg_off, w0, nw, lo, g->d_invL, g->d_wL32,
                                 g->d_wt, g->d_dirs, g->d_urow + g->h_ubase[b], g->d_ubeg + g->h_ubase[b],
                                 g->d_ufirst + (size_t)b * (n + 1), g->h_nunits[b], g->d_multi + g->h_mbase[b],
@@ -1635,7 +1657,7 @@ int rt_grid_member_fs64J(rt_grid *g, const double2 *cs64, const double *B64, con
         const int32_t *off = g->d_csr_off + (size_t)b * (n + 1);
         double *buf = (double *)g->d_segbuf;
         CK(march_block_bits64J(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, cs64, B64, g->I_outer, 0, buf,
-                               g->march_chunk, pbits, st));
+                               g->chunk(), pbits, st));
         CK(gather_J<double>(n, off, g->jt[b], g->d_perm + lo, buf, g->d_ang_seg_off, w0, nw, lo, g->d_wL32,
                             g->d_invL, g->d_wt, g->d_partJ, J, b == 0, st));
     }
@@ -1762,6 +1784,7 @@ int rt_set_opacity(rt_grid *g, const double *chi, const double *eps, const doubl
     g->cw_ok = false;
     g->cw64_ok = false;
     g->nn_ok = false;
+    g->b32_ok = g->b32b_ok = false;
     if (where == RT_HOST) RCK(sync(g));
     reset_ng(g);
     g->history.clear();
@@ -1906,8 +1929,7 @@ int rt_ali_step(rt_grid *g, double *max_rel_dS)
     RCK(check_lost(g));
     CK(cudaSetDevice(g->device));
     double rel = 0.0;
-    RCK(ali_step_impl(g, g->precision, &rel));
-    if (g->ng) RCK(ng_maybe(g, g->d_S, nullptr));
+    RCK(ali_step_impl(g, g->precision, 0.0, &rel));
     if (max_rel_dS) *max_rel_dS = rel;
     return RT_OK;
 }
@@ -1924,10 +1946,9 @@ int rt_solve(rt_grid *g, double tol, int max_iter, int *iters)
     if (g->precision == RT_FP64) {
         for (int it = 1; it <= max_iter; ++it) {
             double rel = 0.0;
-            RCK(ali_step_impl(g, RT_FP64, &rel));
+            RCK(ali_step_impl(g, RT_FP64, tol, &rel));
             if (iters) *iters = it;
             if (rel < tol) return RT_OK;
-            if (g->ng) RCK(ng_maybe(g, g->d_S, nullptr));
         }
         return fail(RT_ENOTCONVERGED, "no convergence to %g in %d iterations", tol, max_iter);
     }
@@ -1979,10 +2000,12 @@ int rt_solve(rt_grid *g, double tol, int max_iter, int *iters)
                                   g->d_maxrel, g->st));
             }
             g->launches++;
+            bool queued = false;
+            RCK(ng_queue(g, g->d_delta, g->d_S, g->d_maxrel, inner_tol, &queued));
             double rd = 0.0;
             RCK(read_maxrel(g, &rd));
             if (rd < inner_tol) break;
-            if (g->ng) RCK(ng_maybe(g, g->d_delta, g->d_S));
+            ng_count(g, queued);
         }
         CK(add_inplace(n, g->d_S, g->d_delta, g->st));
         g->launches++;
@@ -2108,10 +2131,10 @@ int rt_fs_angles(rt_grid *g, const int32_t *omegas, int n, int precision, double
             // results of this block are still in the buffer
         } else if (precision == RT_FP64)
             CK(march_block<double, double2>(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64, g->d_B,
-                                            g->I_outer, 0, para, (double2 *)g->d_segbuf, g->march_chunk, g->st));
+                                            g->I_outer, 0, para, (double2 *)g->d_segbuf, g->chunk(), g->st));
         else
             CK(march_block<float, float2>(g->d_vox, g->d_len32, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs32, g->d_B32,
-                                          (float)g->I_outer, 0, para, (float2 *)g->d_segbuf, g->march_chunk, g->st));
+                                          (float)g->I_outer, 0, para, (float2 *)g->d_segbuf, g->chunk(), g->st));
         marched = b;
         CK(gather_angle_range(nv, off, g->d_perm + lo, g->d_segbuf, 0, precision == RT_MIXED,
                               g->h_ang_seg_off[w] - lo, g->h_ang_seg_off[w + 1] - lo, g->d_invL + (size_t)w * nv, tI,

@@ -275,11 +275,8 @@ struct SwGather {
     int nlong, first;
 };
 // Blocked voxel order of the FP32 march's S lookups: words with the voxel field
-// replaced by its blocked slot vblk[v] (flags RAYSTART, CORE, RESTART kept),
-// and S, B scattered to their slots.
+// replaced by its blocked slot vblk[v] (flags RAYSTART, CORE, RESTART kept).
 cudaError_t make_voxb(const uint32_t *vox, int64_t nseg, const int32_t *vblk, uint32_t *voxb, cudaStream_t st);
-cudaError_t blk_scatter(int nvox, const int32_t *vblk, const float *S, const float *B, float *Sb, float *Bb,
-                        cudaStream_t st);
 cudaError_t sw_bundles(const int64_t *ray_off, int64_t r_lo, int64_t r_hi, int64_t seg_lo, int64_t nseg, int chunk,
                        int2 *bnd, cudaStream_t st);
 cudaError_t march_sw_launch(const SwMarch &m, int coarsen, cudaStream_t st);
@@ -391,11 +388,16 @@ cudaError_t pack_chiS64(int nvox, const double *chi, const double *S, double2 *c
 cudaError_t pack_chiS32(int nvox, const double *chi, const double *S, const double *B, float2 *cs, float *B32, float *S32,
                         cudaStream_t st);
 cudaError_t ali_update(int nvox, double *S, const double *J, const double *Lst, const double *eps, const double *B,
-                       int use_lstar, double *hist_slot, unsigned long long *maxrel, cudaStream_t st);
+                       int use_lstar, double *hist_slot, unsigned long long *maxrel, unsigned long long *zero,
+                       cudaStream_t st);  // *zero <- 0: the word of the next update's maximum
+// S32[vblk[v]] (S32[v] without vblk) = S[v] in FP32.
+cudaError_t prep_S32(int nvox, const double *S, const int32_t *vblk, float *S32, cudaStream_t st);
 // Order-2 Ng from four iterates (y0 newest), weights 1/wref^2 (wref = y0 when null);
-// writes the extrapolation to out only when the 2x2 system is regular (coef[2] = 1).
+// writes the extrapolation to out only when the 2x2 system is regular (coef[2] = 1)
+// and, with rel given, the double there is not below tol.
 cudaError_t ng_extrapolate(int nvox, const double *y0, const double *y1, const double *y2, const double *y3,
-                           const double *wref, double *partial, double *coef, double *out, cudaStream_t st);
+                           const double *wref, double *partial, double *coef, double *out, cudaStream_t st,
+                           const unsigned long long *rel = nullptr, double tol = 0.0);
 int ng_partial_elems(int nvox);
 cudaError_t residual(int nvox, const double *S, const double *J, const double *Lst, const double *eps,
                      const double *B, int use_lstar, double *r, unsigned long long *maxrel, cudaStream_t st);
