@@ -208,23 +208,6 @@ __global__ void __launch_bounds__(256) k_adjoint(const uint32_t *__restrict__ vo
     (void)w_n;
 }
 
-// Per-voxel sums of per-segment values over one block's ownership lists
-// (first = 1 overwrites the outputs).
-__global__ void k_adj_gather(int nvox, const int32_t *off, const int32_t *perm, const double *a, const double *b,
-                             double *oa, double *ob, int first)
-{
-    int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= nvox) return;
-    double sa = 0.0, sb = 0.0;
-    for (int e = off[v]; e < off[v + 1]; ++e) {
-        const int s = perm[e];
-        sa += a[s];
-        if (b) sb += b[s];
-    }
-    oa[v] = first ? sa : oa[v] + sa;
-    if (ob) ob[v] = first ? sb : ob[v] + sb;
-}
-
 // Flux adjoint from the local basis (r, theta, phi) or (R, phi, z) to Cartesian.
 __global__ void k_flux_T(GeomDev G, const double *gF, double *gc)
 {
@@ -398,7 +381,6 @@ int adjoint_pass(rt_grid *g, bool full, int homog, const double *u, const double
         const int w0 = g->blk_w0[b], nw = g->blk_nw[b];
         const int64_t r_lo = g->h_ang_ray_off[w0], r_hi = g->h_ang_ray_off[w0 + nw];
         const int64_t lo = g->h_ang_seg_off[w0], ns = g->h_ang_seg_off[w0 + nw] - lo;
-        const int32_t *off = g->d_csr_off + (size_t)b * (n + 1);
         const int chunk = 512;
         const int64_t blocks = ((ns + chunk - 1) / chunk + 7) / 8;
         if (ns <= 0) continue;
@@ -410,13 +392,17 @@ int adjoint_pass(rt_grid *g, bool full, int homog, const double *u, const double
                 g->d_invL, g->d_wt, g->d_dirs, g->d_ang_seg_off, w0, nw, n, (const double *)g->d_segbuf, nullptr, tC,
                 tB, chunk);
             ACK(cudaGetLastError());
-            k_adj_gather<<<(n + 255) / 256, 256, 0, g->st>>>(n, off, g->d_perm + lo, tC, tB, oC, oB, b == 0);
+            for (int q = 0; q < 2; ++q) {
+                const int rc = rt_grid_gather64(g, b, q ? tB : tC, q ? oB : oC);
+                if (rc != RT_OK) return rc;
+            }
         } else {
             k_adjoint<false><<<(unsigned)blocks, 256, 0, g->st>>>(
                 g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64, g->d_B, g->I_outer, homog, u, gc,
                 g->d_invL, g->d_wt, g->d_dirs, g->d_ang_seg_off, w0, nw, n, nullptr, tS, nullptr, nullptr, chunk);
             ACK(cudaGetLastError());
-            k_adj_gather<<<(n + 255) / 256, 256, 0, g->st>>>(n, off, g->d_perm + lo, tS, nullptr, oS, nullptr, b == 0);
+            const int rc = rt_grid_gather64(g, b, tS, oS);
+            if (rc != RT_OK) return rc;
         }
         ACK(cudaGetLastError());
     }

@@ -34,14 +34,106 @@ __device__ __forceinline__ double inv_fact(int n)
     return f[n];
 }
 
+// 1 / q to about an ulp: the hardware's 20-bit estimate and one step of the
+// cubically convergent iteration r (1 + e + e^2), e = 1 - q r (three FP64
+// instructions where a correctly rounded division takes about ten).  Outside
+// [2^-900, 2^900], where the estimate would leave the normal range: the division.
+__device__ __forceinline__ double rcp64(double q)
+{
+    const unsigned ex = ((unsigned)__double2hiint(q) >> 20) & 0x7ffu;
+    if (ex - 123u > 1800u) return 1.0 / q;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
+    const double e = fma(-q, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// x < 1 for x >= 0, from the high word: off the FP64 pipe (a NaN is not).
+__device__ __forceinline__ bool below_one(double x) { return (unsigned)__double2hiint(x) < 0x3ff00000u; }
+
+// h1(x) = (e^{-x} - 1 + x) / x^2 and h2(x) = f2(x) / x^2 (see below) on [0, 1]:
+// their values at 0 plus x times polynomials fitted to (h - h(0)) / x at Chebyshev
+// nodes (fit error 1e-18 of h, under FP64 rounding).
+__device__ __forceinline__ double h1_small(double x)
+{
+    double h = 7.722609696190044e-12;
+    h = fma(h, x, -1.514301957269351e-10);
+    h = fma(h, x, 2.0743464091464554e-09);
+    h = fma(h, x, -2.5039626817896517e-08);
+    h = fma(h, x, 2.755654152433202e-07);
+    h = fma(h, x, -2.7557286761537225e-06);
+    h = fma(h, x, 2.480158640720805e-05);
+    h = fma(h, x, -0.00019841269825620665);
+    h = fma(h, x, 0.001388888888872712);
+    h = fma(h, x, -0.00833333333333247);
+    h = fma(h, x, 0.04166666666666665);
+    h = fma(h, x, -0.16666666666666666);
+    return fma(h, x, 0.5);
+}
+__device__ __forceinline__ double h2_small(double x)
+{
+    double h = 6.667117678494612e-12;
+    h = fma(h, x, -1.2965202422838241e-10);
+    h = fma(h, x, 1.754862018413882e-09);
+    h = fma(h, x, -2.086586606418334e-08);
+    h = fma(h, x, 2.2546219039428151e-07);
+    h = fma(h, x, -2.204582705953453e-06);
+    h = fma(h, x, 1.9290122676595323e-05);
+    h = fma(h, x, -0.00014880952367301683);
+    h = fma(h, x, 0.0009920634920493816);
+    h = fma(h, x, -0.005555555555554801);
+    h = fma(h, x, 0.024999999999999984);
+    h = fma(h, x, -0.08333333333333333);
+    return fma(h, x, 1.0 / 6.0);
+}
+
 // Weights of one segment of optical depth x followed by p.
-//   e0 = 1 - e^{-x},  f1 = (x - e0)/x,  f2 = (x(2 - e0) - 2 e0)/x
+//   e0 = 1 - e^{-x},  f1 = (x - e0)/x,  f2 = (x(2 - e0) - 2 e0)/x = 2 f1 - e0
 //   parabolic: alpha = e0 - f1 - f2/(x+p), beta = f1 + f2/p, gamma = -x f2/(p (x+p))
 //   linear:    alpha = e0 - f1,           beta = f1,         gamma = 0
-// f1 and f2 are odd/even power series in x that cancel catastrophically when
-// evaluated from e0 at small x; below the threshold they are summed directly
-// (Horner), above it they come from expm1.
+// f1 and f2 cancel catastrophically when evaluated from e0 at small x; below 1
+// they come from polynomials, above it from the exponential.  The three quotients
+// of the parabola share one reciprocal.  The FP64 pipe bounds every kernel that
+// evaluates these: about 41 instructions of it for a small x and 42 for a large one
+// (62 and 80 with the 19-term series, expm1 and divisions of Coef64Series).  Mean
+// errors against 128-bit arithmetic relative to that form's: equal below 0.5, a
+// third to a tenth in [0.5, 1], equal above but for E, which keeps its relative
+// accuracy.
 struct Coef64 {
+    __device__ __forceinline__ static void eval(double x, double p, bool para, double &E, double &al, double &be,
+                                                double &ga)
+    {
+        double e0, f1, f2;
+        if (below_one(x)) {
+            f1 = x * h1_small(x);
+            f2 = (x * x) * h2_small(x);
+            e0 = fma(-x, f1, x);
+            E = 1.0 - e0;
+        } else {
+            E = exp(-x);
+            e0 = 1.0 - E;
+            const double ix = rcp64(x), num = x - e0;
+            f1 = num * ix;
+            f1 = fma(fma(-f1, x, num), ix, f1);  // to half an ulp
+            f2 = fma(2.0, f1, -e0);
+        }
+        al = e0 - f1;
+        be = f1;
+        ga = 0.0;
+        if (para) {
+            const double D = x + p, t = f2 * rcp64(p * D);
+            al = fma(-t, p, al);
+            be = fma(t, D, be);
+            ga = -(x * t);
+        }
+    }
+};
+
+// The same weights from 19-term series and expm1, each quotient divided: those
+// of the nearest-neighbour operator, whose entries stay the same to the last bit
+// (a line problem at eps_l = 1e-4 and chi_l / chi_c = 1e6 turns a change of their
+// rounding into 1e-5 of its iterates).
+struct Coef64Series {
     static constexpr int NS = 19;  // series terms for x < 0.5
     __device__ __forceinline__ static void eval(double x, double p, bool para, double &E, double &al, double &be,
                                                 double &ga)
@@ -137,41 +229,32 @@ struct Coef32 {
 
 // Derivatives of (E, alpha, beta, gamma) with respect to x = dtau_k and
 // p = dtau_{k+1}, from  e0' = E, f1' = (e0 - f1)/x = g1, f2' = e0 - f1 - f2/x = g2
-// (g1, g2 summed as series below the threshold):
+// (below the threshold g1 = 1 - h1 - x h1 and g2 = x (g1 - h2)):
 //   parabolic: alpha = e0 - f1 - f2/(x+p), beta = f1 + f2/p, gamma = -x f2/(p (x+p))
 //   linear:    alpha = e0 - f1,           beta = f1
 struct Coef64D {
-    static constexpr int NS = 19;
     __device__ __forceinline__ static void eval(double x, double p, bool para, double &E, double &al, double &be,
                                                 double &ga, double &dE, double &dal_x, double &dbe_x, double &dga_x,
                                                 double &dal_p, double &dbe_p, double &dga_p)
     {
         double e0, f1, f2, g1, g2;
-        if (x < 0.5) {
-            double h1 = 0.0, h2 = 0.0, k1 = 0.0, k2 = 0.0;
-#pragma unroll
-            for (int n = NS + 1; n >= 2; --n) h1 = inv_fact(n) - x * h1;
-#pragma unroll
-            for (int m = NS + 1; m >= 3; --m) h2 = (double)(m - 2) * inv_fact(m) - x * h2;
-            // g1 = sum_{n>=2} (-1)^n (n-1) x^(n-2) / n!,  g2 = sum_{m>=3} (-1)^(m+1) (m-2)(m-1) x^(m-2) / m!
-#pragma unroll
-            for (int n = NS + 1; n >= 2; --n) k1 = (double)(n - 1) * inv_fact(n) - x * k1;
-#pragma unroll
-            for (int m = NS + 1; m >= 3; --m) k2 = (double)((m - 2) * (m - 1)) * inv_fact(m) - x * k2;
+        if (below_one(x)) {
+            const double h1 = h1_small(x), h2 = h2_small(x);
             f1 = x * h1;
             f2 = (x * x) * h2;
-            g1 = k1;
-            g2 = x * k2;
-            e0 = x - x * f1;
+            e0 = fma(-x, f1, x);
             E = 1.0 - e0;
+            g1 = (1.0 - h1) - f1;  // (e0 - f1) / x
+            g2 = x * (g1 - h2);
         } else {
-            double em = expm1(-x);
-            e0 = -em;
-            E = 1.0 + em;
-            f1 = (x - e0) / x;
-            f2 = (x * (2.0 - e0) - 2.0 * e0) / x;
-            g1 = (e0 - f1) / x;
-            g2 = e0 - f1 - f2 / x;
+            E = exp(-x);
+            e0 = 1.0 - E;
+            const double ix = rcp64(x), num = x - e0;
+            f1 = num * ix;
+            f1 = fma(fma(-f1, x, num), ix, f1);
+            f2 = fma(2.0, f1, -e0);
+            g1 = (e0 - f1) * ix;
+            g2 = fma(-f2, ix, e0 - f1);
         }
         dE = -E;
         if (para) {

@@ -335,7 +335,8 @@ __global__ void __launch_bounds__(256) k_gather_units32(int nvox, int64_t nunits
     finish_unit(u, v, nunits, urow, r0, r1, r2, r3, r4, part, J, Lst, Fc, first);
 }
 
-// FP64 ray march: FP64 weights and sums.
+// FP64 ray march: FP64 weights and sums.  W: the values carry the weights.
+template <bool W>
 __global__ void __launch_bounds__(256) k_gather_units64(int nvox, int64_t nunits, const int32_t *__restrict__ urow,
                                                         const int32_t *__restrict__ order, const int32_t *__restrict__ ulen,
                                                         const int64_t *__restrict__ gbase, const int32_t *__restrict__ sell,
@@ -368,20 +369,28 @@ __global__ void __launch_bounds__(256) k_gather_units64(int nvox, int64_t nunits
             else hi = mid;
         }
         int q = lo;
-        double f = swt[q] * invL[(int64_t)(w0 + q) * nvox + v];
-        for (int k = 0; k < len; ++k) {
-            s = lst[32 * k];
-            while (s >= soff[q + 1]) {
-                ++q;
-                f = swt[q] * invL[(int64_t)(w0 + q) * nvox + v];
+        double f = W ? 1.0 : swt[q] * invL[(int64_t)(w0 + q) * nvox + v];
+        for (int k = 0; k < len; k += 4) {  // four entries in flight
+            int ss[4];
+            double2 val[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) ss[h] = k + h < len ? lst[32 * (k + h)] : -1;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) val[h] = ss[h] >= 0 ? buf[ss[h]] : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                if (ss[h] < 0) break;
+                while (ss[h] >= soff[q + 1]) {
+                    ++q;
+                    if (!W) f = swt[q] * invL[(int64_t)(w0 + q) * nvox + v];
+                }
+                const double tj = W ? val[h].x : f * val[h].x;
+                aj += tj;
+                al += W ? val[h].y : f * val[h].y;
+                fx += sdir[3 * q] * tj;
+                fy += sdir[3 * q + 1] * tj;
+                fz += sdir[3 * q + 2] * tj;
             }
-            double2 val = buf[s];
-            double tj = f * val.x;
-            aj += tj;
-            al += f * val.y;
-            fx += sdir[3 * q] * tj;
-            fy += sdir[3 * q + 1] * tj;
-            fz += sdir[3 * q + 2] * tj;
         }
     }
     finish_unit(u, v, nunits, urow, aj, al, fx, fy, fz, part, J, Lst, Fc, first);
@@ -885,7 +894,7 @@ cudaError_t gather_block(int nvox, const int32_t *csr_off, const int32_t *perm_b
                          const int32_t *ubeg, const int64_t *ufirst, int64_t nunits, const int32_t *multi,
                          int nmulti, const int32_t *order, const int32_t *ulen, const int64_t *gbase,
                          const int32_t *sell, double *part, double *J, double *Lst, double *Fc, int first,
-                         cudaStream_t st)
+                         cudaStream_t st, int weighted)
 {
     (void)csr_off;
     (void)perm_blk;
@@ -895,9 +904,14 @@ cudaError_t gather_block(int nvox, const int32_t *csr_off, const int32_t *perm_b
     if constexpr (sizeof(P) == sizeof(float2))
         k_gather_units32<<<blocks, 256, 0, st>>>(nvox, nunits, urow, order, ulen, gbase, sell, (const float2 *)buf,
                                                  ang_seg_off, w0, nw, seg_lo, wL32, dirs, part, J, Lst, Fc, first);
+    else if (weighted)
+        k_gather_units64<true><<<blocks, 256, 0, st>>>(nvox, nunits, urow, order, ulen, gbase, sell, (const double2 *)buf,
+                                                       ang_seg_off, w0, nw, seg_lo, invL, wt, dirs, part, J, Lst, Fc,
+                                                       first);
     else
-        k_gather_units64<<<blocks, 256, 0, st>>>(nvox, nunits, urow, order, ulen, gbase, sell, (const double2 *)buf,
-                                                 ang_seg_off, w0, nw, seg_lo, invL, wt, dirs, part, J, Lst, Fc, first);
+        k_gather_units64<false><<<blocks, 256, 0, st>>>(nvox, nunits, urow, order, ulen, gbase, sell, (const double2 *)buf,
+                                                        ang_seg_off, w0, nw, seg_lo, invL, wt, dirs, part, J, Lst, Fc,
+                                                        first);
     if (nmulti > 0) k_gather_rows<<<(nmulti * 8 + 255) / 256, 256, 0, st>>>(nmulti, multi, ufirst, part, J, Lst, Fc, first);
     return cudaGetLastError();
 }
@@ -1033,11 +1047,11 @@ template cudaError_t gather_block<float2>(int, const int32_t *, const int32_t *,
                                           int, int64_t, const double *, const float *, const double *, const double *,
                                           const int32_t *, const int32_t *, const int64_t *, int64_t, const int32_t *,
                                           int, const int32_t *, const int32_t *, const int64_t *, const int32_t *,
-                                          double *, double *, double *, double *, int, cudaStream_t);
+                                          double *, double *, double *, double *, int, cudaStream_t, int);
 template cudaError_t gather_block<double2>(int, const int32_t *, const int32_t *, const double2 *, const int64_t *, int,
                                            int, int64_t, const double *, const float *, const double *, const double *,
                                            const int32_t *, const int32_t *, const int64_t *, int64_t, const int32_t *,
                                            int, const int32_t *, const int32_t *, const int64_t *, const int32_t *,
-                                           double *, double *, double *, double *, int, cudaStream_t);
+                                           double *, double *, double *, double *, int, cudaStream_t, int);
 
 }  // namespace rtk

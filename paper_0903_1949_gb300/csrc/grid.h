@@ -177,6 +177,10 @@ struct NnScratch {
 // on first use after rt_set_opacity; returns an RT_ status.
 int rt_grid_build_nn(rt_grid *g);
 
+// out (+)= the sums over block b's ownership lists of its per-segment values buf
+// (segment order), on the grid's stream; block 0 overwrites.
+int rt_grid_gather64(rt_grid *g, int b, const double *buf, double *out);
+
 // y = Lambda^T u (plus Lambda_F^T gc when gc is not NULL) by the streamed-weight
 // transpose of the FP64 march, on the grid's stream.  *done = false (and
 // nothing written) when the streamed weights are off or do not fit.

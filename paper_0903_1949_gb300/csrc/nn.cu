@@ -58,7 +58,7 @@ __device__ __forceinline__ int slot_of(const Ijk &a, const Ijk &b, int sph, int 
 // Interpolation weights (E, alpha, beta, gamma) of the block's segments for chi.
 // The FP64 pipe bounds the walk, and a warp of consecutive segments mixes small
 // and large optical depths, parabolas and lines, and so pays for every branch of
-// Coef64 on each of them.  Here a block sorts COEF_TILE segments into the four
+// Coef64Series on each of them.  Here a block sorts COEF_TILE segments into the four
 // kinds first; every warp then runs one branch.
 constexpr int COEF_TILE = 1024;
 
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(256) k_nn_coef(NnWalk a, int64_t nseg)
             for (int j = threadIdx.x; j < cnt[k]; j += 256) {
                 const int i = idx[k][j];
                 double E, al, be, ga;
-                Coef64::eval(sx[i], sp[i], (k & 1) != 0, E, al, be, ga);
+                Coef64Series::eval(sx[i], sp[i], (k & 1) != 0, E, al, be, ga);
                 double2 *o = reinterpret_cast<double2 *>(a.cw + t0 + i);
                 o[0] = make_double2(E, al);
                 o[1] = make_double2(be, ga);

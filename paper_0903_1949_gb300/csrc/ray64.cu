@@ -88,24 +88,65 @@ __global__ void __launch_bounds__(128) k_slot_fill(Ray64 m, const uint32_t *__re
     });
 }
 
-// FP64 weights (E, alpha, beta + [run start] alpha, gamma) of every slot for the current chi.
+// FP64 weights (E, alpha, beta + [run start] alpha, gamma) of every slot for the
+// current chi.  A CTA sorts the slots of four groups and eight steps by the branch
+// of the weights they take (small or large optical depth, parabola or line), so
+// that a warp runs one of them; the FP64 pipe is the bound.
+constexpr int COEF_SLOTS = 128 * STEPS_PER_WARP;
+
 __global__ void __launch_bounds__(128) k_slot_coef(Ray64 m, const uint32_t *__restrict__ vox,
                                                    const double *__restrict__ len64, const double *__restrict__ chi,
                                                    Wd4 *__restrict__ cw)
 {
-    each_slot(m, [&](int64_t q, int64_t s, int) {
-        const uint32_t w = vox[s];
-        const bool para = (w & RTK_PARA) != 0u;  // set only when segment s + 1 continues the run
-        const double x = chi[w & RTK_VOXMASK] * len64[s];
-        const double p = para ? chi[vox[s + 1] & RTK_VOXMASK] * len64[s + 1] : 0.0;
-        double E, al, be, ga;
-        Coef64::eval(x, p, para, E, al, be, ga);
-        if (w & (RTK_RAYSTART | RTK_RESTART)) {  // S_0 := S_1 at the start of a run
-            be += al;
-            al = 0.0;
+    __shared__ double sx[COEF_SLOTS], sp[COEF_SLOTS];
+    __shared__ uint16_t idx[4][COEF_SLOTS];  // slot of the CTA, bit 15: first of a run
+    __shared__ int64_t base[4];
+    __shared__ int cnt[4], wmax;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const bool on = g < m.ngroups;
+    const int64_t p = m.r_lo + 32 * g + lane;
+    const bool have = on && p < m.r_hi;
+    const int n = have ? m.olen[p] : 0;
+    const int64_t s0 = have ? m.ray_off[m.order[p]] : 0;
+    if (threadIdx.x == 0) wmax = 0;
+    __syncthreads();
+    if (lane == 0) {
+        base[wid] = on ? m.gbase[g] : 0;
+        atomicMax(&wmax, n);
+    }
+    __syncthreads();
+    const int width = wmax;
+    for (int k0 = blockIdx.y * STEPS_PER_WARP; k0 < width; k0 += gridDim.y * STEPS_PER_WARP) {
+        if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
+        __syncthreads();
+        for (int k = k0; k < k0 + STEPS_PER_WARP && k < n; ++k) {
+            const int64_t s = s0 + k;
+            const uint32_t w = vox[s];
+            const bool para = (w & RTK_PARA) != 0u;  // set only when segment s + 1 continues the run
+            const double x = chi[w & RTK_VOXMASK] * len64[s];
+            const int i = (k - k0) * 128 + (int)threadIdx.x;
+            sx[i] = x;
+            sp[i] = para ? chi[vox[s + 1] & RTK_VOXMASK] * len64[s + 1] : 0.0;
+            const int c = (below_one(x) ? 0 : 2) + (para ? 1 : 0);
+            idx[c][atomicAdd(cnt + c, 1)] =
+                (uint16_t)(i | ((w & (RTK_RAYSTART | RTK_RESTART)) ? 0x8000 : 0));
         }
-        cw[q] = Wd4{E, al, be, ga};
-    });
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            for (int j = threadIdx.x; j < cnt[c]; j += 128) {
+                const int q = idx[c][j], i = q & 0x7fff, t = i & 127;
+                double E, al, be, ga;
+                Coef64::eval(sx[i], sp[i], (c & 1) != 0, E, al, be, ga);
+                if (q & 0x8000) {  // S_0 := S_1 at the start of a run
+                    be += al;
+                    al = 0.0;
+                }
+                cw[base[t >> 5] + 32 * (int64_t)(k0 + (i >> 7)) + (t & 31)] = Wd4{E, al, be, ga};
+            }
+        __syncthreads();
+    }
 }
 
 __device__ __forceinline__ Wd4 ldw64(const Wd4 *p)
@@ -149,6 +190,52 @@ __global__ void __launch_bounds__(128) k_march_ray64(Ray64 m, const double *__re
         Sk = Sn;
         Sn = S2;
         w0 = w1;
+        w1 = w2;
+        w2 = w3;
+        c0 = c1;
+        c1 = c2;
+        g0 = g1;
+        g1 = g2;
+    }
+}
+
+// The same march for the full formal solution: per segment of the block, in
+// segment order, c_k I_k and c_k lambda_k with the local Lambda* element lambda_k =
+// dI_k/dS_k = beta_k + gamma_{k-1} E_k (alpha_k is in beta_k at a run start, where
+// the gamma before it is 0).
+__global__ void __launch_bounds__(128) k_march_ray64_full(Ray64 m, const double *__restrict__ S,
+                                                          const double *__restrict__ B, double I_outer, int homog,
+                                                          double2 *__restrict__ out)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (g >= m.ngroups) return;
+    const int64_t p = m.r_lo + 32 * g + lane;
+    const int n = p < m.r_hi ? m.olen[p] : 0;
+    if (n <= 0) return;
+    const int64_t base = m.gbase[g] + lane;
+    const uint2 *wp = m.wp + base;
+    const Wd4 *cw = m.cw + base;
+    const double *cg = m.cg + base;
+    double2 *o2 = out + (m.ray_off[m.order[p]] - m.seg_lo);
+    const Wd4 zero{0.0, 0.0, 0.0, 0.0};
+    uint32_t w0 = __ldcs(wp).x, w1 = n > 1 ? __ldcs(wp + 32).x : 0u, w2 = n > 2 ? __ldcs(wp + 64).x : 0u;
+    Wd4 c0 = ldw64(cw), c1 = n > 1 ? ldw64(cw + 32) : zero;
+    double g0 = __ldcs(cg), g1 = n > 1 ? __ldcs(cg + 32) : 0.0;
+    double Sk = S[w0 & RTK_VOXMASK], Sn = n > 1 ? S[w1 & RTK_VOXMASK] : 0.0, Sm = 0.0, gm = 0.0;
+    double I = homog ? 0.0 : ((w0 & RTK_CORE) ? B[w0 & RTK_VOXMASK] : I_outer);
+    for (int k = 0; k < n; ++k) {
+        const int64_t o = 32 * (int64_t)k;
+        const uint32_t w3 = k + 3 < n ? __ldcs(wp + o + 96).x : 0u;
+        const Wd4 c2 = k + 2 < n ? ldw64(cw + o + 64) : zero;
+        const double g2 = k + 2 < n ? __ldcs(cg + o + 64) : 0.0;
+        const double S2 = k + 2 < n ? S[w2 & RTK_VOXMASK] : 0.0;
+        I = fma(c0.x, I, fma(c0.y, Sm, fma(c0.z, Sk, c0.w * Sn)));
+        __stcg(o2 + k, make_double2(g0 * I, g0 * fma(gm, c0.x, c0.z)));
+        gm = c0.w;
+        Sm = Sk;
+        Sk = Sn;
+        Sn = S2;
         w1 = w2;
         w2 = w3;
         c0 = c1;
@@ -282,6 +369,14 @@ cudaError_t ray64_march(const Ray64 &m, const double *S, const double *B, double
 {
     if (m.ngroups <= 0) return cudaSuccess;
     k_march_ray64<<<rblocks(32 * m.ngroups, 128), 128, 0, st>>>(m, S, B, I_outer, homog, out);
+    return cudaGetLastError();
+}
+
+cudaError_t ray64_full(const Ray64 &m, const double *S, const double *B, double I_outer, int homog, double2 *out,
+                       cudaStream_t st)
+{
+    if (m.ngroups <= 0) return cudaSuccess;
+    k_march_ray64_full<<<rblocks(32 * m.ngroups, 128), 128, 0, st>>>(m, S, B, I_outer, homog, out);
     return cudaGetLastError();
 }
 

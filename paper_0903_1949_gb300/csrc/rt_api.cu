@@ -724,14 +724,23 @@ int alloc_fields(rt_grid *g)
     return RT_OK;
 }
 
+bool use_sw64(rt_grid *g);
+bool sw64_roomy(const rt_grid *g);
+Ray64 ray64_block(rt_grid *g, int b);
+
 // Formal solution of every angle block with the FP64 or FP32 march.
 int run_fs(rt_grid *g, int prec, int homog, const double *S_src, double *J, double *L, double *Fc, double *F)
 {
     const int n = g->nvox;
     const int para = g->interp == RT_PARABOLIC;
-    if (prec == RT_FP64) CK(pack_chiS64(n, g->d_chi, S_src, g->d_cs64, g->st));
-    else CK(pack_chiS32(n, g->d_chi, S_src, g->d_B, g->d_cs32, g->d_B32, g->d_S32, g->st));
-    g->launches++;
+    // FP64: on the streamed weights, which the iterations that follow need anyway
+    const bool ray = prec == RT_FP64 && sw64_roomy(g) && use_sw64(g);
+    CK(cudaGetLastError());
+    if (!ray) {
+        if (prec == RT_FP64) CK(pack_chiS64(n, g->d_chi, S_src, g->d_cs64, g->st));
+        else CK(pack_chiS32(n, g->d_chi, S_src, g->d_B, g->d_cs32, g->d_B32, g->d_S32, g->st));
+        g->launches++;
+    }
     for (int b = 0; b < g->nblk; ++b) {
         int w0 = g->blk_w0[b], nw = g->blk_nw[b];
         int64_t r_lo = g->h_ang_ray_off[w0], r_hi = g->h_ang_ray_off[w0 + nw];
@@ -741,16 +750,19 @@ int run_fs(rt_grid *g, int prec, int homog, const double *S_src, double *J, doub
         if (prec == RT_FP64) {
             double2 *buf = (double2 *)g->d_segbuf;
             t0 = tstart(g, 0);
-            CK(march_block<double, double2>(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64, g->d_B,
-                                            g->I_outer, homog, para, buf, g->chunk(), g->st));
-            tstop(g, t0, 0, ns, 12 * ns);
+            if (ray)
+                CK(ray64_full(ray64_block(g, b), S_src, g->d_B, g->I_outer, homog, buf, g->st));
+            else
+                CK(march_block<double, double2>(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64,
+                                                g->d_B, g->I_outer, homog, para, buf, g->chunk(), g->st));
+            tstop(g, t0, 0, ns, (ray ? 44 : 12) * ns);
             t1 = tstart(g, 1);
             CK(gather_block<double2>(n, off, g->d_perm + lo, buf, g->d_ang_seg_off, w0, nw, lo, g->d_invL, g->d_wL32,
                                      g->d_wt, g->d_dirs, g->d_urow + g->h_ubase[b], g->d_ubeg + g->h_ubase[b],
                                      g->d_ufirst + (size_t)b * (n + 1), g->h_nunits[b], g->d_multi + g->h_mbase[b],
                                      (int)(g->h_mbase[b + 1] - g->h_mbase[b]), g->d_order + g->h_ubase[b],
                                      g->d_ulen + g->h_ubase[b], g->d_gbase + g->h_goff[b], g->d_sell + g->h_soff[b],
-                                     g->d_part, J, L, Fc, b == 0, g->st));
+                                     g->d_part, J, L, Fc, b == 0, g->st, ray));
             tstop(g, t1, 1, ns);
         } else {
             float2 *buf = (float2 *)g->d_segbuf;
@@ -984,6 +996,19 @@ bool ray64_setup(rt_grid *g)
     g->d_cw64 = (Wd4 *)keep_alloc(g, sizeof(Wd4) * (size_t)slots);
     g->d_cg64 = (double *)keep_alloc(g, sizeof(double) * (size_t)slots);
     return g->d_wp64 && g->d_cw64 && g->d_cg64;
+}
+
+// Whether a single FP64 formal solution may set up the streamed weights: they are
+// there already, or leave as much again and the FP32 streams' room free.
+bool sw64_roomy(const rt_grid *g)
+{
+    if (g->sw64_state != 0) return g->sw64_state > 0;
+    size_t room = 0, total = 0;
+    if (cudaMemGetInfo(&room, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (double)room > 2.0 * 50.0 * (double)g->n_seg + 24.0 * (double)g->n_seg + 4e9;
 }
 
 // FP64 streamed weights (48 bytes per slot), the same life cycle.
@@ -1626,6 +1651,15 @@ int rt_grid_member_fs(rt_grid *g, const float2 *cs, const float *B32, const uint
 }
 
 int rt_grid_build_nn(rt_grid *g) { return build_nn(g); }
+
+int rt_grid_gather64(rt_grid *g, int b, const double *buf, double *out)
+{
+    SwGather t = sw_gather(g, b, nullptr, out);
+    t.buf64 = buf;
+    CK(gather_sw_launch(t, g->st));
+    g->launches++;
+    return RT_OK;
+}
 
 int rt_grid_adjoint_ray64(rt_grid *g, const double *u, const double *gc, double *y, bool *done)
 {

@@ -105,6 +105,7 @@ cudaError_t gather_units_fill(int nvox, const int32_t *csr_off, const int64_t *u
 // FP32 gather weights wt_w / L_wv per (solid angle, voxel).
 cudaError_t make_wL32(int n_ang, int nvox, const double *invL, const double *wt, float *wL, cudaStream_t st);
 // J, Lambda*, flux (Cartesian) of one block from the per-segment (l I, l lambda); first = 1 overwrites.
+// weighted = 1 (FP64): the values carry the gather weight w l / L already.
 template <typename P>
 cudaError_t gather_block(int nvox, const int32_t *csr_off, const int32_t *perm_blk, const P *buf,
                          const int64_t *ang_seg_off, int w0, int nw, int64_t seg_lo, const double *invL,
@@ -112,7 +113,7 @@ cudaError_t gather_block(int nvox, const int32_t *csr_off, const int32_t *perm_b
                          const int32_t *ubeg, const int64_t *ufirst, int64_t nunits, const int32_t *multi,
                          int nmulti, const int32_t *order, const int32_t *ulen, const int64_t *gbase,
                          const int32_t *sell, double *part, double *J, double *Lst, double *Fc, int first,
-                         cudaStream_t st);
+                         cudaStream_t st, int weighted = 0);
 // Sliced-ELL layout of one block's work units: unit lengths, order (longest
 // first), per-group width 32*max length (gw, to be scanned into gbase), fill.
 cudaError_t sell_order(int64_t nunits, const int32_t *urow, const int32_t *ubeg, const int32_t *csr_off, int32_t *ulen,
@@ -259,6 +260,9 @@ cudaError_t ray64_fill(const Ray64 &m, const uint32_t *vox, const double *len64,
 cudaError_t ray64_coef(const Ray64 &m, const uint32_t *vox, const double *len64, const double *chi, cudaStream_t st);
 cudaError_t ray64_march(const Ray64 &m, const double *S, const double *B, double I_outer, int homog, double *out,
                         cudaStream_t st);
+// (c I, c lambda) of the block's segments, in segment order (full formal solution).
+cudaError_t ray64_full(const Ray64 &m, const double *S, const double *B, double I_outer, int homog, double2 *out,
+                       cudaStream_t st);
 // out = the block's per-segment shares of Lambda^T u (plus Lambda_F^T gc, the
 // Cartesian flux adjoint, when gc is not NULL).
 cudaError_t ray64_adjoint(const Ray64 &m, const double *u, const double *gc, const double *dirs,
