@@ -826,6 +826,27 @@ int grid_for(int64_t n, int threads)
 
 int64_t radix_tiles(int64_t n) { return (n + RS_TILE - 1) / RS_TILE; }
 
+cudaError_t radix_order(const uint32_t *key, int64_t n, int bits, int32_t *perm, const RadixScratch &rs, cudaStream_t st)
+{
+    cudaError_t e = cudaSuccess;
+    if (n > rs.cap) return cudaErrorInvalidValue;
+    if (n <= 0) return cudaSuccess;
+    const int passes = (bits + 7) / 8;
+    k_rs_init<<<grid_for(n, 256), 256, 0, st>>>(key, n, rs.kA, passes ? rs.vA : perm);
+    const int64_t ntiles = radix_tiles(n);
+    uint32_t *kin = rs.kA, *kout = rs.kB;
+    int32_t *vin = rs.vA, *vout = rs.vB;
+    for (int p = 0; p < passes; ++p) {
+        if (p == passes - 1) vout = perm;
+        k_rs_hist<<<(unsigned)ntiles, 256, 0, st>>>(kin, n, 8 * p, ntiles, rs.hist);
+        if ((e = scan_i32(rs.hist, rs.off, RS_BUCKETS * ntiles, rs.tmp, st)) != cudaSuccess) return e;
+        k_rs_scatter<<<(unsigned)ntiles, 256, 0, st>>>(kin, vin, n, 8 * p, ntiles, rs.off, kout, vout);
+        std::swap(kin, kout);
+        std::swap(vin, vout);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t csr_build(int nvox, const uint32_t *vox_blk, int64_t nseg_blk, int32_t *counts, int32_t *csr_off,
                       int32_t *perm_blk, int64_t *tmp, const RadixScratch &rs, cudaStream_t st)
 {
@@ -841,20 +862,7 @@ cudaError_t csr_build(int nvox, const uint32_t *vox_blk, int64_t nseg_blk, int32
     if (nseg_blk <= 0) return cudaGetLastError();
     int bits = 0;
     while (bits < 31 && ((int64_t)1 << bits) < (int64_t)nvox) ++bits;
-    const int passes = (bits + 7) / 8;
-    k_rs_init<<<grid_for(nseg_blk, 256), 256, 0, st>>>(vox_blk, nseg_blk, rs.kA, passes ? rs.vA : perm_blk);
-    const int64_t ntiles = radix_tiles(nseg_blk);
-    uint32_t *kin = rs.kA, *kout = rs.kB;
-    int32_t *vin = rs.vA, *vout = rs.vB;
-    for (int p = 0; p < passes; ++p) {
-        if (p == passes - 1) vout = perm_blk;
-        k_rs_hist<<<(unsigned)ntiles, 256, 0, st>>>(kin, nseg_blk, 8 * p, ntiles, rs.hist);
-        if ((e = scan_i32(rs.hist, rs.off, RS_BUCKETS * ntiles, rs.tmp, st)) != cudaSuccess) return e;
-        k_rs_scatter<<<(unsigned)ntiles, 256, 0, st>>>(kin, vin, nseg_blk, 8 * p, ntiles, rs.off, kout, vout);
-        std::swap(kin, kout);
-        std::swap(vin, vout);
-    }
-    return cudaGetLastError();
+    return radix_order(vox_blk, nseg_blk, bits, perm_blk, rs, st);
 }
 
 cudaError_t csr_invL(int nvox, const int32_t *csr_off, const int32_t *perm_blk, const double *len64_blk,

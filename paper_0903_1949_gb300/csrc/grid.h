@@ -103,6 +103,16 @@ struct rt_grid {
     int sw64_state = 0;
     int wp64_pos = -1;           // output positions in d_wp64: 1 list order, 0 segment order, -1 not filled
     bool cw64_ok = false;
+    // bundled march of the mixed J-only formal solution (bundle32.cu)
+    struct Bundles {
+        int state = 0;           // 0 not set up yet, 1 there, -1 does not fit
+        bool on = false;         // taken by the current formal solution
+        bool cw_ok = false;      // weights match the current chi
+        std::vector<rtk::Bun32> part;
+        std::vector<rtk::SwGather> ga;
+        std::vector<int64_t> segs, bytes;  // per part: segments, streamed DRAM bytes of a march
+        float *buf[3] = {};      // one value per unit of a part
+    } bun;
     int pos_state = 0;        // list positions: 0 not tried, 1 allocated, -1 not available
     bool cw_ok = false;       // d_cw4 matches the current chi
     bool b32_ok = false, b32b_ok = false;  // d_B32 and d_B32b match the current B

@@ -849,11 +849,271 @@ bool sw_common(rt_grid *g)
     return true;
 }
 
+// Bundles of the mixed J-only formal solution (once per grid): parts of at most
+// BUN_PART segments (whole angle blocks), each one launch of the march and of the
+// gather: small enough that three parts' values (a quarter to a half of the segments,
+// 4 bytes) stay in L2 beside the streams, since a value alone in its sector that
+// leaves L2 costs 32 bytes of HBM each way (four iterations on 65 x 33 x 65 voxels x
+// 32 x 32 solid angles with parts of 22, 11, 5.5 and 3 million: 18.1, 17.2, 17.2,
+// 17.4 ms; on 65^3 cylindrical ones x 16 x 16: 7.2, 6.3, 6.1, 6.2), and not smaller,
+// for every part adds to the set-up.
+// false, with nothing kept, when the arrays do not fit or a characteristic is so
+// long that a bundle could not hold a few of them.
+constexpr int64_t BUN_PART = 7000000;
+bool bun_setup(rt_grid *g)
+{
+    struct Bufs {
+        std::vector<void *> v;
+        ~Bufs()
+        {
+            for (void *q : v) cudaFree(q);
+        }
+        void *get(int64_t bytes)
+        {
+            void *q = nullptr;
+            if (cudaMalloc(&q, (size_t)std::max<int64_t>(1, bytes)) != cudaSuccess) {
+                cudaGetLastError();
+                return nullptr;
+            }
+            v.push_back(q);
+            return q;
+        }
+    } tmp, keep;
+    int64_t kept = 0;
+    auto kget = [&](int64_t bytes) {
+        kept += bytes;
+        return keep.get(bytes);
+    };
+    // the parts' tables come out of larger pieces: an allocation costs more than a table
+    char *piece = nullptr;
+    int64_t left = 0;
+    auto pget = [&](int64_t bytes) -> void * {
+        bytes = (std::max<int64_t>(1, bytes) + 255) / 256 * 256;
+        if (bytes > left) {
+            left = std::max(bytes, std::min<int64_t>((int64_t)256 << 20, g->n_seg));
+            piece = (char *)kget(left);
+            if (!piece) {
+                left = 0;
+                return nullptr;
+            }
+        }
+        piece += bytes;
+        left -= bytes;
+        return piece - bytes;
+    };
+    auto ok = [](cudaError_t e) {
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess;
+    };
+    rt_grid::Bundles &u = g->bun;
+    const int nvox = g->nvox;
+    int32_t *stat = (int32_t *)tmp.get(16), hs[3] = {};  // longest characteristic, most units of a bundle, error
+    if (!stat || !ok(cudaMemsetAsync(stat, 0, 16, g->st)) || !ok(bun_maxlen(g->n_rays, g->d_ray_off, stat, g->st)) ||
+        !ok(cudaMemcpyAsync(hs, stat, 4, cudaMemcpyDeviceToHost, g->st)) || !ok(cudaStreamSynchronize(g->st)))
+        return false;
+    if (hs[0] > BUN_CAP - 256 * BUN_WARPS) return false;
+    // on a small grid smaller bundles, until there are four an SM
+    const int sub = (int)std::min<int64_t>((BUN_CAP - hs[0]) / BUN_WARPS,
+                                           std::max<int64_t>(64, g->n_seg / (152 * 4 * BUN_WARPS)));
+    struct Part {
+        int b0, b1, a0, na;
+        int64_t ns;
+    };
+    std::vector<Part> parts;
+    auto seg_lo = [&](int b) { return b < g->nblk ? g->h_ang_seg_off[g->blk_w0[b]] : g->h_ang_seg_off[g->n_ang]; };
+    int64_t ns_max = 1, nr_max = 1, nsub_all = 0, slots = 0;
+    for (int b = 0; b < g->nblk;) {
+        int e = b + 1;
+        while (e < g->nblk && seg_lo(e + 1) - seg_lo(b) <= BUN_PART) ++e;
+        const int a0 = g->blk_w0[b], a1 = g->blk_w0[e - 1] + g->blk_nw[e - 1];
+        parts.push_back({b, e, a0, a1 - a0, seg_lo(e) - seg_lo(b)});
+        ns_max = std::max(ns_max, parts.back().ns);
+        nr_max = std::max(nr_max, g->h_ang_ray_off[a1] - g->h_ang_ray_off[a0]);
+        b = e;
+    }
+    constexpr int TILE = 32 * BUN_K;
+    std::vector<int64_t> nbun, sub0;
+    for (const Part &p : parts) {
+        nbun.push_back((p.ns + (int64_t)sub * BUN_WARPS - 1) / ((int64_t)sub * BUN_WARPS));
+        sub0.push_back(nsub_all);
+        nsub_all += nbun.back() * BUN_WARPS + 1;
+        slots += p.ns / TILE * TILE + nbun.back() * BUN_WARPS * TILE + TILE;
+    }
+    RadixScratch rs{};
+    rs.cap = std::max(ns_max, nr_max);
+    const int64_t nhist = 256 * radix_tiles(rs.cap);
+    int64_t nbun_max = 1;
+    for (int64_t q : nbun) nbun_max = std::max(nbun_max, q);
+    rs.kA = (uint32_t *)tmp.get(4 * rs.cap);
+    rs.kB = (uint32_t *)tmp.get(4 * rs.cap);
+    rs.vA = (int32_t *)tmp.get(4 * rs.cap);
+    rs.vB = (int32_t *)tmp.get(4 * rs.cap);
+    rs.hist = (int32_t *)tmp.get(4 * nhist);
+    rs.off = (int64_t *)tmp.get(8 * (nhist + 1));
+    rs.tmp = (int64_t *)tmp.get(8 * scan_tmp_elems(nhist));
+    uint32_t *key = (uint32_t *)tmp.get(4 * nr_max), *tv = (uint32_t *)tmp.get(4 * ns_max);
+    uint32_t *tb = (uint32_t *)tmp.get(4 * ns_max), *td = (uint32_t *)tmp.get(4 * ns_max);
+    uint32_t *uvox = (uint32_t *)tmp.get(4 * ns_max);
+    int32_t *perm = (int32_t *)tmp.get(4 * ns_max), *rlen = (int32_t *)tmp.get(4 * g->n_rays);
+    int32_t *cnt = (int32_t *)tmp.get(4 * nvox), *hist = (int32_t *)tmp.get(4 * 128), *lflag = (int32_t *)tmp.get(4 * nvox);
+    int32_t *nch = (int32_t *)tmp.get(4 * nvox), *lrows = (int32_t *)tmp.get(4 * nvox);
+    int32_t *nunit = (int32_t *)tmp.get(4 * nbun_max), *ndist = (int32_t *)tmp.get(4 * nbun_max);
+    int64_t *doff = (int64_t *)tmp.get(8 * (nbun_max + 1));
+    const int64_t nscan = std::max<int64_t>(std::max<int64_t>(nvox + 1, nbun_max + 1), g->n_rays);
+    int64_t *pos1 = (int64_t *)tmp.get(8 * (nvox + 1)), *pos2 = (int64_t *)tmp.get(8 * (nvox + 1));
+    int64_t *uoff = (int64_t *)tmp.get(8 * (nbun_max + 1)), *stmp = (int64_t *)tmp.get(8 * scan_tmp_elems(nscan));
+    int64_t *ctmp = (int64_t *)tmp.get(8 * ((int64_t)nvox + 1 + scan_tmp_elems(nvox)));
+    int64_t *boff = (int64_t *)kget(8 * (g->n_rays + 1));
+    int32_t *order = (int32_t *)kget(4 * g->n_rays);
+    int32_t *sray = (int32_t *)kget(4 * nsub_all), *sseg = (int32_t *)kget(4 * nsub_all);
+    float4 *cw = (float4 *)kget(16 * slots);
+    uint32_t *wd = (uint32_t *)kget(4 * slots);
+    int32_t *off = (int32_t *)kget(4 * (int64_t)parts.size() * (nvox + 1));
+    int2 *ub_all = (int2 *)kget(8 * nsub_all);  // more than a bundle needs
+    for (void *q : {(void *)rs.kA, (void *)rs.kB, (void *)rs.vA, (void *)rs.vB, (void *)rs.hist, (void *)rs.off,
+                    (void *)rs.tmp, (void *)key, (void *)tv, (void *)tb, (void *)td, (void *)uvox, (void *)ndist, (void *)doff, (void *)perm, (void *)rlen, (void *)cnt,
+                    (void *)hist, (void *)lflag, (void *)nch, (void *)lrows, (void *)nunit, (void *)pos1, (void *)pos2,
+                    (void *)uoff, (void *)stmp, (void *)ctmp, (void *)boff, (void *)order, (void *)sray, (void *)sseg,
+                    (void *)cw, (void *)wd, (void *)off, (void *)ub_all})
+        if (!q) return false;
+    for (const Part &p : parts) {  // sorted order of the characteristics
+        const int64_t r0 = g->h_ang_ray_off[p.a0], n = g->h_ang_ray_off[p.a0 + p.na] - r0;
+        int bits = 0;
+        if (!ok(bun_keys(g->d_ray_off, r0, n, g->d_vox, g->d_ray_angle, p.a0, p.na, g->G.n1, g->G.n2, g->G.n3, key, &bits,
+                         g->st)) ||
+            !ok(radix_order(key, n, bits, order + r0, rs, g->st)) ||
+            !ok(ray64_order(r0, n, g->d_ray_off, order, rlen, g->st)))
+            return false;
+    }
+    if (!ok(scan_i32(rlen, boff, g->n_rays, stmp, g->st))) return false;
+    std::vector<Bun32> bp;
+    std::vector<SwGather> bg;
+    std::vector<int64_t> segs, bytes;
+    int64_t slot = 0, ub0 = 0, max_units = 1, max_chunks = 1;
+    for (size_t i = 0; i < parts.size(); ++i) {
+        const Part &p = parts[i];
+        Bun32 m{};
+        m.r_lo = g->h_ang_ray_off[p.a0];
+        m.r_hi = g->h_ang_ray_off[p.a0 + p.na];
+        m.seg_lo = seg_lo(p.b0);
+        m.slot_lo = slot;
+        slot += p.ns / TILE * TILE + nbun[i] * BUN_WARPS * TILE + TILE;
+        m.nbun = (int)nbun[i];
+        m.sub = sub;
+        m.ray_off = g->d_ray_off;
+        m.order = order;
+        m.boff = boff;
+        m.sray = sray + sub0[i];
+        m.sseg = sseg + sub0[i];
+        m.cw = cw;
+        m.wd = wd;
+        int2 *ub = ub_all + ub0;
+        ub0 += nbun[i] + 1;
+        m.ub = ub;
+        int64_t nu = 0, nd = 0;
+        if (m.nbun > 0) {
+            if (!ok(bun_bounds(m, p.ns, sray + sub0[i], sseg + sub0[i], g->st)) ||
+                !ok(bun_units(m, nvox, g->d_vox, tv, tb, td, nunit, ndist, stat + 2, g->st)) ||
+                !ok(scan_i32(nunit, uoff, m.nbun, stmp, g->st)) || !ok(scan_i32(ndist, doff, m.nbun, stmp, g->st)) ||
+                !ok(bun_ub(m.nbun, uoff, doff, ub, stat + 1, g->st)) ||
+                !ok(cudaMemcpyAsync(&nd, doff + m.nbun, 8, cudaMemcpyDeviceToHost, g->st)) ||
+                !ok(cudaMemcpyAsync(&nu, uoff + m.nbun, 8, cudaMemcpyDeviceToHost, g->st)) ||
+                !ok(cudaStreamSynchronize(g->st)))
+                return false;
+        }
+        int32_t *slab = (int32_t *)pget(4 * (nd + 2 * nu) + 16);  // 16 bytes to spare: prefetched in 16-byte pieces
+        m.upos = slab;
+        m.ubeg = (uint32_t *)slab + nu;
+        m.dvox = (uint32_t *)slab + 2 * nu;
+        int32_t *po = off + (int64_t)i * (nvox + 1);
+        if (!slab) return false;
+        if (m.nbun > 0 && !ok(bun_compact(m, tv, tb, td, uvox, g->st))) return false;
+        int64_t tots[2] = {0, 0};
+        if (!ok(csr_build(nvox, uvox, nu, cnt, po, perm, ctmp, rs, g->st)) ||
+            !ok(inv_perm(perm, nu, m.upos, g->st)) || !ok(gatherJ_classify(nvox, po, hist, lflag, nch, g->st)) ||
+            !ok(scan_i32(lflag, pos1, nvox, stmp, g->st)) || !ok(scan_i32(nch, pos2, nvox, stmp, g->st)) ||
+            !ok(cudaMemcpyAsync(&tots[0], pos1 + nvox, 8, cudaMemcpyDeviceToHost, g->st)) ||
+            !ok(cudaMemcpyAsync(&tots[1], pos2 + nvox, 8, cudaMemcpyDeviceToHost, g->st)) ||
+            !ok(cudaStreamSynchronize(g->st)))
+            return false;
+        int32_t *tab = (int32_t *)pget(4 * (2 * tots[0] + 3 * tots[1]));
+        int32_t *lcnt = tab, *lfirst = tab + tots[0], *crow = lfirst + tots[0], *cbeg = crow + tots[1];
+        int32_t *clr = cbeg + tots[1];
+        if (!tab || (tots[0] > 0 &&
+                     (!ok(cudaMemsetAsync(lcnt, 0, 4 * (size_t)tots[0], g->st)) ||
+                      !ok(gatherJ_long(nvox, po, lflag, pos1, pos2, lrows, lfirst, crow, cbeg, clr, g->st)))))
+            return false;
+        SwGather t{};
+        t.off = po;
+        t.crow = crow;
+        t.cbeg = cbeg;
+        t.clr = clr;
+        t.lfirst = lfirst;
+        t.cnt = lcnt;
+        t.nchunks = tots[1];
+        t.nlong = (int)tots[0];
+        t.first = i == 0;
+        bp.push_back(m);
+        bg.push_back(t);
+        segs.push_back(p.ns);
+        bytes.push_back(20 * p.ns + 8 * nu + 4 * nd);
+        max_units = std::max(max_units, nu);
+        max_chunks = std::max(max_chunks, tots[1]);
+        g->launches += 30;
+    }
+    double *part = (double *)kget(8 * max_chunks);
+    float *buf[3];
+    const int nbuf = (int)std::min<size_t>(3, bp.size());
+    for (int q = 0; q < 3; ++q) buf[q] = q < nbuf ? (float *)kget(4 * max_units) : buf[0];
+    if (!part || !buf[0] || !buf[1] || !buf[2] || !ok(cudaMemcpyAsync(hs, stat, 12, cudaMemcpyDeviceToHost, g->st)) ||
+        !ok(cudaStreamSynchronize(g->st)) || hs[2] != 0)
+        return false;
+    for (Bun32 &m : bp) m.dmax = hs[1];
+    for (SwGather &t : bg) t.part = part;
+    g->allocs.insert(g->allocs.end(), keep.v.begin(), keep.v.end());
+    keep.v.clear();
+    g->bytes += kept;
+    u.part = std::move(bp);
+    u.ga = std::move(bg);
+    u.segs = std::move(segs);
+    u.bytes = std::move(bytes);
+    for (int q = 0; q < 3; ++q) u.buf[q] = buf[q];
+    return true;
+}
+
+// Whether the mixed J-only formal solution runs in bundles: with the default
+// march (weights with the gather weight folded in, one segment per lane and chunk
+// not chosen); any other setting keeps the march of fs_sw.cu.
+bool use_bun(rt_grid *g)
+{
+    rt_grid::Bundles &u = g->bun;
+    u.on = false;
+    if (!g->sw_enabled || !g->sw_fold || g->sw_stages != 0 || g->sw_coarsen != 1 || g->march_chunk != 512 || u.state < 0)
+        return false;
+    if (u.state == 0) {
+        u.state = bun_setup(g) ? 1 : -1;
+        u.cw_ok = false;
+        if (u.state < 0) return false;
+    }
+    if (!u.cw_ok) {
+        for (const Bun32 &m : u.part) {
+            if (m.nbun > 0 && bun_coef(m, g->d_vox, g->d_len64, g->d_chi, g->d_ray_angle, g->d_wt, g->d_invL, g->nvox,
+                                       g->st) != cudaSuccess)
+                return false;
+            g->launches++;
+        }
+        u.cw_ok = true;
+    }
+    u.on = true;
+    return true;
+}
+
 // FP32 streamed weights: allocated on first use (w l / L computed then, from the
 // geometry), (E, alpha, beta, gamma) refreshed after chi changed.  false when
 // disabled or out of memory (the FP32 march then evaluates the weights itself).
 bool use_sw(rt_grid *g)
 {
+    if (use_bun(g)) return true;
     if (!g->sw_enabled || g->sw_state < 0) return false;
     const int fold = g->sw_fold && g->sw_stages == 0;
     if (g->sw_state == 0) {
@@ -1185,19 +1445,35 @@ int run_fs_J_sw(rt_grid *g, int prec, int homog, const double *S_src, double *J)
     const bool scatter = g->sw_scatter && g->d_pos;
     // double (FP64) or up to triple (FP32) buffer of per-segment values: the
     // segment buffer holds 16 bytes per segment of the largest block
+    const bool bun = !f64 && g->bun.on;
+    const int nblk = bun ? (int)g->bun.part.size() : g->nblk;
     float *b32[3] = {(float *)g->d_segbuf, (float *)g->d_segbuf + g->max_blk_seg,
                      (float *)g->d_segbuf + 2 * g->max_blk_seg};
+    if (bun)
+        for (int q = 0; q < 3; ++q) b32[q] = g->bun.buf[q];
     double *b64[2] = {(double *)g->d_segbuf, (double *)g->d_segbuf + g->max_blk_seg};
     const bool fold = !f64 && g->sw_fold && g->sw_stages == 0;  // no separate gather-weight stream
     const int64_t bps = f64 ? 48 : (scatter ? 28 : 24) - (fold ? 4 : 0);  // streamed bytes per segment
     auto segs = [&](int b) -> int64_t {
+        if (bun) return g->bun.segs[b];
         return g->h_ang_seg_off[g->blk_w0[b] + g->blk_nw[b]] - g->h_ang_seg_off[g->blk_w0[b]];
     };
+    auto mbytes = [&](int b) -> int64_t { return bun ? g->bun.bytes[b] : bps * segs(b); };
     auto march = [&](int b, int q, cudaStream_t st) -> cudaError_t {
+        if (bun) {
+            const Bun32 &m = g->bun.part[b];
+            return m.nbun > 0 ? bun_march(m, S_src, g->d_B, (float)g->I_outer, homog, b32[q], st) : cudaSuccess;
+        }
         if (!f64) return march_sw_launch(sw_march(g, b, homog, b32[q]), g->sw_coarsen, st);
         return ray64_march(ray64_block(g, b), S_src, g->d_B, g->I_outer, homog, b64[q], st);
     };
     auto gather = [&](int b, int q, cudaStream_t st) -> cudaError_t {
+        if (bun) {
+            SwGather t = g->bun.ga[b];
+            t.buf = b32[q];
+            t.J = J;
+            return gather_rows_sw_launch(t, g->nvox, st);
+        }
         SwGather t = sw_gather(g, b, b32[q], J);
         if (f64) {
             t.buf = nullptr;
@@ -1206,11 +1482,11 @@ int run_fs_J_sw(rt_grid *g, int prec, int homog, const double *S_src, double *J)
         return scatter ? gather_rows_sw_launch(t, g->nvox, st) : gather_sw_launch(t, st);
     };
     if (!g->sw_overlap) {
-        if (!f64) RCK(prep32(g, S_src, g->st));
-        for (int b = 0; b < g->nblk; ++b) {
+        if (!f64 && !bun) RCK(prep32(g, S_src, g->st));
+        for (int b = 0; b < nblk; ++b) {
             int t0 = tstart(g, 0);
             CK(march(b, 0, g->st));
-            tstop(g, t0, 0, segs(b), bps * segs(b));
+            tstop(g, t0, 0, segs(b), mbytes(b));
             t0 = tstart(g, 1);
             CK(gather(b, 0, g->st));
             tstop(g, t0, 1, segs(b));
@@ -1275,20 +1551,36 @@ int run_fs_J_sw_streams(rt_grid *g, int prec, int homog, const double *S_src, do
 {
     const bool f64 = prec == RT_FP64;
     const bool scatter = g->sw_scatter && g->d_pos;
+    const bool bun = !f64 && g->bun.on;
+    const int nblk = bun ? (int)g->bun.part.size() : g->nblk;
     float *b32[3] = {(float *)g->d_segbuf, (float *)g->d_segbuf + g->max_blk_seg,
                      (float *)g->d_segbuf + 2 * g->max_blk_seg};
+    if (bun)
+        for (int q = 0; q < 3; ++q) b32[q] = g->bun.buf[q];
     double *b64[2] = {(double *)g->d_segbuf, (double *)g->d_segbuf + g->max_blk_seg};
     const bool fold = !f64 && g->sw_fold && g->sw_stages == 0;  // no separate gather-weight stream
     const int64_t bps = f64 ? 48 : (scatter ? 28 : 24) - (fold ? 4 : 0);  // streamed bytes per segment
     auto segs = [&](int b) -> int64_t {
+        if (bun) return g->bun.segs[b];
         return g->h_ang_seg_off[g->blk_w0[b] + g->blk_nw[b]] - g->h_ang_seg_off[g->blk_w0[b]];
     };
-    if (!f64) RCK(prep32(g, S_src, base));
+    if (!f64 && !bun) RCK(prep32(g, S_src, base));
+    auto mbytes = [&](int b) -> int64_t { return bun ? g->bun.bytes[b] : bps * segs(b); };
     auto march = [&](int b, int q, cudaStream_t st) -> cudaError_t {
+        if (bun) {
+            const Bun32 &m = g->bun.part[b];
+            return m.nbun > 0 ? bun_march(m, S_src, g->d_B, (float)g->I_outer, homog, b32[q], st) : cudaSuccess;
+        }
         if (!f64) return march_sw_launch(sw_march(g, b, homog, b32[q]), g->sw_coarsen, st);
         return ray64_march(ray64_block(g, b), S_src, g->d_B, g->I_outer, homog, b64[q], st);
     };
     auto gather = [&](int b, int q, cudaStream_t st) -> cudaError_t {
+        if (bun) {
+            SwGather t = g->bun.ga[b];
+            t.buf = b32[q];
+            t.J = J;
+            return gather_rows_sw_launch(t, g->nvox, st);
+        }
         SwGather t = sw_gather(g, b, b32[q], J);
         if (f64) {
             t.buf = nullptr;
@@ -1298,7 +1590,7 @@ int run_fs_J_sw_streams(rt_grid *g, int prec, int homog, const double *S_src, do
     };
     // events: fork, join, march done and gather done per buffer, join of each extra march stream
     cudaEvent_t fork = g->sev[0], join = g->sev[1], *mdone = g->sev + 2, *gdone = g->sev + 5, *mjoin = g->sev + 8;
-    const int nms = std::min(g->nblk, f64 ? std::min(g->sw_mstreams, 2) : g->sw_mstreams);
+    const int nms = std::min(nblk, f64 ? std::min(g->sw_mstreams, 2) : g->sw_mstreams);
     const int nbuf = std::max(2, nms);  // a buffer per march that may run at once
     cudaStream_t ms[3] = {base, g->st3, g->st4};
     for (int q = 1; q < nms; ++q) {
@@ -1309,13 +1601,13 @@ int run_fs_J_sw_streams(rt_grid *g, int prec, int homog, const double *S_src, do
     CK(cudaEventRecord(fork, base));
     CK(cudaStreamWaitEvent(g->st2, fork, 0));
     for (int q = 1; q < nms; ++q) CK(cudaStreamWaitEvent(ms[q], fork, 0));
-    for (int b = 0; b < g->nblk; ++b) {
+    for (int b = 0; b < nblk; ++b) {
         const int q = b % nbuf;
         cudaStream_t s = ms[b % nms];
         if (b >= nbuf) CK(cudaStreamWaitEvent(s, gdone[q], 0));  // the gather that read buffer q
         int t0 = tstart(g, 0, s);
         CK(march(b, q, s));
-        tstop(g, t0, 0, segs(b), bps * segs(b), s);
+        tstop(g, t0, 0, segs(b), mbytes(b), s);
         CK(cudaEventRecord(mdone[q], s));
         CK(cudaStreamWaitEvent(g->st2, mdone[q], 0));
         t0 = tstart(g, 1, g->st2);
@@ -1816,6 +2108,7 @@ int rt_set_opacity(rt_grid *g, const double *chi, const double *eps, const doubl
     g->launches++;
     g->lstar_prec = -1;
     g->cw_ok = false;
+    g->bun.cw_ok = false;
     g->cw64_ok = false;
     g->nn_ok = false;
     g->b32_ok = g->b32b_ok = false;

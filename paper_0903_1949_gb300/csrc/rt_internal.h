@@ -92,6 +92,8 @@ struct RadixScratch {
 int64_t radix_tiles(int64_t n);
 // Ownership (CSR) lists of one angle block: csr_off (nvox + 1) and perm_blk, every
 // voxel's segment indices in increasing order.
+// Indices 0..n-1 in the order of their keys' low `bits` bits, stable.
+cudaError_t radix_order(const uint32_t *key, int64_t n, int bits, int32_t *perm, const RadixScratch &rs, cudaStream_t st);
 cudaError_t csr_build(int nvox, const uint32_t *vox_blk, int64_t nseg_blk, int32_t *counts, int32_t *csr_off,
                       int32_t *perm_blk, int64_t *tmp, const RadixScratch &rs, cudaStream_t st);
 cudaError_t csr_invL(int nvox, const int32_t *csr_off, const int32_t *perm_blk, const double *len64_blk,
@@ -267,6 +269,41 @@ cudaError_t ray64_full(const Ray64 &m, const double *S, const double *B, double 
 // Cartesian flux adjoint, when gc is not NULL).
 cudaError_t ray64_adjoint(const Ray64 &m, const double *u, const double *gc, const double *dirs,
                           const int32_t *ray_angle, double *out, cudaStream_t st);
+// One part of the solid angles of the bundled mixed-precision J-only formal
+// solution (bundle32.cu): its characteristics [r_lo, r_hi) in sorted order, cut into
+// bundles of BUN_WARPS shares of about `sub` segments.
+constexpr int BUN_CAP = 6144;   // segments of a bundle at most
+constexpr int BUN_WARPS = 8;    // shares of a bundle
+constexpr int BUN_K = 4;        // consecutive segments of a lane
+constexpr int BUN_RUN = 32;     // values of a unit at most
+struct Bun32 {
+    int64_t r_lo, r_hi, seg_lo, slot_lo;
+    int nbun, sub, dmax;    // dmax: different voxels of a bundle at most
+    const int64_t *ray_off;
+    const int32_t *order;   // characteristics in sorted order (all parts)
+    const int64_t *boff;    // first segment of each in that order (all parts)
+    const int32_t *sray, *sseg;  // shares: first characteristic and segment, of the part
+    float4 *cw;             // weights with the gather weight folded in, by slot
+    uint32_t *wd;           // unit, flags and place, by slot
+    const int2 *ub;         // first unit and first voxel of each bundle
+    uint32_t *dvox;         // the bundles' different voxels
+    int32_t *upos;          // place of each unit in the part's voxel order
+    uint32_t *ubeg;         // first place of each unit in its bundle, and its length << 16
+};
+// Sort keys (and their bits) of the part's characteristics, for radix_order.
+cudaError_t bun_keys(const int64_t *ray_off, int64_t r_lo, int64_t n, const uint32_t *vox, const int32_t *ray_angle,
+                     int a0, int n_ang, int n1, int n2, int n3, uint32_t *key, int *bits, cudaStream_t st);
+cudaError_t bun_maxlen(int64_t n_rays, const int64_t *ray_off, int32_t *mx, cudaStream_t st);
+cudaError_t bun_bounds(const Bun32 &m, int64_t nseg, int32_t *sray, int32_t *sseg, cudaStream_t st);
+cudaError_t bun_units(const Bun32 &m, int nvox, const uint32_t *vox, uint32_t *tv, uint32_t *tb, uint32_t *td, int32_t *nunit,
+                      int32_t *ndist, int *err,                      cudaStream_t st);
+cudaError_t bun_ub(int nbun, const int64_t *uoff, const int64_t *doff, int2 *ub, int32_t *mx, cudaStream_t st);
+cudaError_t bun_compact(const Bun32 &m, const uint32_t *tv, const uint32_t *tb, const uint32_t *td, uint32_t *uvox,
+                        cudaStream_t st);
+cudaError_t bun_coef(const Bun32 &m, const uint32_t *vox, const double *len64, const double *chi,
+                     const int32_t *ray_angle, const double *wt, const double *invL, int nvox, cudaStream_t st);
+cudaError_t bun_march(const Bun32 &m, const double *S, const double *B, float I_outer, int homog, float *out,
+                      cudaStream_t st);
 struct SwGather {
     const int32_t *off, *jorder, *jsell, *crow, *cbeg, *clr, *lfirst, *perm;
     const int64_t *jgbase;
