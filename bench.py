@@ -167,7 +167,7 @@ def hbm_peak():
         return DEFAULT_HBM_FALLBACK, "fallback"
 
 
-MARCH_SRC = os.path.join(ROOT, "paper_0903_1949_gb300", "csrc", "fs_sw.cu")
+MARCH_SRC = os.path.join(ROOT, "paper_0903_1949_gb300", "csrc", "bundle32.cu")
 TIMING_EVERY = 8  # sample of march launches bracketed by events in the timed region
 
 
@@ -183,7 +183,7 @@ def ncu_traffic(segments_per_launch):
     return d["dram_bytes_per_segment"] * segments_per_launch, d.get("capture")
 
 
-FP64_SRC = [os.path.join(ROOT, "paper_0903_1949_gb300", "csrc", f) for f in ("fs_sw.cu", "march.cu", "coef.cuh")]
+FP64_SRC = [os.path.join(ROOT, "paper_0903_1949_gb300", "csrc", f) for f in ("ray64.cu", "march.cu", "coef.cuh")]
 
 
 def fp64_flops_per_segment():
@@ -505,7 +505,7 @@ def main():
             "fp64": {"value": value64, "unit": UNIT, "ms_per_step": ms64, "steps": k64, "fp64_peak": fp64_peak,
                      "mixed_over_fp64": value / value64,
                      "roofline": fp64_roofline(flops64, flops64_src, info["n_segments"], ms64, ms64p, fp64_peak),
-                     "path": "FP64 march with FP64 weights streamed per chi (48 B per segment), FP64 gather",
+                     "path": "FP64 march with FP64 weights streamed per chi (48 B per segment), one characteristic per lane, FP64 gather",
                      "plain": {"value": value64p, "ms_per_step": ms64p, "steps": 2,
                                "mixed_over_fp64_plain": value / value64p,
                                "path": "FP64 march evaluating its weights per segment (FP64-ALU bound)"}},
@@ -513,19 +513,21 @@ def main():
                          "frac": achieved / peak, "traffic": traffic,
                          "traffic_over_algorithmic": (traffic / (ALGO_BYTES_PER_SEGMENT * seg_per_launch)
                                                       if traffic else None),
-                         "kernel": "k_march_sw (FP32 streamed-weight ray march, J only)",
+                         "kernel": "k_march_bun (FP32 streamed-weight march of bundles of characteristics, J only)",
                          "algorithmic_bytes": "%d B per crossing segment (int32 voxel id + FP32 path length, the "
                                               "method's minimum stream)" % ALGO_BYTES_PER_SEGMENT,
                          "design_bytes": {"per_segment": bytes_per_seg, "achieved": achieved_design,
                                           "frac": achieved_design / peak,
-                                          "what": "bytes this design streams per segment: u32 voxel word + four FP32 "
-                                                  "weights (E, alpha, beta, gamma, with the gather weight w l/L folded "
-                                                  "in when 24 B) + i32 list position"},
+                                          "what": "bytes this design streams per segment: four FP32 weights (E, alpha, "
+                                                  "beta, gamma, with the gather weight w l/L folded in), a u32 word "
+                                                  "(voxel and place in the bundle), and 8 bytes per unit and 4 per "
+                                                  "voxel of a bundle"},
                          "segments_per_launch": seg_per_launch, "avg_launch_ms": march_avg_ms,
                          "avg_launch_ms_events": march_event_ms,
                          "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs)" % peak_src if peak_src == "measured"
                          else "fallback 6800 GB/s", "traffic_source": traffic_src,
-                         "timing": "march bytes of a step (one launch per angle block, %d blocks) over the "
+                         "timing": "march bytes of a step (a launch per angle block, small ones together, %d "
+                                   "blocks) over the "
                                    "event-timed step on the bench stream (avg_launch_ms = step / blocks): the "
                                    "marches alternate between three streams and overlap at their ends, the J gathers "
                                    "run in block order on a fourth, the whole J-only formal solution replayed as one "

@@ -157,7 +157,13 @@ int rt_set_precision(rt_grid *g, int precision);
  * per segment of device memory with the gather weight folded in, see
  * RT_TUNE_FOLD_WEIGHT; 20 without), as FP64 for RT_FP64 (48 bytes), each
  * allocated at its first use; 0, or when that memory is not available: the
- * march evaluates the weights itself from chi and l.
+ * march evaluates the weights itself from chi and l.  With the default settings
+ * of RT_TUNE_MARCH_COARSEN, RT_TUNE_MARCH_CHUNK, RT_TUNE_MARCH_STAGES and
+ * RT_TUNE_FOLD_WEIGHT the RT_MIXED march takes bundles of neighbouring
+ * characteristics whose values are added in shared memory; RT_TUNE_SCATTER,
+ * RT_TUNE_S_BLOCKED and RT_TUNE_MARCH_LOOKAHEAD then have no effect.  Any other
+ * setting, or tables that do not fit: the march in launch order, to which those
+ * three belong.
  * RT_TUNE_MARCH_COARSEN: segments per lane of the streamed-weight march, 1
  * (default), 2 or 4.  RT_TUNE_OVERLAP (default 1): the J gather of angle block b
  * runs on a second stream of the library while block b + 1 is marched (the
@@ -509,7 +515,8 @@ typedef struct rt_timing {
     int64_t kernel_launches;  /* every kernel this library launched on the grid since the reset */
     int64_t march_bytes;      /* DRAM bytes the timed march launches stream by design (per segment:
                                  8 FP32, 12 FP64; streamed-weight FP32 24, or 20 without RT_TUNE_SCATTER,
-                                 4 more without RT_TUNE_FOLD_WEIGHT; streamed-weight FP64 48) */
+                                 4 more without RT_TUNE_FOLD_WEIGHT; streamed-weight FP32 in bundles 20
+                                 and 8 per unit, 4 per voxel of a bundle; streamed-weight FP64 48) */
     double os_ms;             /* summed event time of the nearest-neighbour OS-step solves (timing 1 only) */
     int64_t os_solves;        /* OS-step solves since the reset (counted at any timing setting) */
     int64_t os_krylov_its;    /* their BiCGSTAB iterations */

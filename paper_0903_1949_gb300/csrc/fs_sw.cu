@@ -1,6 +1,8 @@
 // fs_sw.cu -- J-only formal solution of the ALI iteration with streamed
-// segment weights (the hot loop of the mixed-precision path, FP32; the FP64
-// march is in ray64.cu, its gathers are here).
+// segment weights, the characteristics in launch order (FP32), and the J gathers.
+// The mixed-precision path takes the bundles of bundle32.cu by default (1.06 to
+// 1.56 times as fast) and this march where their tables do not fit or a setting
+// that belongs to it is chosen; the FP64 march is in ray64.cu.
 //
 // The weights of a segment in the recurrence I_k = I_{k-1} E_k + alpha_k
 // S_{k-1} + beta_k S_k + gamma_k S_{k+1} (scheme R6 of Papers I-II, Sect. 2)

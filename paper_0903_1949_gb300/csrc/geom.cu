@@ -726,7 +726,7 @@ struct PredVisit {
     }
 };
 
-// The coverage completion of k_complete with a guess of which candidates will
+// The serial coverage completion with a guess of which candidates will
 // be hit.  A round looks at the unhit voxels in increasing order, 32 at a time:
 // each is walked in float (pwalk) and, in voxel order, either held back (an
 // earlier chosen candidate's guessed line crosses it: stamp[v] == round) or
