@@ -21,6 +21,7 @@ CASES = [  # coord, n, angles, inner boundary, interpolation, angle_block, again
     (I.CYLINDRICAL, (33, 9, 5), (12, 12), I.TRANSPARENT, rt.RT_PARABOLIC, 0, True),
     (I.SPHERICAL, (17, 9, 33), (24, 24), I.CORE_B, rt.RT_PARABOLIC, 0, False),  # full bundles, long lists
     (I.SPHERICAL, (33, 17, 33), (24, 24), I.CORE_B, rt.RT_PARABOLIC, 0, False),  # several parts
+    (I.SPHERICAL, (129, 64, 65), (1, 2), I.CORE_B, rt.RT_PARABOLIC, 0, False),  # 64-bit keys of the tables' sort
 ]
 
 
