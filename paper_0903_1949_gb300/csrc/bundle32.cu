@@ -347,38 +347,40 @@ __global__ void k_bun_ub(int n, const int64_t *uoff, const int64_t *doff, int2 *
 
 // Weights of every segment for the current chi, with the gather weight folded in,
 // as k_coef_stream_fold forms them (same values), to the segments' slots: a warp per
-// share, its lanes along a characteristic.
+// characteristic (a warp per share waited for one characteristic after another).
 __global__ void __launch_bounds__(256) k_bun_coef(Bun32 m, const uint32_t *__restrict__ vox,
                                                   const double *__restrict__ len64, const double *__restrict__ chi,
                                                   const int32_t *__restrict__ ray_angle, const double *__restrict__ wt,
                                                   const double *__restrict__ invL, int nvox)
 {
-    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (k >= (int64_t)m.nbun * NW) return;
-    const int lane = threadIdx.x & 31, sb = m.sseg[k];
-    const int64_t base = share_base(m, k, sb);
-    for (int q = m.sray[k]; q < m.sray[k + 1]; ++q) {
-        const int64_t r = m.order[m.r_lo + q], s0 = m.ray_off[r];
-        const int len = (int)(m.ray_off[r + 1] - s0), at = (int)(m.boff[m.r_lo + q] - m.seg_lo) - sb;
-        const int a = ray_angle[r];
-        const double *iL = invL + (int64_t)a * nvox;
-        for (int i = lane; i < len; i += 32) {
-            const int64_t s = s0 + i;
-            const uint32_t w = vox[s];
-            const bool para = (w & RTK_PARA) != 0u;
-            const float x = (float)(chi[w & RTK_VOXMASK] * len64[s]);
-            const float p = para ? (float)(chi[vox[s + 1] & RTK_VOXMASK] * len64[s + 1]) : 0.0f;
-            float E, al, be, ga;
-            Coef32::eval(x, p, para, E, al, be, ga);
-            if (w & (RTK_RAYSTART | RTK_RESTART)) {
-                be += al;
-                al = 0.0f;
-            }
-            const float c = (float)(wt[a] * len64[s] * iL[w & RTK_VOXMASK]);
-            float A = c * E;
-            if (!(w & RTK_RAYSTART)) A = __fdividef(A, (float)(wt[a] * len64[s - 1] * iL[vox[s - 1] & RTK_VOXMASK]));
-            __stcs(m.cw + slot_of(base, at + i), make_float4(A, c * al, c * be, c * ga));
+    const int64_t q = m.r_lo + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+    if (q >= m.r_hi) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t r = m.order[q], s0 = m.ray_off[r];
+    const int len = (int)(m.ray_off[r + 1] - s0), at0 = (int)(m.boff[q] - m.seg_lo);
+    if (len <= 0) return;
+    const int64_t k = at0 / m.sub;  // its share, by k_bun_bounds
+    const int at = at0 - m.sseg[k];
+    const int64_t base = share_base(m, k, m.sseg[k]);
+    const int a = ray_angle[r];
+    const double wa = wt[a];
+    const double *iL = invL + (int64_t)a * nvox;
+    for (int i = lane; i < len; i += 32) {
+        const int64_t s = s0 + i;
+        const uint32_t w = vox[s];
+        const bool para = (w & RTK_PARA) != 0u;
+        const float x = (float)(chi[w & RTK_VOXMASK] * len64[s]);
+        const float p = para ? (float)(chi[vox[s + 1] & RTK_VOXMASK] * len64[s + 1]) : 0.0f;
+        float E, al, be, ga;
+        Coef32::eval(x, p, para, E, al, be, ga);
+        if (w & (RTK_RAYSTART | RTK_RESTART)) {
+            be += al;
+            al = 0.0f;
         }
+        const float c = (float)(wa * len64[s] * iL[w & RTK_VOXMASK]);
+        float A = c * E;
+        if (!(w & RTK_RAYSTART)) A = __fdividef(A, (float)(wa * len64[s - 1] * iL[vox[s - 1] & RTK_VOXMASK]));
+        __stcs(m.cw + slot_of(base, at + i), make_float4(A, c * al, c * be, c * ga));
     }
 }
 
@@ -645,8 +647,8 @@ cudaError_t bun_compact(const Bun32 &m, const uint32_t *tv, const uint32_t *tb, 
 cudaError_t bun_coef(const Bun32 &m, const uint32_t *vox, const double *len64, const double *chi,
                      const int32_t *ray_angle, const double *wt, const double *invL, int nvox, cudaStream_t st)
 {
-    const int64_t nsub = (int64_t)m.nbun * NW;
-    k_bun_coef<<<(unsigned)((nsub + 7) / 8), 256, 0, st>>>(m, vox, len64, chi, ray_angle, wt, invL, nvox);
+    if (m.r_hi <= m.r_lo) return cudaSuccess;
+    k_bun_coef<<<(unsigned)((m.r_hi - m.r_lo + 7) / 8), 256, 0, st>>>(m, vox, len64, chi, ray_angle, wt, invL, nvox);
     return cudaGetLastError();
 }
 
