@@ -260,10 +260,14 @@ __global__ void k_line_rhs(int nvox, int nf, const double *J, const double *phi,
     y[v] = (1.0 - eps_l[v]) * jb + eps_l[v] * B[v] - S_l[v];
 }
 
-// Segments of a wave at most (unless one item alone has more): 48 MB of FP32
-// values, so that with the next wave's in its other buffer they stay in L2 from
-// the march to the gather, and two bundles for every resident warp of the march.
-constexpr int64_t WAVE_SEG = 12000000;
+// Segments of a wave at most (unless one item alone has more).  Small waves keep
+// their values in L2 for the gather, large ones fill the march's resident warps to
+// the end, which is worth more.  12, 24, 48, 100, 200 million: twelve members on
+// 65 x 33 x 65 and 33 x 17 x 33 voxels x 8 x 8 solid angles 35.7, 33.9, 33.3, 33.0, 33.2
+// ms; 256 members x 16 x 16, an iteration, 1284, 1176, 1123, -, 1089; 32 frequencies of
+// a line on 65 x 33 x 65 x 32 x 32, an iteration, 417, 388, 372, -, 364.  The two
+// buffers take 8 bytes a segment of the largest wave.
+constexpr int64_t WAVE_SEG = 100000000;
 
 struct Wave {
     int n = 0;            // items
