@@ -41,7 +41,7 @@
 //     neighbour rows without branches         26.2 / 20.6 / 21.4 us
 //   + two phases                              23.7 / 18.8 / 18.6 us
 //   + polls of the packets' numbers alone (the partials in the polled words cost
-//     3500 cycles a poll), two-float sums, beta without waiting for omega
+//     3500 cycles a poll), two-float sums
 //                                             17.1 / 12.8 / 13.3 (17.5 / 48.2) us
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -396,7 +396,7 @@ __device__ __forceinline__ void put(Scal &s, int i, double v)
 
 // The BiCGSTAB coefficients and the stopping rules, kept by thread 0.
 struct Coefs {
-    double rho, alpha, omega, beta, best, ts, tt;
+    double rho, alpha, omega, beta, best;
     int best_it;
     bool bad;
     __device__ void start() { rho = 0.0, alpha = omega = 1.0, beta = 0.0, best = INFINITY, best_it = 0, bad = false; }
@@ -416,11 +416,11 @@ struct Coefs {
             omega = 0.0;
         }
     }
-    // after set_omega(ts, tt): omega = ts / tt, so beta = (rho / rho_old) (alpha / omega)
-    // is one division that does not wait for omega's
-    __device__ void set_rho(double rho_new, double ts, double tt)
+    // after set_omega: quotients of like sizes, so that a source function of any scale
+    // passes (rho and the sums go with its square, their products with its fourth power)
+    __device__ void set_rho(double rho_new)
     {
-        beta = (rho_new * alpha * tt) / (rho * ts);
+        beta = (rho_new / rho) * (alpha / omega);
         rho = rho_new;
         if (!isfinite(beta) || !(rho != 0.0)) bad = true;
     }
@@ -507,7 +507,6 @@ __device__ __forceinline__ int bicgstab(const Kv &a, const Inner<T> &b, double t
         if (!grid_reduce<2, 0u>(a, bar, w2, tot)) return -1;
         if (threadIdx.x == 0) {
             q.set_omega(tot[0], tot[1]);
-            q.ts = tot[0], q.tt = tot[1];
             put(sc, 1, q.omega);
         }
         __syncthreads();
@@ -526,7 +525,7 @@ __device__ __forceinline__ int bicgstab(const Kv &a, const Inner<T> &b, double t
         }
         if (!grid_reduce<2, 2u>(a, bar, w3, tot)) return -1;
         if (threadIdx.x == 0) {
-            q.set_rho(tot[0], q.ts, q.tt);
+            q.set_rho(tot[0]);
             sc.stop = q.stop(tot[1], tol, it, window);
             put(sc, 0, q.beta);
         }
@@ -676,7 +675,7 @@ __device__ __forceinline__ int bicgstab_tile(const Kv &a, double tol, int window
             }
             if (threadIdx.x == 0) {
                 k.set_omega(tot[0], tot[1]);
-                k.set_rho(tot[2] - k.omega * tot[3], tot[0], tot[1]);
+                k.set_rho(tot[2] - k.omega * tot[3]);
                 put(sc, 0, k.beta);
                 put(sc, 1, k.omega);
             }
