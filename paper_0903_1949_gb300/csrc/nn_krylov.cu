@@ -89,6 +89,7 @@ struct Kv {  // the solve's vectors and constants
     int halo;       // halo reach in voxel index either side of the block's range
     int hcap;       // halo buffer length in shared memory (floats, a multiple of 4)
     int tile;       // the FP32 solve keeps its halos in shared memory
+    int own_rho;    // ... and takes (rh, r) from a reduction of its own
     int msm;        // ... and the block's FP32 rows M too
     int far;        // the halo leaves out the neighbours across the phi seam (cylindrical)
 };
@@ -543,6 +544,11 @@ __device__ __forceinline__ float form_p(float r, float p, float v, float bt, flo
     return fmaf(bt, fmaf(-om, v, p), r);
 }
 __device__ __forceinline__ float form_s(float r, float v, float al) { return fmaf(-al, v, r); }
+__device__ __forceinline__ float4 form_p4(float4 r, float4 p, float4 v, float bt, float om)
+{
+    return make_float4(form_p(r.x, p.x, v.x, bt, om), form_p(r.y, p.y, v.y, bt, om), form_p(r.z, p.z, v.z, bt, om),
+                       form_p(r.w, p.w, v.w, bt, om));
+}
 
 // u_v - sum over q != 13 of M_q,v u[neighbour q of v], u read from the halo h
 // (voxels hb .. he-1) or, past it, formed by far(j); M from the block's copy sm
@@ -617,10 +623,12 @@ __device__ __forceinline__ float row_tile(const Kv &a, const float *sm, int lo, 
 //      (t, s), (t, t), (rh, s) and (rh, t), from which rho = (rh, s) - omega (rh, t)
 // so rho needs no third phase; the stopping test of an iteration comes with the
 // next one's A.  A barrier, its reduction and the halo's way through L2 are most
-// of a phase.  Adds d to x.  Returns the iterations, or -1 when a barrier wait
-// gave up.
+// of a phase.  With OWN, (rh, r) and max |r| are reduced as soon as r is formed
+// (a third barrier between the two lines of A, the iterates of bicgstab<float>).
+// Adds d to x.  Returns the iterations, or -1 when a barrier wait gave up.
 constexpr int TPF = 3;  // 16-byte pieces of the t halo a thread has in flight while thread 0 forms the scalars
 
+template <bool OWN_RHO>
 __device__ __forceinline__ int bicgstab_tile(const Kv &a, double tol, int window, Bar &bar, double *tot, int lo, int hi)
 {
     extern __shared__ float4 dsm4[];
@@ -675,29 +683,22 @@ __device__ __forceinline__ int bicgstab_tile(const Kv &a, double tol, int window
             }
             if (threadIdx.x == 0) {
                 k.set_omega(tot[0], tot[1]);
-                k.set_rho(tot[2] - k.omega * tot[3]);
-                put(sc, 0, k.beta);
+                if (!OWN_RHO) {
+                    k.set_rho(tot[2] - k.omega * tot[3]);
+                    put(sc, 0, k.beta);
+                }
                 put(sc, 1, k.omega);
             }
             __syncthreads();
-            bt = sc.f[0];
+            if (!OWN_RHO) bt = sc.f[0];
             om = sc.f[1];
             OWN(i) sd[i - lo] = fmaf(om, hr[i - hb], fmaf(al, hp[i - hb], sd[i - lo]));
             __syncthreads();  // the own range's s and p are read before they change
             auto update = [&](int j, float4 t) {
                 float4 &r4 = reinterpret_cast<float4 *>(hr)[j], &p4 = reinterpret_cast<float4 *>(hp)[j];
-                const float4 v4 = reinterpret_cast<const float4 *>(hv)[j];
-                float4 r = r4, p = p4;
-                r.x = form_s(r.x, t.x, om);
-                r.y = form_s(r.y, t.y, om);
-                r.z = form_s(r.z, t.z, om);
-                r.w = form_s(r.w, t.w, om);
-                p.x = form_p(r.x, p.x, v4.x, bt, om);
-                p.y = form_p(r.y, p.y, v4.y, bt, om);
-                p.z = form_p(r.z, p.z, v4.z, bt, om);
-                p.w = form_p(r.w, p.w, v4.w, bt, om);
-                r4 = r;
-                p4 = p;
+                r4 = make_float4(form_s(r4.x, t.x, om), form_s(r4.y, t.y, om), form_s(r4.z, t.z, om),
+                                 form_s(r4.w, t.w, om));
+                if (!OWN_RHO) p4 = form_p4(r4, p4, reinterpret_cast<const float4 *>(hv)[j], bt, om);
             };
 #pragma unroll
             for (int u = 0; u < TPF; ++u) {
@@ -707,6 +708,30 @@ __device__ __forceinline__ int bicgstab_tile(const Kv &a, double tol, int window
             for (int j = (int)threadIdx.x + TPF * (int)blockDim.x; j < hl4; j += (int)blockDim.x)
                 update(j, __ldcg(t4 + j));
             __syncthreads();
+            if (OWN_RHO) {
+                float w3[2] = {0.0f, 0.0f};
+                OWN(i)
+                {
+                    const float ri = hr[i - hb];
+                    w3[0] = fmaf(srh[i - lo], ri, w3[0]);
+                    w3[1] = maxb(w3[1], absb(ri));
+                }
+                if (!grid_reduce<2, 2u>(a, bar, w3, tot)) return -1;
+                if (threadIdx.x == 0) {
+                    k.set_rho(tot[0]);
+                    sc.stop = k.stop(tot[1], tol, it, window) || it >= a.kmax;
+                    put(sc, 0, k.beta);
+                }
+                __syncthreads();
+                if (sc.stop) break;  // d holds the iterations done
+                bt = sc.f[0];
+                for (int j = threadIdx.x; j < hl4; j += (int)blockDim.x) {
+                    float4 &p4 = reinterpret_cast<float4 *>(hp)[j];
+                    p4 = form_p4(reinterpret_cast<const float4 *>(hr)[j], p4, reinterpret_cast<const float4 *>(hv)[j], bt,
+                                 om);
+                }
+                __syncthreads();
+            }
         }
         // v = (I - M) p; alpha = rho / (rh, v).  Past the halo (the phi seam of the
         // cylindrical grid) p is published too and read there.
@@ -729,7 +754,7 @@ __device__ __forceinline__ int bicgstab_tile(const Kv &a, double tol, int window
         // B: halo of v; alpha; s over the halo; t = (I - M) s
         halo_copy(hv, gv, hb, he);
         if (threadIdx.x == 0) {
-            sc.stop = it > 0 && (k.stop(tot[1], tol, it, window) || it >= a.kmax);
+            sc.stop = !OWN_RHO && it > 0 && (k.stop(tot[1], tol, it, window) || it >= a.kmax);
             k.set_alpha(tot[0]);
             put(sc, 0, k.alpha);
         }
@@ -825,7 +850,8 @@ __global__ void __launch_bounds__(RT_, 1) k_os_solve(Kv a)
             if (round > 0 && !(mr < 0.5 * prev)) fp64 = true;  // the FP32 corrections stopped paying
             prev = mr;
             const int k = fp64 ? bicgstab(a, a.i64, 0.5 * a.jtol * mx, 64, bar, tot, lo, hi)
-                    : a.tile ? bicgstab_tile(a, TOL32 * mr, 16, bar, tot, lo, hi)
+                    : a.tile ? (a.own_rho ? bicgstab_tile<true>(a, TOL32 * mr, 16, bar, tot, lo, hi)
+                                          : bicgstab_tile<false>(a, TOL32 * mr, 16, bar, tot, lo, hi))
                              : bicgstab(a, a.i32, TOL32 * mr, 16, bar, tot, lo, hi);
             if (k < 0) return;
             its += k;
@@ -987,6 +1013,7 @@ cudaError_t nn_os_solve(const NnOs &o, cudaStream_t st, double **x_out, int *kry
     a.kmax = std::max(1, o.kmax);
     a.jmax = std::max(1, o.jmax);
     a.stall = o.stall;
+    a.own_rho = o.own_rho;
     a.rows = (int)round4((N + nb - 1) / nb);
     // stencil reach in voxel index: n2 n3 + n3 + 1, and on the spherical grid also
     // the k neighbours across the phi seam (n3 - 1 away); across the cylindrical
@@ -1001,8 +1028,8 @@ cudaError_t nn_os_solve(const NnOs &o, cudaStream_t st, double **x_out, int *kry
         return os_tile_smem(a.hcap, a.rows, threads, &smem, &a.msm);
     };
     const int64_t n23 = (int64_t)o.n2 * o.n3;
-    if (!o.own_rho && (e = halo(o.sph ? n23 + 2 * o.n3 : 2 * n23)) != cudaSuccess) return e;
-    if (!o.own_rho && !o.sph && !a.msm) {
+    if ((e = halo(o.sph ? n23 + 2 * o.n3 : 2 * n23)) != cudaSuccess) return e;
+    if (!o.sph && !a.msm) {
         if ((e = halo(n23 + o.n3 + 1)) != cudaSuccess) return e;
         a.far = 1;
     }

@@ -409,7 +409,7 @@ struct NnOs {
     double jtol;
     int jmax, krylov, kmax;
     int stall;
-    int own_rho;  // != 0: rho of the FP32 BiCGSTAB from a dot product of its own (three reductions an
+    int own_rho;  // != 0: rho of the FP32 BiCGSTAB from a reduction of its own (three grid barriers an
                   // iteration instead of two), see rt_line_step's solve
 };
 int64_t nn_os_work_elems(int nvox);
