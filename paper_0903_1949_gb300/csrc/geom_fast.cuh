@@ -16,7 +16,8 @@
 // Parameters are measured from the line's closest approach to the origin (to
 // the axis on the cylindrical grid): s = t - tm, X = P + s d with P . d = 0, so
 // that P and s are as small as the geometry around the cell and FP32 resolves
-// about 1e-6 of a cell's distance from the centre.
+// about 1e-6 of a cell's distance from the centre.  Lengths and parameters are
+// multiplied by the power of two F.scale, which changes no rounding.
 //
 // Margins.  u = 2^-24 bounds the relative rounding of an operation and of a
 // table entry.  With |x| the size of the terms of a sum, first order in u:
@@ -36,7 +37,7 @@
 constexpr float U24 = 5.9604645e-8f;
 
 struct FastLine {
-    double tm;                       // closest approach
+    double tm;                       // closest approach (unscaled)
     float px, py, pz, dx, dy, dz;    // P and the direction
     float p, p2;                     // |P| (of x, y on the cylindrical grid) and its square
     float pm, pzm, pxy, adz, dxy;    // sizes: |P|, |Pz|, |Px| + |Py| with the FP64 rounding; |dz|, |dx| + |dy|
@@ -46,13 +47,14 @@ struct FastLine {
     bool usable;
 };
 
-__device__ __forceinline__ FastLine fast_line(const GeomDev &G, const Line &L)
+__device__ __forceinline__ FastLine fast_line(const GeomDev &G, const Line &L, double scale)
 {
     FastLine f;
     const bool sph = G.coord == RT_SPHERICAL;
     f.usable = L.a > 1e-8;
     f.tm = f.usable ? -(L.b / L.a) : 0.0;
-    const double x = L.x + f.tm * L.dx, y = L.y + f.tm * L.dy, z = L.z + f.tm * L.dz;
+    const double x = (L.x + f.tm * L.dx) * scale, y = (L.y + f.tm * L.dy) * scale, z = (L.z + f.tm * L.dz) * scale;
+    const float tm = fabsf((float)(f.tm * scale));
     const double p2 = sph ? (x * x + y * y) + z * z : x * x + y * y;
     f.px = (float)x;
     f.py = (float)y;
@@ -62,8 +64,8 @@ __device__ __forceinline__ FastLine fast_line(const GeomDev &G, const Line &L)
     f.dz = (float)L.dz;
     f.p2 = (float)p2;
     f.p = sqrtf(f.p2);
-    const float x2 = (float)(sph ? L.p2 : L.p2 + L.z2);
-    f.fl = 2e-8f * (sqrtf(x2) + fabsf((float)f.tm));
+    const float x2 = (float)((sph ? L.p2 : L.p2 + L.z2) * scale * scale);
+    f.fl = 2e-8f * (sqrtf(x2) + tm);
     f.c64 = 1e-14f * x2;
     f.pm = f.p + f.fl;
     f.pzm = fabsf(f.pz) + f.fl;
@@ -74,7 +76,7 @@ __device__ __forceinline__ FastLine fast_line(const GeomDev &G, const Line &L)
     f.zs = (L.dz > 0.0) - (L.dz < 0.0);
     f.rdz = __fdividef(1.0f, f.dz);
     // squares within FP32's range
-    f.usable = f.usable && x2 < 1e16f && x2 > 1e-16f && fabsf((float)f.tm) < 1e8f;
+    f.usable = f.usable && x2 < 1e16f && x2 > 1e-16f && tm < 1e8f;
     return f;
 }
 
@@ -317,11 +319,11 @@ __device__ __forceinline__ int fast_walk(const GeomDev &G, const GeomF &F, doubl
                          int j, int k, Visit &vis)
 {
     const Line L = make_line(G, x0, y0, z0, dx, dy, dz);
-    const FastLine f = fast_line(G, L);
+    const FastLine f = fast_line(G, L, F.scale);
     const bool sph = G.coord == RT_SPHERICAL;
     const int nsteps = max_steps(G);
     int kind = R_START, surf = 0;
-    float cur = (float)(-f.tm), mcur = 8.0f * U24 * fabsf(cur) + 1e-37f;
+    float cur = (float)(-f.tm * F.scale), mcur = 8.0f * U24 * fabsf(cur) + 1e-37f;
     for (int step = 0; step < nsteps; ++step) {
         const int v = vid(G, i, j, k);
         Nearest N;
@@ -404,7 +406,7 @@ __device__ __forceinline__ int fast_walk(const GeomDev &G, const GeomF &F, doubl
             const int end = exact_step(G, L, exact_root(G, L, kind, surf), i, j, k, tn, kind, surf);
             if (end != RTK_END_LOST) vis.cell(v);
             if (end) return end;
-            cur = (float)(tn - f.tm);
+            cur = (float)((tn - f.tm) * F.scale);
             mcur = 8.0f * U24 * fabsf(cur) + 1e-37f;
         }
     }

@@ -37,6 +37,7 @@ struct GeomF {
     const float *cp, *sp;     // cos/sin of phi_k
     const float *cpm, *spm;   // cos/sin of phi mid-points
     int r0_zero;              // the innermost edge is 0 (cylindrical)
+    double scale;             // power of two that the lengths e1, e3 carry (geom_fast.cuh)
 };
 
 enum { PRED_EXIT = 0, PRED_CORE = 1, PRED_LOST = 2 };

@@ -273,8 +273,10 @@ int upload_tables(rt_grid *g)
 int g_geom_predict = 0;
 
 // Float copies of the geometry tables for the launch set, on the device
-// (freed by the caller through dfree).
-int upload_tables_f(rt_grid *g, GeomF &F, std::vector<void *> &owned)
+// (freed by the caller through dfree).  Lengths are multiplied by the power of two
+// F.scale that brings the largest one between 1 and 2, so that radii in any unit
+// have squares within FP32's range (the guided completion's guess has no scale).
+int upload_tables_f(rt_grid *g, bool guided, GeomF &F, std::vector<void *> &owned)
 {
     const bool sph = g->coord == RT_SPHERICAL;
     const std::vector<double> &pe = sph ? g->h_e[2] : g->h_e[1];
@@ -301,7 +303,12 @@ int upload_tables_f(rt_grid *g, GeomF &F, std::vector<void *> &owned)
             stm[j] = (float)std::sin(tm);
         }
     }
-    std::vector<float> e1(g->h_e[0].begin(), g->h_e[0].end()), e3(g->h_e[2].begin(), g->h_e[2].end());
+    double big = std::fabs(g->h_e[0].back());
+    if (!sph) big = std::max({big, std::fabs(g->h_e[2].front()), std::fabs(g->h_e[2].back())});
+    F.scale = guided ? 1.0 : std::ldexp(1.0, -std::ilogb(big));
+    std::vector<float> e1, e3;
+    for (double e : g->h_e[0]) e1.push_back((float)(e * F.scale));
+    for (double e : g->h_e[2]) e3.push_back((float)(e * F.scale));
     auto up = [&](const std::vector<float> &h, const float **out) -> int {
         float *p = nullptr;
         RCK(dalloc(g, &p, h.size()));
@@ -357,7 +364,7 @@ int build_geometry(rt_grid *g)
     RCK(dalloc(g, &scratch, guided ? (size_t)chunk * 32 * cap : (size_t)(ctas * geom_cover_scratch(g->G))));
     GeomF F{};
     std::vector<void *> ftab;
-    RCK(upload_tables_f(g, F, ftab));
+    RCK(upload_tables_f(g, guided, F, ftab));
     if (guided) {
         RCK(dalloc(g, &pscr, (size_t)chunk * 32 * cap));
         RCK(dalloc(g, &stamp, (size_t)chunk * nvox));
