@@ -148,7 +148,7 @@ int rt_set_precision(rt_grid *g, int precision);
 
 /* Runtime tuning knobs (rt_tune).  RT_TUNE_MARCH_CHUNK: crossing segments per
  * warp bundle in the ray march, 64..16384 (default 512, which a grid too small to
- * give every SM 16 bundles halves down to 64); a bundle always holds whole
+ * give every SM 16 bundles halves down to 64 unless RT_TUNE_BUNDLES is 0); a bundle always holds whole
  * characteristics, so results do not depend on it beyond rounding. */
 #define RT_TUNE_MARCH_CHUNK 1
 /* RT_TUNE_STREAMED_WEIGHTS (default 1): the J-only march of the ALI iteration
@@ -157,13 +157,8 @@ int rt_set_precision(rt_grid *g, int precision);
  * per segment of device memory with the gather weight folded in, see
  * RT_TUNE_FOLD_WEIGHT; 20 without), as FP64 for RT_FP64 (48 bytes), each
  * allocated at its first use; 0, or when that memory is not available: the
- * march evaluates the weights itself from chi and l.  With the default settings
- * of RT_TUNE_MARCH_COARSEN, RT_TUNE_MARCH_CHUNK, RT_TUNE_MARCH_STAGES and
- * RT_TUNE_FOLD_WEIGHT the RT_MIXED march takes bundles of neighbouring
- * characteristics whose values are added in shared memory; RT_TUNE_SCATTER,
- * RT_TUNE_S_BLOCKED and RT_TUNE_MARCH_LOOKAHEAD then have no effect.  Any other
- * setting, or tables that do not fit: the march in launch order, to which those
- * three belong.
+ * march evaluates the weights itself from chi and l.  See RT_TUNE_BUNDLES for the
+ * two forms of the RT_MIXED march.
  * RT_TUNE_MARCH_COARSEN: segments per lane of the streamed-weight march, 1
  * (default), 2 or 4.  RT_TUNE_OVERLAP (default 1): the J gather of angle block b
  * runs on a second stream of the library while block b + 1 is marched (the
@@ -250,6 +245,17 @@ int rt_set_precision(rt_grid *g, int precision);
  * not updated and the knob is 0 again.  It tests the bounded waits without a
  * device fault. */
 #define RT_TUNE_NN_TEST_STALL 18
+/* RT_TUNE_BUNDLES (default 1): the streamed-weight RT_MIXED march takes bundles of
+ * neighbouring characteristics whose values are added in shared memory on grids
+ * where that pays: at least 4e7 crossing segments, four a voxel and solid angle on
+ * average (their tables, once per grid, cost as much as the gain of 50 to 60
+ * iterations there, and of more elsewhere).  2: on every grid whose tables fit.  Both
+ * only with the default settings of RT_TUNE_MARCH_COARSEN, RT_TUNE_MARCH_CHUNK,
+ * RT_TUNE_MARCH_STAGES and RT_TUNE_FOLD_WEIGHT and characteristics of at most 4096
+ * segments; RT_TUNE_SCATTER, RT_TUNE_S_BLOCKED and RT_TUNE_MARCH_LOOKAHEAD then have
+ * no effect.  0, any other setting, or tables that do not fit: the march in launch
+ * order, to which those three belong.  The forms agree to FP32 rounding. */
+#define RT_TUNE_BUNDLES 19
 int rt_tune(rt_grid *g, int knob, int value);
 
 /* Formal solution from the current S with the grid's precision: J, the

@@ -77,13 +77,15 @@ struct rt_grid {
     std::vector<int64_t> ev_segs;
     int64_t launches = 0;
     int march_chunk = 512;  // segments per warp bundle (RT_TUNE_MARCH_CHUNK)
+    int sw_bundles = 1;     // bundled mixed march: 0 never, 1 where it pays, 2 where it fits (RT_TUNE_BUNDLES)
     // The bundle size in use: the default is lowered on small grids until the
     // largest angle block has 16 bundles an SM (a warp takes its bundle 32 segments
-    // after 32: 16 us for 2.7e4 segments in bundles of 512).
+    // after 32: 16 us for 2.7e4 segments in bundles of 512).  With RT_TUNE_BUNDLES 0 the
+    // size is the one given.
     int chunk() const
     {
         int c = march_chunk;
-        while (march_chunk == 512 && c > 64 && max_blk_seg < (int64_t)c * 152 * 16) c /= 2;
+        while (sw_bundles != 0 && march_chunk == 512 && c > 64 && max_blk_seg < (int64_t)c * 152 * 16) c /= 2;
         return c;
     }
     std::vector<int64_t> ev_bytes;  // streamed DRAM bytes of each timed march launch

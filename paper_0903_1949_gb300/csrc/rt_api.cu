@@ -1088,15 +1088,30 @@ bool bun_setup(rt_grid *g)
     return true;
 }
 
+// Whether the bundles of a grid pay for their tables.  The tables cost 0.15 to 0.2 ns a
+// segment once, and what an iteration gains depends on how many characteristics of a
+// solid angle cross a voxel: 5.9 on spherical grids, 2.8 on cylindrical ones, where
+// most lookups and sums stay a voxel's only ones.  Iterations after which a new grid
+// gains (march in launch order -> bundles, and the tables, ms): 8.4e8 segments
+// spherical 50 (6.76 -> 4.33, 122), 2.1e8 51 (1.76 -> 1.13, 32), 5.4e7 60 (0.485 ->
+// 0.331, 9.3); 2.6e7 137, 6.5e6 100, 3.3e6 170, 8e5 above 1000; cylindrical 2e8 450
+// (1.60 -> 1.52, 37), 5.1e7 1000, 6.4e6 460.
+bool bun_pays(const rt_grid *g)
+{
+    return g->n_seg >= 40000000 && g->n_seg >= (int64_t)4 * g->n_ang * g->nvox;
+}
+
 // Whether the mixed J-only formal solution runs in bundles: with the default
 // march (weights with the gather weight folded in, one segment per lane and chunk
-// not chosen); any other setting keeps the march of fs_sw.cu.
+// not chosen) where they pay or are asked for; any other setting keeps the march of
+// fs_sw.cu.
 bool use_bun(rt_grid *g)
 {
     rt_grid::Bundles &u = g->bun;
     u.on = false;
     if (!g->sw_enabled || !g->sw_fold || g->sw_stages != 0 || g->sw_coarsen != 1 || g->march_chunk != 512 || u.state < 0)
         return false;
+    if (g->sw_bundles == 0 || (g->sw_bundles == 1 && !bun_pays(g))) return false;
     if (u.state == 0) {
         u.state = bun_setup(g) ? 1 : -1;
         u.cw_ok = false;
@@ -2156,6 +2171,11 @@ int rt_tune(rt_grid *g, int knob, int value)
     if (knob == RT_TUNE_MARCH_CHUNK) {
         if (value < 64 || value > 16384) return fail(RT_EINVAL, "march chunk must be in [64, 16384]");
         g->march_chunk = value;
+        return RT_OK;
+    }
+    if (knob == RT_TUNE_BUNDLES) {
+        if (value < 0 || value > 2) return fail(RT_EINVAL, "bundles: 0, 1 or 2");
+        g->sw_bundles = value;
         return RT_OK;
     }
     if (knob == RT_TUNE_STREAMED_WEIGHTS) {
