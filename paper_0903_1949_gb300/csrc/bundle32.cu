@@ -14,7 +14,7 @@
 // (2.9e3 on 65^3 cylindrical voxels).  So S is fetched once per voxel of the
 // bundle into shared memory, the lines are marched out of shared memory, c I goes
 // to its place in the bundle's own lists in shared memory, and a voxel's values
-// are added there (compensated); one value per voxel and bundle goes to L2, to
+// are added there (compensated); one sum per voxel and bundle goes to L2, to
 // its place in the voxel order of a part of the solid angles, and the gather of
 // a part adds a quarter as many values.  A voxel with more than BUN_RUN values
 // in a bundle is split into units, and units of equal length lie side by side, a
@@ -397,9 +397,13 @@ __device__ __forceinline__ void l2_prefetch_range(const void *p, int64_t a, int6
     if (hi > lo) l2_prefetch((const void *)lo, (uint32_t)(hi - lo));
 }
 
-__device__ __forceinline__ void st_keep(float *p, float x, uint64_t pol)
+__device__ __forceinline__ void st_keep(float *p, float x, float y, uint64_t pol)
 {
-    asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(p), "f"(x), "l"(pol) : "memory");
+    asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(p), "f"(x + y), "l"(pol) : "memory");
+}
+__device__ __forceinline__ void st_keep(float2 *p, float x, float y, uint64_t pol)
+{
+    asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(p), "f"(x), "f"(y), "l"(pol) : "memory");
 }
 
 // One tile of a share: K slots of this lane; past the share's end neutral weights and the
@@ -427,10 +431,12 @@ __device__ __forceinline__ void load_tile(const float4 *cf, const uint32_t *wp, 
 // share, a tile of K segments per lane at a time, the lane maps I -> A I + b
 // composed by a shuffle scan, the next tile's stream in flight meanwhile and the
 // third one on its way to L2; the values of a unit added in the order of the
-// march, compensated.  Four CTAs an SM cover each other's phases.
+// march, compensated.  Four CTAs an SM cover each other's phases.  OUT: float or
+// float2, a unit's sum with its compensation added or as a second float.
+template <typename OUT>
 __global__ void __launch_bounds__(32 * NW, 4) k_march_bun(Bun32 m, const double *__restrict__ S,
                                                           const double *__restrict__ B, float I_outer, int homog,
-                                                          float *__restrict__ out)
+                                                          OUT *__restrict__ out)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     float *val = reinterpret_cast<float *>(smem), *Ss = val + PLACES + 1;
@@ -561,8 +567,8 @@ __global__ void __launch_bounds__(32 * NW, 4) k_march_bun(Bun32 m, const double 
             sc = (x - s) - y;
             s = x;
         }
-        st_keep(out + po, s - sc, pol);
-        if (v < nu) st_keep(out + qo, r - rc, pol);
+        st_keep(out + po, s, -sc, pol);
+        if (v < nu) st_keep(out + qo, r, -rc, pol);
     }
 }
 
@@ -652,15 +658,23 @@ cudaError_t bun_coef(const Bun32 &m, const uint32_t *vox, const double *len64, c
     return cudaGetLastError();
 }
 
-cudaError_t bun_march(const Bun32 &m, const double *S, const double *B, float I_outer, int homog, float *out,
-                      cudaStream_t st)
+template <typename OUT>
+static cudaError_t bun_march_as(const Bun32 &m, const double *S, const double *B, float I_outer, int homog, OUT *out,
+                                cudaStream_t st)
 {
     static std::atomic<uint64_t> done{0};
-    const cudaError_t e = allow_smem(k_march_bun, sizeof(float) * (PLACES + 1 + BUN_CAP), done);
+    const cudaError_t e = allow_smem(k_march_bun<OUT>, sizeof(float) * (PLACES + 1 + BUN_CAP), done);
     if (e != cudaSuccess) return e;
     const size_t bytes = sizeof(float) * (size_t)(PLACES + 1 + m.dmax);
-    k_march_bun<<<(unsigned)m.nbun, 32 * NW, bytes, st>>>(m, S, B, I_outer, homog, out);
+    k_march_bun<OUT><<<(unsigned)m.nbun, 32 * NW, bytes, st>>>(m, S, B, I_outer, homog, out);
     return cudaGetLastError();
+}
+
+cudaError_t bun_march(const Bun32 &m, const double *S, const double *B, float I_outer, int homog, void *out, bool pair,
+                      cudaStream_t st)
+{
+    return pair ? bun_march_as(m, S, B, I_outer, homog, static_cast<float2 *>(out), st)
+                : bun_march_as(m, S, B, I_outer, homog, static_cast<float *>(out), st);
 }
 
 }  // namespace rtk

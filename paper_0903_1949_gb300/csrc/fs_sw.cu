@@ -22,6 +22,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "coef.cuh"
 #include "rt_internal.h"
@@ -38,6 +39,14 @@ struct Kahan {
         const float y = x - c;
         const float t = s + y;
         c = (t - s) - y;
+        s = t;
+    }
+    // an unevaluated sum of two floats, without rounding x.y away: Knuth's two-sum
+    __device__ __forceinline__ void add(float2 x)
+    {
+        const float t = s + x.x;
+        const float bb = t - s;
+        c -= ((s - (t - bb)) + (x.x - bb)) + x.y;
         s = t;
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
@@ -68,6 +77,7 @@ struct Sum64 {
 };
 template <typename T> struct AccOf;
 template <> struct AccOf<float> { using type = Kahan; };
+template <> struct AccOf<float2> { using type = Kahan; };
 template <> struct AccOf<double> { using type = Sum64; };
 // 16-byte vectors of a row and their entries added in order
 template <typename T> struct Vec16;
@@ -81,6 +91,14 @@ template <> struct Vec16<float> {
         acc.add(x.w);
     }
 };
+template <> struct Vec16<float2> {
+    using type = float4;
+    template <typename A> __device__ __forceinline__ static void add_to(A &acc, const float4 &x)
+    {
+        acc.add(make_float2(x.x, x.y));
+        acc.add(make_float2(x.z, x.w));
+    }
+};
 template <> struct Vec16<double> {
     using type = double2;
     template <typename A> __device__ __forceinline__ static void add_to(A &acc, const double2 &x)
@@ -91,6 +109,7 @@ template <> struct Vec16<double> {
 };
 template <typename T> __device__ __forceinline__ const T *gbuf(const SwGather &t);
 template <> __device__ __forceinline__ const float *gbuf<float>(const SwGather &t) { return t.buf; }
+template <> __device__ __forceinline__ const float2 *gbuf<float2>(const SwGather &t) { return t.buf2; }
 template <> __device__ __forceinline__ const double *gbuf<double>(const SwGather &t) { return t.buf64; }
 
 __device__ __forceinline__ int64_t lb64(const int64_t *a, int64_t lo, int64_t hi, int64_t key)
@@ -629,7 +648,7 @@ __global__ void __launch_bounds__(256) k_gather_rows_sw(SwGather t, int nvox, in
         // length of their lists, since a warp's additions, bound by the FP64 pipe, run to
         // its longest row (5.4e6 values of 65 x 33 x 65 voxels: 46 us in voxel order).
         int v = (int)(cta * 256 + threadIdx.x);
-        if constexpr (sizeof(T) == sizeof(double)) {
+        if constexpr (std::is_same<T, double>::value) {
             if (v >= t.nshort) return;
             v = t.jorder[v];
         }
@@ -648,13 +667,14 @@ __global__ void __launch_bounds__(256) k_gather_rows_sw(SwGather t, int nvox, in
         using V = typename Vec16<T>::type;
         const V *rv = reinterpret_cast<const V *>(row + head);
         const int nvec = (L - head) / NV;
-        for (int q = 0; q < nvec; q += 4) {
-            V x[4];
+        constexpr int U = std::is_same<T, float2>::value ? 8 : 4;  // 16 values in flight (FP64: 8)
+        for (int q = 0; q < nvec; q += U) {
+            V x[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < U; ++u)
                 if (q + u < nvec) x[u] = __ldg(rv + q + u);
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < U; ++u)
                 if (q + u < nvec) Vec16<T>::add_to(acc, x[u]);
         }
         for (int k = head + nvec * NV; k < L; ++k) acc.add(__ldg(row + k));
@@ -672,7 +692,7 @@ __global__ void __launch_bounds__(256) k_gather_rows_sw(SwGather t, int nvox, in
     for (int k = e0 + lane; k < e1; k += 32 * 8) {
         T val[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) val[j] = (k + 32 * j < e1) ? __ldcg(buf + k + 32 * j) : T(0);
+        for (int j = 0; j < 8; ++j) val[j] = (k + 32 * j < e1) ? __ldcg(buf + k + 32 * j) : T{};
 #pragma unroll
         for (int j = 0; j < 8; ++j)
             if (k + 32 * j < e1) acc.add(val[j]);
@@ -879,6 +899,7 @@ cudaError_t gather_rows_sw_launch(const SwGather &t, int nvox, cudaStream_t st)
     const int64_t grid = nvb + (t.nchunks * 32 + 255) / 256;
     if (grid <= 0) return cudaSuccess;
     if (t.buf64) k_gather_rows_sw<double><<<(unsigned)grid, 256, 0, st>>>(t, nvox, nvb);
+    else if (t.buf2) k_gather_rows_sw<float2><<<(unsigned)grid, 256, 0, st>>>(t, nvox, nvb);
     else k_gather_rows_sw<float><<<(unsigned)grid, 256, 0, st>>>(t, nvox, nvb);
     return cudaGetLastError();
 }

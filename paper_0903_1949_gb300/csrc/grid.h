@@ -113,7 +113,8 @@ struct rt_grid {
         std::vector<rtk::Bun32> part;
         std::vector<rtk::SwGather> ga;
         std::vector<int64_t> segs, bytes;  // per part: segments, streamed DRAM bytes of a march
-        float *buf[3] = {};      // one value per unit of a part
+        bool pair = false;       // a unit's sum is two floats
+        void *buf[3] = {};       // one sum per unit of a part
     } bun;
     int pos_state = 0;        // list positions: 0 not tried, 1 allocated, -1 not available
     bool cw_ok = false;       // d_cw4 matches the current chi

@@ -302,7 +302,8 @@ cudaError_t bun_compact(const Bun32 &m, const uint32_t *tv, const uint32_t *tb, 
                         cudaStream_t st);
 cudaError_t bun_coef(const Bun32 &m, const uint32_t *vox, const double *len64, const double *chi,
                      const int32_t *ray_angle, const double *wt, const double *invL, int nvox, cudaStream_t st);
-cudaError_t bun_march(const Bun32 &m, const double *S, const double *B, float I_outer, int homog, float *out,
+// out: a float, or with pair two floats, for each unit's sum.
+cudaError_t bun_march(const Bun32 &m, const double *S, const double *B, float I_outer, int homog, void *out, bool pair,
                       cudaStream_t st);
 struct SwGather {
     const int32_t *off, *jorder, *jsell, *crow, *cbeg, *clr, *lfirst, *perm;
@@ -310,6 +311,7 @@ struct SwGather {
     int *cnt;
     double *part;
     const float *buf;      // c_s I_s of the block (FP32 march)
+    const float2 *buf2;    // unit sums of a part (bundles), two floats each; used when not NULL
     const double *buf64;   // c_s I_s of the block (FP64 march); used when not NULL
     double *J;
     int64_t nshort, nchunks, nbs;

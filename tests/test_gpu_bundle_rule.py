@@ -118,3 +118,39 @@ def test_large_spherical_grid_takes_bundles():
     assert per != 24
     _, per = _run(p, I.CORE_B, LAUNCH, timing=True)
     assert per == 24
+
+
+def test_unit_sums_keep_their_compensation():
+    """One solid angle: most voxels' values make one unit, and a sum of four FP32 values or more is rarely an
+    FP32 number itself (as in launch order, where the compensated sum is taken over the whole list)."""
+    p = tiny_problem(I.SPHERICAL, (17, 9, 17), 1, 1, I.CORE_B, eps=0.1, seed=48)
+    for knobs in (LAUNCH, FORCE):
+        with rt.Grid(p["coord"], p["edges"], p["dirs"], p["weights"], inner_bc=I.CORE_B, precision=rt.RT_MIXED, ng=False,
+                     I_outer=0.25) as g:
+            for k, v in knobs.items():
+                g.tune(k, v)
+            g.set_opacity(p["chi"], p["eps"], p["B"])
+            g.ali_step()
+            g.ali_step()
+            J = g.J()
+            many = np.bincount(g.crossings(0)["vox"], minlength=p["nvox"]) >= 4
+        assert many.sum() > 100 and np.mean((J == J.astype(np.float32))[many]) < 0.5, knobs
+
+
+def test_error_against_fp64():
+    """Few solid angles: bundles are no further from FP64 than launch order (1 % for the other order of the scan)."""
+    p = I.make_problem("sph65", n=(65, 33, 65), n_mu=2, n_phi=4, tau=1e3, noise=0.2)
+    rng = np.random.default_rng(9)
+    S = p["B"] * np.exp(0.5 * rng.standard_normal(p["B"].size))
+    J = {}
+    for name, prec, knobs in (("fp64", rt.RT_FP64, {}), ("launch", rt.RT_MIXED, LAUNCH), ("bundles", rt.RT_MIXED, FORCE)):
+        with rt.Grid(p["coord"], p["edges"], p["dirs"], p["weights"], inner_bc=I.CORE_B, precision=prec, ng=False) as g:
+            for k, v in knobs.items():
+                g.tune(k, v)
+            g.set_opacity(p["chi"], p["eps"], p["B"])
+            g.ali_step()
+            g.set_S(S)
+            g.ali_step()
+            J[name] = g.J()
+    rms = {k: float(np.sqrt(np.mean((J[k] / J["fp64"] - 1.0) ** 2))) for k in ("launch", "bundles")}
+    assert rms["bundles"] < 1.01 * rms["launch"], rms
