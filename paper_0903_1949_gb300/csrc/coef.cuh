@@ -34,22 +34,36 @@ __device__ __forceinline__ double inv_fact(int n)
     return f[n];
 }
 
-// 1 / q to about an ulp: the hardware's 20-bit estimate and one step of the
-// cubically convergent iteration r (1 + e + e^2), e = 1 - q r (three FP64
-// instructions where a correctly rounded division takes about ten).  Outside
-// [2^-900, 2^900], where the estimate would leave the normal range: the division.
+// 1 / q to about an ulp: the hardware's 20-bit estimate and one step of the third
+// order Householder iteration for a reciprocal, r (1 + e + e^2) with e = 1 - q r
+// (A. S. Householder, The Numerical Treatment of a Single Nonlinear Equation, 1970,
+// ch. 4): three FP64 instructions where a correctly rounded division takes about
+// ten.  Outside [2^-900, 2^900], where the estimate would leave the normal range:
+// the division.
+__device__ __forceinline__ bool rcp64_in_range(double q)
+{
+    return (((unsigned)__double2hiint(q) >> 20) & 0x7ffu) - 123u <= 1800u;
+}
 __device__ __forceinline__ double rcp64(double q)
 {
-    const unsigned ex = ((unsigned)__double2hiint(q) >> 20) & 0x7ffu;
-    if (ex - 123u > 1800u) return 1.0 / q;
+    if (!rcp64_in_range(q)) return 1.0 / q;
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
     const double e = fma(-q, r, 1.0);
     return fma(r, fma(e, e, e), r);
 }
 
-// x < 1 for x >= 0, from the high word: off the FP64 pipe (a NaN is not).
+// a / q to half an ulp or a little more: its residual corrects a rcp64(q).
+__device__ __forceinline__ double div64(double a, double q)
+{
+    if (!rcp64_in_range(q)) return a / q;
+    const double r = rcp64(q), t = a * r;
+    return fma(fma(-t, q, a), r, t);
+}
+
+// x < 1 and x < 1/2 for x >= 0, from the high word: off the FP64 pipe (a NaN is neither).
 __device__ __forceinline__ bool below_one(double x) { return (unsigned)__double2hiint(x) < 0x3ff00000u; }
+__device__ __forceinline__ bool below_half(double x) { return (unsigned)__double2hiint(x) < 0x3fe00000u; }
 
 // h1(x) = (e^{-x} - 1 + x) / x^2 and h2(x) = f2(x) / x^2 (see below) on [0, 1]:
 // their values at 0 plus x times polynomials fitted to (h - h(0)) / x at Chebyshev
@@ -93,12 +107,13 @@ __device__ __forceinline__ double h2_small(double x)
 //   linear:    alpha = e0 - f1,           beta = f1,         gamma = 0
 // f1 and f2 cancel catastrophically when evaluated from e0 at small x; below 1
 // they come from polynomials, above it from the exponential.  The three quotients
-// of the parabola share one reciprocal.  The FP64 pipe bounds every kernel that
-// evaluates these: about 41 instructions of it for a small x and 42 for a large one
+// of the parabola share one.  The FP64 pipe bounds every kernel that
+// evaluates these: about 45 instructions of it for a small x and 44 for a large one
 // (62 and 80 with the 19-term series, expm1 and divisions of Coef64Series).  Mean
-// errors against 128-bit arithmetic relative to that form's: equal below 0.5, a
-// third to a tenth in [0.5, 1], equal above but for E, which keeps its relative
-// accuracy.
+// errors of E, alpha, beta, gamma in half ulps of their terms, Coef64Series -> here:
+// below 0.5 0.27, 0.28, 0.49, 0.77 -> 0.27, 0.29, 0.50, 0.69; in [0.5, 1] 0.57, 0.74,
+// 1.58, 11.0 -> 0.46, 0.38, 0.56, 0.70; in [1, 4] 3.2, 0.37, 0.69, 2.51 -> 0.38, 0.40,
+// 0.73, 2.51; above, E keeps its relative accuracy, 0.18, 0.39, 0.67 -> 0.18, 0.40, 0.72.
 struct Coef64 {
     __device__ __forceinline__ static void eval(double x, double p, bool para, double &E, double &al, double &be,
                                                 double &ga)
@@ -108,20 +123,18 @@ struct Coef64 {
             f1 = x * h1_small(x);
             f2 = (x * x) * h2_small(x);
             e0 = fma(-x, f1, x);
-            E = 1.0 - e0;
+            E = below_half(x) ? 1.0 - e0 : fma(x, f1, 1.0 - x);  // 1 - x is exact from 1/2 on
         } else {
             E = exp(-x);
             e0 = 1.0 - E;
-            const double ix = rcp64(x), num = x - e0;
-            f1 = num * ix;
-            f1 = fma(fma(-f1, x, num), ix, f1);  // to half an ulp
+            f1 = div64(x - e0, x);
             f2 = fma(2.0, f1, -e0);
         }
         al = e0 - f1;
         be = f1;
         ga = 0.0;
         if (para) {
-            const double D = x + p, t = f2 * rcp64(p * D);
+            const double D = x + p, t = div64(f2, p * D);
             al = fma(-t, p, al);
             be = fma(t, D, be);
             ga = -(x * t);
@@ -229,7 +242,7 @@ struct Coef32 {
 
 // Derivatives of (E, alpha, beta, gamma) with respect to x = dtau_k and
 // p = dtau_{k+1}, from  e0' = E, f1' = (e0 - f1)/x = g1, f2' = e0 - f1 - f2/x = g2
-// (below the threshold g1 = 1 - h1 - x h1 and g2 = x (g1 - h2)):
+// (below 1 their power series, 19 terms: 1 - h1 - x h1 loses up to half the bits of an ulp more):
 //   parabolic: alpha = e0 - f1 - f2/(x+p), beta = f1 + f2/p, gamma = -x f2/(p (x+p))
 //   linear:    alpha = e0 - f1,           beta = f1
 struct Coef64D {
@@ -239,22 +252,26 @@ struct Coef64D {
     {
         double e0, f1, f2, g1, g2;
         if (below_one(x)) {
-            const double h1 = h1_small(x), h2 = h2_small(x);
-            f1 = x * h1;
-            f2 = (x * x) * h2;
+            constexpr int NS = 19;
+            double k1 = 0.0, k2 = 0.0;
+            // g1 = sum_{n>=2} (-1)^n (n-1) x^(n-2) / n!,  g2 = sum_{m>=3} (-1)^(m+1) (m-2)(m-1) x^(m-2) / m!
+#pragma unroll
+            for (int n = NS + 1; n >= 2; --n) k1 = fma(-x, k1, (double)(n - 1) * inv_fact(n));
+#pragma unroll
+            for (int m = NS + 1; m >= 3; --m) k2 = fma(-x, k2, (double)((m - 2) * (m - 1)) * inv_fact(m));
+            f1 = x * h1_small(x);
+            f2 = (x * x) * h2_small(x);
             e0 = fma(-x, f1, x);
-            E = 1.0 - e0;
-            g1 = (1.0 - h1) - f1;  // (e0 - f1) / x
-            g2 = x * (g1 - h2);
+            E = below_half(x) ? 1.0 - e0 : fma(x, f1, 1.0 - x);
+            g1 = k1;
+            g2 = x * k2;
         } else {
             E = exp(-x);
             e0 = 1.0 - E;
-            const double ix = rcp64(x), num = x - e0;
-            f1 = num * ix;
-            f1 = fma(fma(-f1, x, num), ix, f1);
+            f1 = div64(x - e0, x);
             f2 = fma(2.0, f1, -e0);
-            g1 = (e0 - f1) * ix;
-            g2 = fma(-f2, ix, e0 - f1);
+            g1 = div64(e0 - f1, x);
+            g2 = (e0 - f1) - div64(f2, x);
         }
         dE = -E;
         if (para) {
