@@ -158,7 +158,11 @@ int rt_set_precision(rt_grid *g, int precision);
  * RT_TUNE_FOLD_WEIGHT; 20 without), as FP64 for RT_FP64 (48 bytes), each
  * allocated at its first use; 0, or when that memory is not available: the
  * march evaluates the weights itself from chi and l.  See RT_TUNE_BUNDLES for the
- * two forms of the RT_MIXED march.
+ * two forms of the RT_MIXED march.  Full RT_FP64 formal solutions (rt_formal_solution,
+ * the first iteration after rt_set_opacity) run on the FP64 streams too, and set them
+ * up, when these take at most a quarter of the device's memory and leave as much again
+ * and 24 bytes per segment and 4 GB free; the grid's first one decides that for all of
+ * them.  J, Lambda* and flux of the two ways differ by the rounding of FP64 sums.
  * RT_TUNE_MARCH_COARSEN: segments per lane of the streamed-weight march, 1
  * (default), 2 or 4.  RT_TUNE_OVERLAP (default 1): the J gather of angle block b
  * runs on a second stream of the library while block b + 1 is marched (the

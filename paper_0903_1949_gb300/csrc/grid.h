@@ -103,6 +103,7 @@ struct rt_grid {
     rtk::Wd4 *d_cw64 = nullptr;  // FP64 weights
     double *d_cg64 = nullptr;    // FP64 w l / L
     int sw64_state = 0;
+    int fs64_ray = 0;            // full FP64 formal solutions on these streams: 0 not decided yet, 1 yes, -1 no
     int wp64_pos = -1;           // output positions in d_wp64: 1 list order, 0 segment order, -1 not filled
     bool cw64_ok = false;
     // bundled march of the mixed J-only formal solution (bundle32.cu)

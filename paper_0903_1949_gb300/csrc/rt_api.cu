@@ -732,7 +732,7 @@ int alloc_fields(rt_grid *g)
 }
 
 bool use_sw64(rt_grid *g);
-bool sw64_roomy(const rt_grid *g);
+bool fs64_streams(rt_grid *g);
 Ray64 ray64_block(rt_grid *g, int b);
 
 // Formal solution of every angle block with the FP64 or FP32 march.
@@ -741,7 +741,7 @@ int run_fs(rt_grid *g, int prec, int homog, const double *S_src, double *J, doub
     const int n = g->nvox;
     const int para = g->interp == RT_PARABOLIC;
     // FP64: on the streamed weights, which the iterations that follow need anyway
-    const bool ray = prec == RT_FP64 && sw64_roomy(g) && use_sw64(g);
+    const bool ray = prec == RT_FP64 && fs64_streams(g) && use_sw64(g);
     CK(cudaGetLastError());
     if (!ray) {
         if (prec == RT_FP64) CK(pack_chiS64(n, g->d_chi, S_src, g->d_cs64, g->st));
@@ -1291,17 +1291,25 @@ bool ray64_setup(rt_grid *g)
     return g->d_wp64 && g->d_cw64 && g->d_cg64;
 }
 
-// Whether a single FP64 formal solution may set up the streamed weights: they are
-// there already, or leave as much again and the FP32 streams' room free.
-bool sw64_roomy(const rt_grid *g)
+// Whether full FP64 formal solutions run on the streamed weights, whose results differ
+// from those of the march without them in the last bits: decided at the grid's first
+// one, for all of them.  The streams take a quarter of the device's memory at most, and
+// when they have to be set up for it, they leave as much again and the FP32 streams'
+// room free.
+bool fs64_streams(rt_grid *g)
 {
-    if (g->sw64_state != 0) return g->sw64_state > 0;
-    size_t room = 0, total = 0;
-    if (cudaMemGetInfo(&room, &total) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
+    if (g->fs64_ray == 0) {
+        size_t room = 0, total = 0;
+        g->fs64_ray = -1;
+        if (cudaMemGetInfo(&room, &total) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        const double seg = (double)g->n_seg, streams = 50.0 * seg;
+        const bool there = g->sw64_state > 0, fits = (double)room > 2.0 * streams + 24.0 * seg + 4e9;
+        if (streams <= 0.25 * (double)total && (there || (g->sw64_state == 0 && fits))) g->fs64_ray = 1;
     }
-    return (double)room > 2.0 * 50.0 * (double)g->n_seg + 24.0 * (double)g->n_seg + 4e9;
+    return g->fs64_ray > 0;
 }
 
 // FP64 streamed weights (48 bytes per slot), the same life cycle.
@@ -1309,7 +1317,9 @@ bool use_sw64(rt_grid *g)
 {
     if (!g->sw_enabled || g->sw64_state < 0) return false;
     if (g->sw64_state == 0) {
+        const int64_t before = g->bytes;
         if (!ray64_setup(g)) {
+            g->bytes = before;
             for (void *q : {(void *)g->d_rorder, (void *)g->d_rlen, (void *)g->d_rgbase, (void *)g->d_wp64,
                             (void *)g->d_cw64, (void *)g->d_cg64})
                 dfree(g, q);
