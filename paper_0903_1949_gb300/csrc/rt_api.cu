@@ -795,14 +795,10 @@ int run_fs(rt_grid *g, int prec, int homog, const double *S_src, double *J, doub
     return RT_OK;
 }
 
-// Streamed-weight march: allocate its per-segment arrays on first use (w l / L
-// computed then, from the geometry) and refresh (E, alpha, beta, gamma) after
-// chi changed.  Returns false when disabled or when the arrays do not fit; the
-// FP32 march then evaluates the weights itself.
-// Streamed-weight march, parts shared by both precisions: list positions
-// (optional; without them the gather reads through perm) and the bundle bounds
-// of the current chunk.  Returns false when they cannot be set up.
-bool sw_common(rt_grid *g)
+// Place of every segment in its ownership list, for the streamed-weight marches of
+// both precisions (optional; without them the gather reads through perm).  Returns
+// false on a CUDA error.
+bool sw_positions(rt_grid *g)
 {
     if (g->pos_state == 0) {
         void *c = nullptr;
@@ -822,7 +818,14 @@ bool sw_common(rt_grid *g)
             g->pos_state = -1;
         }
     }
-    if (g->bnd_chunk != g->chunk()) {  // bundle bounds for the current chunk
+    return true;
+}
+
+// Bundle bounds of the current chunk, for the FP32 march in launch order.  Returns
+// false when they cannot be set up.
+bool sw_bounds(rt_grid *g)
+{
+    if (g->bnd_chunk != g->chunk()) {
         std::vector<int64_t> off(g->nblk + 1, 0);
         for (int b = 0; b < g->nblk; ++b) {
             const int w0 = g->blk_w0[b], nw = g->blk_nw[b];
@@ -834,6 +837,7 @@ bool sw_common(rt_grid *g)
             for (auto &q : g->allocs)
                 if (q == (void *)g->d_bnd) q = nullptr;
             g->d_bnd = nullptr;
+            g->bnd_chunk = 0;
         }
         void *q = nullptr;
         if (cudaMalloc(&q, sizeof(int2) * (size_t)std::max<int64_t>(1, off[g->nblk])) != cudaSuccess) {
@@ -1185,7 +1189,7 @@ bool use_sw(rt_grid *g)
         g->cw_ok = true;
         g->cw_fold = fold;
     }
-    return sw_common(g);
+    return sw_positions(g) && sw_bounds(g);
 }
 
 // One angle block of the FP64 streamed march.
@@ -1336,7 +1340,7 @@ bool use_sw64(rt_grid *g)
         g->wp64_pos = -1;
         g->cw64_ok = false;
     }
-    if (!sw_common(g)) return false;
+    if (!sw_positions(g)) return false;
     const int pos = g->sw_scatter && g->d_pos ? 1 : 0;
     if (g->wp64_pos != pos) {
         for (int b = 0; b < g->nblk; ++b)
