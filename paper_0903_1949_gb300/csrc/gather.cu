@@ -847,6 +847,20 @@ cudaError_t radix_order(const uint32_t *key, int64_t n, int bits, int32_t *perm,
     return cudaGetLastError();
 }
 
+int radix_launches(int64_t n, int bits)
+{
+    return n > 0 ? 1 + (bits + 7) / 8 * (2 + scan_launches(RS_BUCKETS * radix_tiles(n))) : 0;
+}
+
+static int voxel_bits(int nvox)
+{
+    int bits = 0;
+    while (bits < 31 && ((int64_t)1 << bits) < (int64_t)nvox) ++bits;
+    return bits;
+}
+
+int csr_launches(int nvox, int64_t n) { return 2 + scan_launches(nvox) + radix_launches(n, voxel_bits(nvox)); }
+
 cudaError_t csr_build(int nvox, const uint32_t *vox_blk, int64_t nseg_blk, int32_t *counts, int32_t *csr_off,
                       int32_t *perm_blk, int64_t *tmp, const RadixScratch &rs, cudaStream_t st)
 {
@@ -860,9 +874,7 @@ cudaError_t csr_build(int nvox, const uint32_t *vox_blk, int64_t nseg_blk, int32
     if ((e = scan_i32(counts, off64, nvox, stmp, st)) != cudaSuccess) return e;
     k_off32<<<(nvox + 256) / 256, 256, 0, st>>>(off64, csr_off, nvox + 1);
     if (nseg_blk <= 0) return cudaGetLastError();
-    int bits = 0;
-    while (bits < 31 && ((int64_t)1 << bits) < (int64_t)nvox) ++bits;
-    return radix_order(vox_blk, nseg_blk, bits, perm_blk, rs, st);
+    return radix_order(vox_blk, nseg_blk, voxel_bits(nvox), perm_blk, rs, st);
 }
 
 cudaError_t csr_invL(int nvox, const int32_t *csr_off, const int32_t *perm_blk, const double *len64_blk,

@@ -786,7 +786,7 @@ int run_fs(rt_grid *g, int prec, int homog, const double *S_src, double *J, doub
                                      g->d_part, J, L, Fc, b == 0, g->st));
             tstop(g, t1, 1, ns);
         }
-        g->launches += 3;
+        g->launches += 2 + (g->h_mbase[b + 1] > g->h_mbase[b] ? 1 : 0);
     }
     if (F) {
         CK(flux_local(g->G, Fc, F, g->st));
@@ -1004,8 +1004,10 @@ bool bun_setup(rt_grid *g)
             !ok(radix_order(key, n, bits, order + r0, rs, g->st)) ||
             !ok(ray64_order(r0, n, g->d_ray_off, order, rlen, g->st)))
             return false;
+        g->launches += n > 0 ? 2 + radix_launches(n, bits) : 0;
     }
     if (!ok(scan_i32(rlen, boff, g->n_rays, stmp, g->st))) return false;
+    g->launches += 1 + scan_launches(g->n_rays);
     std::vector<Bun32> bp;
     std::vector<SwGather> bg;
     std::vector<int64_t> segs, bytes;
@@ -1079,7 +1081,8 @@ bool bun_setup(rt_grid *g)
         bytes.push_back(20 * p.ns + 8 * nu + 4 * nd);
         max_units = std::max(max_units, nu);
         max_chunks = std::max(max_chunks, tots[1]);
-        g->launches += 30;
+        g->launches += m.nbun > 0 ? 4 + 2 * scan_launches(m.nbun) : 0;
+        g->launches += csr_launches(nvox, nu) + (nu > 0 ? 1 : 0) + 1 + 2 * scan_launches(nvox) + (tots[0] > 0 ? 1 : 0);
     }
     double *part = (double *)kget(8 * max_chunks);
     void *buf[3];
@@ -1134,8 +1137,9 @@ bool use_bun(rt_grid *g)
     }
     if (!u.cw_ok) {
         for (const Bun32 &m : u.part) {
-            if (m.nbun > 0 && bun_coef(m, g->d_vox, g->d_len64, g->d_chi, g->d_ray_angle, g->d_wt, g->d_invL, g->nvox,
-                                       g->st) != cudaSuccess)
+            if (m.nbun <= 0) continue;
+            if (bun_coef(m, g->d_vox, g->d_len64, g->d_chi, g->d_ray_angle, g->d_wt, g->d_invL, g->nvox, g->st) !=
+                cudaSuccess)
                 return false;
             g->launches++;
         }
@@ -1288,7 +1292,8 @@ bool ray64_setup(rt_grid *g)
         cudaMemcpyAsync(&slots, g->d_rgbase + ng, sizeof(int64_t), cudaMemcpyDeviceToHost, g->st) != cudaSuccess ||
         cudaStreamSynchronize(g->st) != cudaSuccess)
         return false;
-    g->launches += 4 + 12 * g->nblk;
+    g->launches += 1 + scan_launches(ng);
+    for (int b = 0; b < g->nblk; ++b) g->launches += csr_launches(cap + 1, nrays(b)) + (nrays(b) > 0 ? 2 : 0);
     g->d_wp64 = (uint2 *)keep_alloc(g, sizeof(uint2) * (size_t)slots);
     g->d_cw64 = (Wd4 *)keep_alloc(g, sizeof(Wd4) * (size_t)slots);
     g->d_cg64 = (double *)keep_alloc(g, sizeof(double) * (size_t)slots);
@@ -1824,7 +1829,7 @@ int nn_lstar_into(rt_grid *g, const double *chi, const uint32_t *pbits, double *
         un.multi = g->d_multi + g->h_mbase[b];
         un.nmulti = g->h_mbase[b + 1] - g->h_mbase[b];
         CK(nn_gather(n, g->d_csr_off + (size_t)b * (n + 1), g->d_perm + a.seg_lo, slot, val, un, part, L27, b == 0, st));
-        g->launches += 4;
+        g->launches += 3 + (un.nmulti > 0 ? 1 : 0);
     }
     return RT_OK;
 }

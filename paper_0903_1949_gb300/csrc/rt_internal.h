@@ -76,6 +76,7 @@ cudaError_t geom_complete_pred(const GeomDev &G, const GeomF &F, const double *d
 // out[0] = 0, out[i+1] = out[i] + in[i]  (n + 1 outputs); tmp holds >= scan_tmp_elems(n) int64.
 int64_t scan_tmp_elems(int64_t n);
 cudaError_t scan_i32(const int32_t *in, int64_t *out, int64_t n, int64_t *tmp, cudaStream_t st);
+int scan_launches(int64_t n);  // kernels it launches
 cudaError_t gather_i64(const int64_t *src, const int64_t *idx, int64_t *dst, int n, cudaStream_t st);
 
 // ---- ownership lists and gather (gather.cu) ----
@@ -90,10 +91,13 @@ struct RadixScratch {
     int64_t cap;
 };
 int64_t radix_tiles(int64_t n);
-// Ownership (CSR) lists of one angle block: csr_off (nvox + 1) and perm_blk, every
-// voxel's segment indices in increasing order.
+// Kernels that radix_order and csr_build launch.
+int radix_launches(int64_t n, int bits);
+int csr_launches(int nvox, int64_t n);
 // Indices 0..n-1 in the order of their keys' low `bits` bits, stable.
 cudaError_t radix_order(const uint32_t *key, int64_t n, int bits, int32_t *perm, const RadixScratch &rs, cudaStream_t st);
+// Ownership (CSR) lists of one angle block: csr_off (nvox + 1) and perm_blk, every
+// voxel's segment indices in increasing order.
 cudaError_t csr_build(int nvox, const uint32_t *vox_blk, int64_t nseg_blk, int32_t *counts, int32_t *csr_off,
                       int32_t *perm_blk, int64_t *tmp, const RadixScratch &rs, cudaStream_t st);
 cudaError_t csr_invL(int nvox, const int32_t *csr_off, const int32_t *perm_blk, const double *len64_blk,

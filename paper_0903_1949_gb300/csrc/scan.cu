@@ -111,6 +111,8 @@ cudaError_t scan_i32(const int32_t *in, int64_t *out, int64_t n, int64_t *tmp, c
     return cudaGetLastError();
 }
 
+int scan_launches(int64_t n) { return n > 0 ? 3 : 1; }
+
 cudaError_t gather_i64(const int64_t *src, const int64_t *idx, int64_t *dst, int n, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
