@@ -12,6 +12,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -860,6 +861,40 @@ bool sw_bounds(rt_grid *g)
     return true;
 }
 
+// Device arrays that share one allocation (a cudaMalloc and its cudaFree cost as much
+// as several of the small kernels that use them): want() each, then get() once.
+struct Shared {
+    std::vector<std::function<void(char *)>> set;
+    size_t size = 0;
+    void *base = nullptr;
+    template <typename T>
+    void want(T *&p, int64_t n)
+    {
+        const size_t at = size;
+        p = nullptr;
+        set.push_back([&p, at](char *b) { p = reinterpret_cast<T *>(b + at); });
+        size += (sizeof(T) * (size_t)std::max<int64_t>(1, n) + 255) / 256 * 256;
+    }
+    bool get()
+    {
+        if (cudaMalloc(&base, std::max<size_t>(1, size)) != cudaSuccess) {
+            cudaGetLastError();
+            base = nullptr;
+            return false;
+        }
+        for (auto &f : set) f((char *)base);
+        return true;
+    }
+    // the allocation lives on with the grid
+    void keep(rt_grid *g)
+    {
+        g->allocs.push_back(base);
+        g->bytes += (int64_t)size;
+        base = nullptr;
+    }
+    ~Shared() { cudaFree(base); }
+};
+
 // Bundles of the mixed J-only formal solution (once per grid): parts of at most
 // BUN_PART segments (whole angle blocks), each one launch of the march and of the
 // gather: small enough that three parts' values (a quarter to a half of the segments,
@@ -964,38 +999,48 @@ bool bun_setup(rt_grid *g)
     const int64_t nhist = 256 * radix_tiles(rs.cap);
     int64_t nbun_max = 1;
     for (int64_t q : nbun) nbun_max = std::max(nbun_max, q);
-    rs.kA = (uint32_t *)tmp.get(4 * rs.cap);
-    rs.kB = (uint32_t *)tmp.get(4 * rs.cap);
-    rs.vA = (int32_t *)tmp.get(4 * rs.cap);
-    rs.vB = (int32_t *)tmp.get(4 * rs.cap);
-    rs.hist = (int32_t *)tmp.get(4 * nhist);
-    rs.off = (int64_t *)tmp.get(8 * (nhist + 1));
-    rs.tmp = (int64_t *)tmp.get(8 * scan_tmp_elems(nhist));
-    uint32_t *key = (uint32_t *)tmp.get(4 * nr_max), *tv = (uint32_t *)tmp.get(4 * ns_max);
-    uint32_t *tb = (uint32_t *)tmp.get(4 * ns_max), *td = (uint32_t *)tmp.get(4 * ns_max);
-    uint32_t *uvox = (uint32_t *)tmp.get(4 * ns_max);
-    int32_t *perm = (int32_t *)tmp.get(4 * ns_max), *rlen = (int32_t *)tmp.get(4 * g->n_rays);
-    int32_t *cnt = (int32_t *)tmp.get(4 * nvox), *hist = (int32_t *)tmp.get(4 * 128), *lflag = (int32_t *)tmp.get(4 * nvox);
-    int32_t *nch = (int32_t *)tmp.get(4 * nvox), *lrows = (int32_t *)tmp.get(4 * nvox);
-    int32_t *nunit = (int32_t *)tmp.get(4 * nbun_max), *ndist = (int32_t *)tmp.get(4 * nbun_max);
-    int64_t *doff = (int64_t *)tmp.get(8 * (nbun_max + 1));
-    const int64_t nscan = std::max<int64_t>(std::max<int64_t>(nvox + 1, nbun_max + 1), g->n_rays);
-    int64_t *pos1 = (int64_t *)tmp.get(8 * (nvox + 1)), *pos2 = (int64_t *)tmp.get(8 * (nvox + 1));
-    int64_t *uoff = (int64_t *)tmp.get(8 * (nbun_max + 1)), *stmp = (int64_t *)tmp.get(8 * scan_tmp_elems(nscan));
-    int64_t *ctmp = (int64_t *)tmp.get(8 * ((int64_t)nvox + 1 + scan_tmp_elems(nvox)));
-    int64_t *boff = (int64_t *)kget(8 * (g->n_rays + 1));
-    int32_t *order = (int32_t *)kget(4 * g->n_rays);
-    int32_t *sray = (int32_t *)kget(4 * nsub_all), *sseg = (int32_t *)kget(4 * nsub_all);
-    float4 *cw = (float4 *)kget(16 * slots);
-    uint32_t *wd = (uint32_t *)kget(4 * slots);
-    int32_t *off = (int32_t *)kget(4 * (int64_t)parts.size() * (nvox + 1));
-    int2 *ub_all = (int2 *)kget(8 * nsub_all);  // more than a bundle needs
-    for (void *q : {(void *)rs.kA, (void *)rs.kB, (void *)rs.vA, (void *)rs.vB, (void *)rs.hist, (void *)rs.off,
-                    (void *)rs.tmp, (void *)key, (void *)tv, (void *)tb, (void *)td, (void *)uvox, (void *)ndist, (void *)doff, (void *)perm, (void *)rlen, (void *)cnt,
-                    (void *)hist, (void *)lflag, (void *)nch, (void *)lrows, (void *)nunit, (void *)pos1, (void *)pos2,
-                    (void *)uoff, (void *)stmp, (void *)ctmp, (void *)boff, (void *)order, (void *)sray, (void *)sseg,
-                    (void *)cw, (void *)wd, (void *)off, (void *)ub_all})
-        if (!q) return false;
+    Shared work, tabs;
+    uint32_t *key, *tv, *tb, *td, *uvox, *wd;
+    int32_t *perm, *rlen, *cnt, *hist, *lflag, *nch, *lrows, *nunit, *ndist, *order, *sray, *sseg, *off;
+    int64_t *doff, *pos1, *pos2, *uoff, *stmp, *ctmp, *boff;
+    float4 *cw;
+    int2 *ub_all;
+    work.want(rs.kA, rs.cap);
+    work.want(rs.kB, rs.cap);
+    work.want(rs.vA, rs.cap);
+    work.want(rs.vB, rs.cap);
+    work.want(rs.hist, nhist);
+    work.want(rs.off, nhist + 1);
+    work.want(rs.tmp, scan_tmp_elems(nhist));
+    work.want(key, nr_max);
+    work.want(tv, ns_max);
+    work.want(tb, ns_max);
+    work.want(td, ns_max);
+    work.want(uvox, ns_max);
+    work.want(perm, ns_max);
+    work.want(rlen, g->n_rays);
+    work.want(cnt, nvox);
+    work.want(hist, RTK_JSHORT + 1);
+    work.want(lflag, nvox);
+    work.want(nch, nvox);
+    work.want(lrows, nvox);
+    work.want(nunit, nbun_max);
+    work.want(ndist, nbun_max);
+    work.want(doff, nbun_max + 1);
+    work.want(uoff, nbun_max + 1);
+    work.want(pos1, nvox + 1);
+    work.want(pos2, nvox + 1);
+    work.want(stmp, scan_tmp_elems(std::max<int64_t>(std::max<int64_t>(nvox + 1, nbun_max + 1), g->n_rays)));
+    work.want(ctmp, (int64_t)nvox + 1 + scan_tmp_elems(nvox));
+    tabs.want(boff, g->n_rays + 1);
+    tabs.want(order, g->n_rays);
+    tabs.want(sray, nsub_all);
+    tabs.want(sseg, nsub_all);
+    tabs.want(cw, slots);
+    tabs.want(wd, slots);
+    tabs.want(off, (int64_t)parts.size() * (nvox + 1));
+    tabs.want(ub_all, nsub_all);  // more than a bundle needs
+    if (!work.get() || !tabs.get()) return false;
     for (const Part &p : parts) {  // sorted order of the characteristics
         const int64_t r0 = g->h_ang_ray_off[p.a0], n = g->h_ang_ray_off[p.a0 + p.na] - r0;
         int bits = 0;
@@ -1094,6 +1139,7 @@ bool bun_setup(rt_grid *g)
         return false;
     for (Bun32 &m : bp) m.dmax = hs[1];
     for (SwGather &t : bg) t.part = part;
+    tabs.keep(g);
     g->allocs.insert(g->allocs.end(), keep.v.begin(), keep.v.end());
     keep.v.clear();
     g->bytes += kept;
@@ -1111,9 +1157,9 @@ bool bun_setup(rt_grid *g)
 // solid angle cross a voxel: 5.9 on spherical grids, 2.8 on cylindrical ones, where
 // most lookups and sums stay a voxel's only ones.  Iterations after which a new grid
 // gains (march in launch order -> bundles, and the tables, ms): 8.4e8 segments
-// spherical 50 (6.76 -> 4.33, 122), 2.1e8 51 (1.76 -> 1.13, 32), 5.4e7 60 (0.485 ->
-// 0.331, 9.3); 2.6e7 137, 6.5e6 100, 3.3e6 170, 8e5 above 1000; cylindrical 2e8 450
-// (1.60 -> 1.52, 37), 5.1e7 1000, 6.4e6 460.
+// spherical 50 (6.76 -> 4.37, 121), 2.1e8 62 (1.76 -> 1.27, 30), 5.4e7 98 (0.485 ->
+// 0.40, 8.3); 2.6e7 and less 140 to 1000; cylindrical 2e8 450 (1.60 -> 1.52, 37),
+// 5.1e7 1000, 6.4e6 460.
 bool bun_pays(const rt_grid *g)
 {
     return g->n_seg >= 40000000 && g->n_seg >= (int64_t)4 * g->n_ang * g->nvox;
@@ -1215,19 +1261,6 @@ Ray64 ray64_block(rt_grid *g, int b)
     return m;
 }
 
-// Device memory that lives as long as the grid, counted; NULL when it does not fit.
-void *keep_alloc(rt_grid *g, size_t bytes)
-{
-    void *q = nullptr;
-    if (cudaMalloc(&q, std::max<size_t>(1, bytes)) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    g->allocs.push_back(q);
-    g->bytes += (int64_t)bytes;
-    return q;
-}
-
 // The slots of the FP64 streamed march (once per grid): characteristics sorted
 // by length within their angle blocks, groups of 32, one slot per step and
 // characteristic.  false when the arrays do not fit.
@@ -1243,42 +1276,28 @@ bool ray64_setup(rt_grid *g)
         rs.cap = std::max(rs.cap, nrays(b));
     }
     const int64_t ng = g->h_rg0[g->nblk];
-    struct Tmp {
-        std::vector<void *> v;
-        ~Tmp()
-        {
-            for (void *q : v) cudaFree(q);
-        }
-        void *get(size_t bytes)
-        {
-            void *q = nullptr;
-            if (cudaMalloc(&q, bytes) != cudaSuccess) {
-                cudaGetLastError();
-                return nullptr;
-            }
-            v.push_back(q);
-            return q;
-        }
-    } tmp;
     const int64_t nhist = 256 * radix_tiles(rs.cap);
-    rs.kA = (uint32_t *)tmp.get(4 * (size_t)rs.cap);
-    rs.kB = (uint32_t *)tmp.get(4 * (size_t)rs.cap);
-    rs.vA = (int32_t *)tmp.get(4 * (size_t)rs.cap);
-    rs.vB = (int32_t *)tmp.get(4 * (size_t)rs.cap);
-    rs.hist = (int32_t *)tmp.get(4 * (size_t)nhist);
-    rs.off = (int64_t *)tmp.get(8 * (size_t)(nhist + 1));
-    rs.tmp = (int64_t *)tmp.get(8 * (size_t)scan_tmp_elems(nhist));
-    uint32_t *key = (uint32_t *)tmp.get(4 * (size_t)g->n_rays);
-    int32_t *cnt = (int32_t *)tmp.get(4 * (size_t)(cap + 1)), *coff = (int32_t *)tmp.get(4 * (size_t)(cap + 2));
-    int64_t *ctmp = (int64_t *)tmp.get(8 * (size_t)(cap + 2 + scan_tmp_elems(cap + 1)));
-    int32_t *gw = (int32_t *)tmp.get(4 * std::max<int64_t>(1, ng));
-    int64_t *stmp = (int64_t *)tmp.get(8 * (size_t)scan_tmp_elems(ng));
-    g->d_rorder = (int32_t *)keep_alloc(g, 4 * (size_t)g->n_rays);
-    g->d_rlen = (int32_t *)keep_alloc(g, 4 * (size_t)g->n_rays);
-    g->d_rgbase = (int64_t *)keep_alloc(g, 8 * (size_t)(ng + 1));
-    if (!rs.kA || !rs.kB || !rs.vA || !rs.vB || !rs.hist || !rs.off || !rs.tmp || !key || !cnt || !coff || !ctmp || !gw ||
-        !stmp || !g->d_rorder || !g->d_rlen || !g->d_rgbase)
-        return false;
+    Shared work, tabs, streams;
+    uint32_t *key;
+    int32_t *cnt, *coff, *gw;
+    int64_t *ctmp, *stmp;
+    work.want(rs.kA, rs.cap);
+    work.want(rs.kB, rs.cap);
+    work.want(rs.vA, rs.cap);
+    work.want(rs.vB, rs.cap);
+    work.want(rs.hist, nhist);
+    work.want(rs.off, nhist + 1);
+    work.want(rs.tmp, scan_tmp_elems(nhist));
+    work.want(key, g->n_rays);
+    work.want(cnt, cap + 1);
+    work.want(coff, cap + 2);
+    work.want(ctmp, cap + 2 + scan_tmp_elems(cap + 1));
+    work.want(gw, ng);
+    work.want(stmp, scan_tmp_elems(ng));
+    tabs.want(g->d_rorder, g->n_rays);
+    tabs.want(g->d_rlen, g->n_rays);
+    tabs.want(g->d_rgbase, ng + 1);
+    if (!work.get() || !tabs.get()) return false;
     // stable: characteristics of one length stay in launch order, so that the lanes
     // of a group have neighbouring origins and look up neighbouring voxels
     if (ray64_keys(g->n_rays, g->d_ray_off, cap, key, g->st) != cudaSuccess) return false;
@@ -1294,10 +1313,13 @@ bool ray64_setup(rt_grid *g)
         return false;
     g->launches += 1 + scan_launches(ng);
     for (int b = 0; b < g->nblk; ++b) g->launches += csr_launches(cap + 1, nrays(b)) + (nrays(b) > 0 ? 2 : 0);
-    g->d_wp64 = (uint2 *)keep_alloc(g, sizeof(uint2) * (size_t)slots);
-    g->d_cw64 = (Wd4 *)keep_alloc(g, sizeof(Wd4) * (size_t)slots);
-    g->d_cg64 = (double *)keep_alloc(g, sizeof(double) * (size_t)slots);
-    return g->d_wp64 && g->d_cw64 && g->d_cg64;
+    streams.want(g->d_wp64, slots);
+    streams.want(g->d_cw64, slots);
+    streams.want(g->d_cg64, slots);
+    if (!streams.get()) return false;
+    tabs.keep(g);
+    streams.keep(g);
+    return true;
 }
 
 // Whether full FP64 formal solutions run on the streamed weights, whose results differ
@@ -1326,12 +1348,7 @@ bool use_sw64(rt_grid *g)
 {
     if (!g->sw_enabled || g->sw64_state < 0) return false;
     if (g->sw64_state == 0) {
-        const int64_t before = g->bytes;
-        if (!ray64_setup(g)) {
-            g->bytes = before;
-            for (void *q : {(void *)g->d_rorder, (void *)g->d_rlen, (void *)g->d_rgbase, (void *)g->d_wp64,
-                            (void *)g->d_cw64, (void *)g->d_cg64})
-                dfree(g, q);
+        if (!ray64_setup(g)) {  // nothing of it is kept
             g->d_rorder = g->d_rlen = nullptr;
             g->d_rgbase = nullptr;
             g->d_wp64 = nullptr;
