@@ -763,7 +763,7 @@ int run_fs(rt_grid *g, int prec, int homog, const double *S_src, double *J, doub
             else
                 CK(march_block<double, double2>(g->d_vox, g->d_len64, g->d_ray_off, r_lo, r_hi, lo, ns, g->d_cs64,
                                                 g->d_B, g->I_outer, homog, para, buf, g->chunk(), g->st));
-            tstop(g, t0, 0, ns, (ray ? 44 : 12) * ns);
+            tstop(g, t0, 0, ns, (ray ? 48 : 12) * ns);
             t1 = tstart(g, 1);
             CK(gather_block<double2>(n, off, g->d_perm + lo, buf, g->d_ang_seg_off, w0, nw, lo, g->d_invL, g->d_wL32,
                                      g->d_wt, g->d_dirs, g->d_urow + g->h_ubase[b], g->d_ubeg + g->h_ubase[b],
