@@ -1032,12 +1032,12 @@ bool bun_setup(rt_grid *g)
     work.want(pos2, nvox + 1);
     work.want(stmp, scan_tmp_elems(std::max<int64_t>(std::max<int64_t>(nvox + 1, nbun_max + 1), g->n_rays)));
     work.want(ctmp, (int64_t)nvox + 1 + scan_tmp_elems(nvox));
+    tabs.want(cw, slots);
+    tabs.want(wd, slots);
     tabs.want(boff, g->n_rays + 1);
     tabs.want(order, g->n_rays);
     tabs.want(sray, nsub_all);
     tabs.want(sseg, nsub_all);
-    tabs.want(cw, slots);
-    tabs.want(wd, slots);
     tabs.want(off, (int64_t)parts.size() * (nvox + 1));
     tabs.want(ub_all, nsub_all);  // more than a bundle needs
     if (!work.get() || !tabs.get()) return false;
@@ -1313,8 +1313,8 @@ bool ray64_setup(rt_grid *g)
         return false;
     g->launches += 1 + scan_launches(ng);
     for (int b = 0; b < g->nblk; ++b) g->launches += csr_launches(cap + 1, nrays(b)) + (nrays(b) > 0 ? 2 : 0);
-    streams.want(g->d_wp64, slots);
     streams.want(g->d_cw64, slots);
+    streams.want(g->d_wp64, slots);
     streams.want(g->d_cg64, slots);
     if (!streams.get()) return false;
     tabs.keep(g);
