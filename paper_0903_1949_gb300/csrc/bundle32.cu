@@ -21,16 +21,19 @@
 // warp's values 32 places apart: without the order by length the additions took
 // twice the instructions.
 //
-// Measured, one GB300, per formal solution: 8.4e8 segments (65 x 33 x 65 voxels x
-// 32 x 32 solid angles) 6.75 -> 4.3 ms, 2e8 (65^3 cylindrical x 16 x 16) 1.63 ->
-// 1.54 ms.  A part of 1.1e7 segments takes 66 us and moves 25.7 bytes a segment
-// to and from HBM (20 of them its stream), 4.2 of 6.8 TB/s; with S, the sums and
-// the scan left out the same stream takes 3.8 of the 4.3 ms, so what is left is
-// the HBM latency that 32 warps an SM (64 registers, 40 kB of shared memory a
-// bundle) cover.  Not better: two segments a lane and five CTAs an SM (4.8 ms),
-// persistent CTAs that fetch the next bundle's S during the additions (4.9),
-// bundles of 8192 (5.5 without the order by length).  The tables cost about
-// 0.12 s once per grid at 8.4e8 segments.
+// Below 1000 solid angles a unit's sum is two floats (BUN_PAIR in rt_api.cu), and only
+// grids on which the tables pay take this march by default (bun_pays there).
+//
+// Measured, one GB300, per formal solution against the march in launch order: 8.4e8
+// segments (65 x 33 x 65 voxels x 32 x 32 solid angles) 6.76 -> 4.33 ms, 2.1e8 (16 x 16,
+// two floats) 1.76 -> 1.27, 2e8 (65^3 cylindrical x 16 x 16) 1.60 -> 1.52.  A part of
+// 6.2e6 segments takes 41 us and moves 25 bytes a segment to and from HBM (20 of them
+// its stream), 3.8 of 6.8 TB/s; with S, the sums and the scan left out the same
+// stream took 3.8 of the 4.3 ms, so what is left is the HBM latency that 32 warps an SM
+// (64 registers, 40 kB of shared memory a bundle) cover.  Not better: two segments a
+// lane and five CTAs an SM (4.8 ms), persistent CTAs that fetch the next bundle's S
+// during the additions (4.9), bundles of 8192 (5.5 without the order by length).  The
+// tables cost about 0.12 s once per grid at 8.4e8 segments.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -622,7 +625,7 @@ cudaError_t bun_bounds(const Bun32 &m, int64_t nseg, int32_t *sray, int32_t *sse
 }
 
 cudaError_t bun_units(const Bun32 &m, int nvox, const uint32_t *vox, uint32_t *tv, uint32_t *tb, uint32_t *td, int32_t *nunit,
-                      int32_t *ndist, int *err,                      cudaStream_t st)
+                      int32_t *ndist, int *err, cudaStream_t st)
 {
     static std::atomic<uint64_t> done32{0}, done64{0};
     if (nvox <= 1 << 19) {

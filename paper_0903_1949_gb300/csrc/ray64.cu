@@ -12,11 +12,12 @@
 // an angle block are sorted by length, 32 of a warp have nearly the same one,
 // and the streams are stored by step across them (slot = group base + 32 k +
 // lane), so that every load of a step but the S lookups is one coalesced
-// request; the next two steps' are in flight while one is computed.  Measured
-// on 65 x 33 x 65 voxels with 16 x 16 solid angles (2.1e8 segments, 37 angle
-// blocks): the ALI iteration takes 3.77 ms, 7.21 ms with the warp scan; one
-// sweep of the adjoint iteration on 33 x 17 x 33 x 64 (6.5e6 segments) 0.18 ms
-// with its gather, 1.9 ms with the march that evaluates the weights each time.
+// request; what is in flight meanwhile stands beside each kernel.  Measured on
+// 65 x 33 x 65 voxels with 16 x 16 solid angles (2.1e8 segments, 37 angle blocks): the
+// ALI iteration takes 3.4 ms, 7.2 ms with the warp scan; a block's march 98 us with the
+// FP64 pipe 60 % active.  One sweep of the adjoint iteration on 33 x 17 x 33 x 64 (6.5e6
+// segments) takes 0.18 ms with its gather, 1.9 ms with the march that evaluates the
+// weights each time.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

@@ -300,7 +300,7 @@ cudaError_t bun_keys(const int64_t *ray_off, int64_t r_lo, int64_t n, const uint
 cudaError_t bun_maxlen(int64_t n_rays, const int64_t *ray_off, int32_t *mx, cudaStream_t st);
 cudaError_t bun_bounds(const Bun32 &m, int64_t nseg, int32_t *sray, int32_t *sseg, cudaStream_t st);
 cudaError_t bun_units(const Bun32 &m, int nvox, const uint32_t *vox, uint32_t *tv, uint32_t *tb, uint32_t *td, int32_t *nunit,
-                      int32_t *ndist, int *err,                      cudaStream_t st);
+                      int32_t *ndist, int *err, cudaStream_t st);
 cudaError_t bun_ub(int nbun, const int64_t *uoff, const int64_t *doff, int2 *ub, int32_t *mx, cudaStream_t st);
 cudaError_t bun_compact(const Bun32 &m, const uint32_t *tv, const uint32_t *tb, const uint32_t *td, uint32_t *uvox,
                         cudaStream_t st);
