@@ -208,23 +208,82 @@ constexpr size_t units_smem()
     return sizeof(KEY) * SORT_CAP + sizeof(uint32_t) * SORT_CAP + 2 * sizeof(uint16_t) * (SORT_CAP + 8);
 }
 
+// One stable pass of a radix sort over the CTA: n <= SORT_CAP items get(i) go to dst in
+// the order of their digit (get(i) >> shift) & (2^bits - 1), place i at dst[put(i)].  A warp
+// takes a run of SORT_CAP / 32 items; items of one digit in a warp are ranked by
+// __match_any_sync.
+constexpr int DIGIT = 6;
+struct RadixSmem {
+    uint16_t cnt[UT / 32][1 << DIGIT];
+    int sh[32];
+};
+template <typename G, typename P>
+__device__ __forceinline__ void cta_radix_pass(RadixSmem &r, G get, P put, uint32_t *dst, int n, int shift, int bits)
+{
+    constexpr int R = SORT_CAP / UT;  // items of a thread
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, mask = (1 << bits) - 1;
+    for (int d = lane; d < 1 << DIGIT; d += 32) r.cnt[w][d] = 0;
+    __syncwarp();
+    uint32_t x[R];
+    int at[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int i = w * (SORT_CAP / 32) + 32 * q + lane;
+        const bool on = i < n;
+        x[q] = on ? get(i) : 0u;
+        const int d = on ? (int)(x[q] >> shift) & mask : 1 << DIGIT;
+        const unsigned same = __match_any_sync(FULL, d), below = same & ((1u << lane) - 1u);
+        const int before = on ? r.cnt[w][d] : 0;
+        at[q] = before + __popc(below);
+        __syncwarp();
+        if (on && below == 0u) r.cnt[w][d] = (uint16_t)(before + __popc(same));
+        __syncwarp();
+    }
+    __syncthreads();
+    // first place of every (digit, warp): digits in order, a digit's warps in order
+    constexpr int E = (1 << DIGIT) * (UT / 32) / UT;  // counters of a thread
+    int c[E], sum = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int k = E * threadIdx.x + e;
+        c[e] = r.cnt[k % (UT / 32)][k / (UT / 32)];
+        sum += c[e];
+    }
+    int first = cta_scan<false>(sum, r.sh) - sum;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int k = E * threadIdx.x + e;
+        r.cnt[k % (UT / 32)][k / (UT / 32)] = (uint16_t)first;
+        first += c[e];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+        if (w * (SORT_CAP / 32) + 32 * q + lane < n) dst[put(r.cnt[w][(int)(x[q] >> shift) & mask] + at[q])] = x[q];
+    __syncthreads();
+}
+
 // Tables of one bundle per CTA (once per grid): its segments sorted by voxel,
 // stable in the order of the march; runs of a voxel cut into units of at most
 // BUN_RUN; the units sorted by falling length, so that the threads of a warp add
 // equally long ones; voxel (its number among the bundle's) and place of every
 // segment into its word.  The units' voxels, first places and lengths go to tv and
 // tb, the different voxels in order to td, each from the bundle's first segment on.
-// KEY: 32 bits hold (voxel, number in the bundle) on grids of up to 2^19 voxels.
+// KEY: 32 bits hold (voxel, number in the bundle) on grids of up to 2^19 voxels; they
+// are sorted by the voxel's vbits bits in radix passes (the bitonic sort, which 64-bit
+// keys keep, took half of the tables' time).
 template <typename KEY>
 __global__ void __launch_bounds__(UT, sizeof(KEY) == 4 ? 2 : 1)
-    k_bun_units(Bun32 m, const uint32_t *__restrict__ vox, uint32_t *__restrict__ tv, uint32_t *__restrict__ tb,
-                uint32_t *__restrict__ td, int32_t *__restrict__ nunit, int32_t *__restrict__ ndist, int *err)
+    k_bun_units(Bun32 m, int vbits, const uint32_t *__restrict__ vox, uint32_t *__restrict__ tv,
+                uint32_t *__restrict__ tb, uint32_t *__restrict__ td, int32_t *__restrict__ nunit,
+                int32_t *__restrict__ ndist, int *err)
 {
+    constexpr bool WIDE = sizeof(KEY) == 8;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int sh[32], gbase[SORT_CAP / 32];
-    KEY *key = reinterpret_cast<KEY *>(smem);
-    uint32_t *key2 = reinterpret_cast<uint32_t *>(key + SORT_CAP);  // sort of the units, then:
-    uint16_t *unit = reinterpret_cast<uint16_t *>(key2), *place = unit + SORT_CAP;
+    __shared__ RadixSmem rs;
+    KEY *key = reinterpret_cast<KEY *>(smem);  // the sorted segments
+    uint32_t *key2 = reinterpret_cast<uint32_t *>(key + SORT_CAP);  // sort of the units, then unit and place
     uint16_t *ustart = reinterpret_cast<uint16_t *>(key2 + SORT_CAP), *now = ustart + SORT_CAP + 8;
     const int64_t b = blockIdx.x;
     const int32_t *sr = m.sray + b * NW, *ss = m.sseg + b * NW;
@@ -238,17 +297,33 @@ __global__ void __launch_bounds__(UT, sizeof(KEY) == 4 ? 2 : 1)
     }
     int N = 8;
     while (N < n) N <<= 1;
-    for (int i = threadIdx.x; i < N; i += UT) key[padded(i)] = ~(KEY)0;
-    __syncthreads();
+    if (WIDE) {
+        for (int i = threadIdx.x; i < N; i += UT) key[padded(i)] = ~(KEY)0;
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31;
     for (int q = sr[0] + (threadIdx.x >> 5); q < sr[NW]; q += UT / 32) {
         const int64_t r = m.order[m.r_lo + q], s0 = m.ray_off[r];
         const int len = (int)(m.ray_off[r + 1] - s0), at = (int)(m.boff[m.r_lo + q] - m.seg_lo) - seg0;
         for (int i = lane; i < len; i += 32)
-            key[padded(at + i)] = (KEY)(vox[s0 + i] & RTK_VOXMASK) << 13 | (uint32_t)(at + i);
+            key[WIDE ? padded(at + i) : at + i] = (KEY)(vox[s0 + i] & RTK_VOXMASK) << 13 | (uint32_t)(at + i);
     }
     __syncthreads();
-    cta_sort(key, N);
+    if constexpr (WIDE) {
+        cta_sort(key, N);
+    } else {
+        const int passes = (vbits + DIGIT - 1) / DIGIT;
+        for (int q = 0; q < passes; ++q) {
+            const uint32_t *from = key;
+            const bool last = q == passes - 1;
+            cta_radix_pass(rs, [from](int i) { return from[i]; }, [last](int i) { return last ? padded(i) : i; }, key2, n,
+                           13 + DIGIT * q, min(DIGIT, vbits - DIGIT * q));
+            uint32_t *const t = key;
+            key = key2;
+            key2 = t;
+        }
+    }
+    uint16_t *unit = reinterpret_cast<uint16_t *>(key2), *place = unit + SORT_CAP;
     // first places of the voxels' runs, then heads of units
     const int p0 = threadIdx.x * UE;
     auto newvox = [&](int p) { return p == 0 || key[padded(p)] >> 13 != key[padded(p - 1)] >> 13; };
@@ -285,20 +360,18 @@ __global__ void __launch_bounds__(UT, sizeof(KEY) == 4 ? 2 : 1)
         ustart[U] = (uint16_t)n;
         nunit[b] = U;
     }
-    int N2 = 8;
-    while (N2 < U) N2 <<= 1;
     __syncthreads();
-    for (int i = threadIdx.x; i < N2; i += UT)
-        key2[padded(i)] = i < U ? (uint32_t)(BUN_RUN - (ustart[i + 1] - ustart[i])) << 16 | (uint32_t)i : ~0u;
-    __syncthreads();
-    cta_sort(key2, N2);
+    // units by falling length: one pass over 0 .. BUN_RUN - 1
+    static_assert(BUN_RUN <= 1 << DIGIT, "a length is one digit");
+    cta_radix_pass(rs, [ustart](int i) { return (uint32_t)(BUN_RUN - (ustart[i + 1] - ustart[i])) << 16 | (uint32_t)i; },
+                   [](int i) { return i; }, key2, U, 16, DIGIT);
     const int ng = (U + 31) / 32;  // at most SORT_CAP / 32 = 256 groups
-    const int glen = (int)threadIdx.x < ng ? 32 * (BUN_RUN - (int)(key2[padded(32 * threadIdx.x)] >> 16)) : 0;
+    const int glen = (int)threadIdx.x < ng ? 32 * (BUN_RUN - (int)(key2[32 * threadIdx.x] >> 16)) : 0;
     const int gend = cta_scan<false>(glen, sh);
     if ((int)threadIdx.x < ng) gbase[threadIdx.x] = gend - glen;
     __syncthreads();
     for (int i = threadIdx.x; i < U; i += UT) {
-        const int o = (int)(key2[padded(i)] & 0xffffu), s = ustart[o];
+        const int o = (int)(key2[i] & 0xffffu), s = ustart[o];
         now[o] = (uint16_t)i;
         tv[seg0 + i] = (uint32_t)(key[padded(s)] >> 13);
         tb[seg0 + i] = (uint32_t)(gbase[i >> 5] + (i & 31)) | (uint32_t)(ustart[o + 1] - s) << 16;
@@ -628,14 +701,16 @@ cudaError_t bun_units(const Bun32 &m, int nvox, const uint32_t *vox, uint32_t *t
                       int32_t *ndist, int *err, cudaStream_t st)
 {
     static std::atomic<uint64_t> done32{0}, done64{0};
+    int vbits = 1;
+    while (vbits < 31 && (int64_t)1 << vbits < nvox) ++vbits;
     if (nvox <= 1 << 19) {
         const cudaError_t e = allow_smem(k_bun_units<uint32_t>, units_smem<uint32_t>(), done32);
         if (e != cudaSuccess) return e;
-        k_bun_units<uint32_t><<<(unsigned)m.nbun, UT, units_smem<uint32_t>(), st>>>(m, vox, tv, tb, td, nunit, ndist, err);
+        k_bun_units<uint32_t><<<(unsigned)m.nbun, UT, units_smem<uint32_t>(), st>>>(m, vbits, vox, tv, tb, td, nunit, ndist, err);
     } else {
         const cudaError_t e = allow_smem(k_bun_units<uint64_t>, units_smem<uint64_t>(), done64);
         if (e != cudaSuccess) return e;
-        k_bun_units<uint64_t><<<(unsigned)m.nbun, UT, units_smem<uint64_t>(), st>>>(m, vox, tv, tb, td, nunit, ndist, err);
+        k_bun_units<uint64_t><<<(unsigned)m.nbun, UT, units_smem<uint64_t>(), st>>>(m, vbits, vox, tv, tb, td, nunit, ndist, err);
     }
     return cudaGetLastError();
 }
