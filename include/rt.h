@@ -252,7 +252,7 @@ int rt_set_precision(rt_grid *g, int precision);
 /* RT_TUNE_BUNDLES (default 1): the streamed-weight RT_MIXED march takes bundles of
  * neighbouring characteristics whose values are added in shared memory on grids
  * where that pays: at least 4e7 crossing segments, four a voxel and solid angle on
- * average (their tables, once per grid, cost as much as the gain of 50 to 100
+ * average (their tables, once per grid, cost as much as the gain of 40 to 60
  * iterations there, and of more elsewhere).  2: on every grid whose tables fit.  Both
  * only with the default settings of RT_TUNE_MARCH_COARSEN, RT_TUNE_MARCH_CHUNK,
  * RT_TUNE_MARCH_STAGES and RT_TUNE_FOLD_WEIGHT and characteristics of at most 4096

@@ -26,14 +26,14 @@
 //
 // Measured, one GB300, per formal solution against the march in launch order: 8.4e8
 // segments (65 x 33 x 65 voxels x 32 x 32 solid angles) 6.76 -> 4.33 ms, 2.1e8 (16 x 16,
-// two floats) 1.76 -> 1.27, 2e8 (65^3 cylindrical x 16 x 16) 1.60 -> 1.52.  A part of
-// 6.2e6 segments takes 41 us and moves 25 bytes a segment to and from HBM (20 of them
-// its stream), 3.8 of 6.8 TB/s; with S, the sums and the scan left out the same
-// stream took 3.8 of the 4.3 ms, so what is left is the HBM latency that 32 warps an SM
-// (64 registers, 40 kB of shared memory a bundle) cover.  Not better: two segments a
-// lane and five CTAs an SM (4.8 ms), persistent CTAs that fetch the next bundle's S
-// during the additions (4.9), bundles of 8192 (5.5 without the order by length).  The
-// tables cost about 0.12 s once per grid at 8.4e8 segments.
+// two floats) 1.76 -> 1.24, 2e8 (65^3 cylindrical x 16 x 16) 1.60 -> 1.91, or 1.52 with
+// one float.  A part of 5.7e6 segments takes 41 to 43 us and moves 25.4 bytes a segment to
+// and from HBM (20 of them its stream), 3.4 of 6.8 TB/s; with S, the sums and the scan
+// left out the same stream took 3.8 of the 4.3 ms, so what is left is the HBM latency
+// that 32 warps an SM (64 registers, 40 kB of shared memory a bundle) cover.  Not
+// better: two segments a lane and five CTAs an SM (4.8 ms), persistent CTAs that fetch
+// the next bundle's S during the additions (4.9), bundles of 8192 (5.5 without the order
+// by length).  The tables cost about 0.09 s once per grid at 8.4e8 segments.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

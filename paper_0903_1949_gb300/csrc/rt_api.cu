@@ -1152,14 +1152,15 @@ bool bun_setup(rt_grid *g)
     return true;
 }
 
-// Whether the bundles of a grid pay for their tables.  The tables cost 0.15 to 0.2 ns a
-// segment once, and what an iteration gains depends on how many characteristics of a
-// solid angle cross a voxel: 5.9 on spherical grids, 2.8 on cylindrical ones, where
-// most lookups and sums stay a voxel's only ones.  Iterations after which a new grid
-// gains (march in launch order -> bundles, and the tables, ms): 8.4e8 segments
-// spherical 50 (6.76 -> 4.37, 121), 2.1e8 62 (1.76 -> 1.27, 30), 5.4e7 98 (0.485 ->
-// 0.40, 8.3); 2.6e7 and less 140 to 1000; cylindrical 2e8 450 (1.60 -> 1.52, 37),
-// 5.1e7 1000, 6.4e6 460.
+// Whether the bundles of a grid pay for their tables.  The tables cost 0.11 ns a segment
+// once (more on small grids), and what an iteration gains depends on how many
+// characteristics of a solid angle cross a voxel: 5.9 on spherical grids, 2.8 on
+// cylindrical ones, where most lookups and sums stay a voxel's only ones.  March in
+// launch order -> bundles, the tables, all in ms, and the iterations after which a new
+// grid gains: 8.4e8 segments spherical 6.72 -> 4.32, 92, 38; 2.1e8 1.76 -> 1.24, 24, 45;
+// 1.0e8 0.87 -> 0.69, 11, 61; 5.4e7 0.48 -> 0.37, 6.3, 59; 2.6e7 0.244 -> 0.228, 3.6, 233;
+// 2.0e7 0.208 -> 0.166, 3.0, 72; 6.5e6 0.092 -> 0.080, 1.0, 80; 8e5 equal; cylindrical
+// 2e8 1.60 -> 1.91, 5.1e7 0.46 -> 0.52 (two floats a unit; 1.52 and 0.44 with one).
 bool bun_pays(const rt_grid *g)
 {
     return g->n_seg >= 40000000 && g->n_seg >= (int64_t)4 * g->n_ang * g->nvox;
