@@ -89,7 +89,6 @@ struct Kv {  // the solve's vectors and constants
     int halo;       // halo reach in voxel index either side of the block's range
     int hcap;       // halo buffer length in shared memory (floats, a multiple of 4)
     int tile;       // the FP32 solve keeps its halos in shared memory
-    int own_rho;    // ... and takes (rh, r) from a reduction of its own
     int msm;        // ... and the block's FP32 rows M too
     int far;        // the halo leaves out the neighbours across the phi seam (cylindrical)
 };
@@ -700,9 +699,11 @@ __device__ __forceinline__ int bicgstab_tile(const Kv &a, double tol, int window
             __syncthreads();  // the own range's s and p are read before they change
             auto update = [&](int j, float4 t) {
                 float4 &r4 = reinterpret_cast<float4 *>(hr)[j], &p4 = reinterpret_cast<float4 *>(hp)[j];
-                r4 = make_float4(form_s(r4.x, t.x, om), form_s(r4.y, t.y, om), form_s(r4.z, t.z, om),
-                                 form_s(r4.w, t.w, om));
-                if (!OWN_RHO) p4 = form_p4(r4, p4, reinterpret_cast<const float4 *>(hv)[j], bt, om);
+                float4 r = r4, p, v;
+                if (!OWN_RHO) p = p4, v = reinterpret_cast<const float4 *>(hv)[j];
+                r = make_float4(form_s(r.x, t.x, om), form_s(r.y, t.y, om), form_s(r.z, t.z, om), form_s(r.w, t.w, om));
+                r4 = r;
+                if (!OWN_RHO) p4 = form_p4(r, p, v, bt, om);
             };
 #pragma unroll
             for (int u = 0; u < TPF; ++u) {
@@ -799,6 +800,8 @@ __device__ __forceinline__ int bicgstab_tile(const Kv &a, double tol, int window
     return it;
 }
 
+// OWN_RHO: the form of the FP32 solve, a kernel each.
+template <bool OWN_RHO>
 __global__ void __launch_bounds__(RT_, 1) k_os_solve(Kv a)
 {
     __shared__ double tot[4];
@@ -854,8 +857,7 @@ __global__ void __launch_bounds__(RT_, 1) k_os_solve(Kv a)
             if (round > 0 && !(mr < 0.5 * prev)) fp64 = true;  // the FP32 corrections stopped paying
             prev = mr;
             const int k = fp64 ? bicgstab(a, a.i64, 0.5 * a.jtol * mx, 64, bar, tot, lo, hi)
-                    : a.tile ? (a.own_rho ? bicgstab_tile<true>(a, TOL32 * mr, 16, bar, tot, lo, hi)
-                                          : bicgstab_tile<false>(a, TOL32 * mr, 16, bar, tot, lo, hi))
+                    : a.tile ? bicgstab_tile<OWN_RHO>(a, TOL32 * mr, 16, bar, tot, lo, hi)
                              : bicgstab(a, a.i32, TOL32 * mr, 16, bar, tot, lo, hi);
             if (k < 0) return;
             its += k;
@@ -909,9 +911,10 @@ __global__ void __launch_bounds__(RT_, 1) k_os_solve(Kv a)
 
 // blocks of the cooperative launch on the current device: SMs x resident
 // blocks per SM (at most OS_BLOCKS_PER_SM), cached per device
-cudaError_t os_blocks(int *nb)
+cudaError_t os_blocks(const void *kernel, bool own_rho, int *nb)
 {
-    static std::atomic<int> cache[64];
+    static std::atomic<int> caches[2][64];
+    std::atomic<int> *const cache = caches[own_rho];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -921,7 +924,7 @@ cudaError_t os_blocks(int *nb)
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) != cudaSuccess) return e;
     if (!coop) return cudaErrorNotSupported;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_os_solve, RT_, 0)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, RT_, 0)) != cudaSuccess) return e;
     if (per < 1) return cudaErrorLaunchOutOfResources;
     *nb = std::min(MAXB, sms * std::min(per, OS_BLOCKS_PER_SM));
     if (cached) cache[dev].store(*nb, std::memory_order_release);
@@ -933,7 +936,7 @@ cudaError_t os_blocks(int *nb)
 // (*msm = 1) when that fits too, beside the kernel's static shared memory on
 // the current device, with the kernel's attribute raised to it; 0 (the
 // global-memory solve) when even the halos do not fit.
-cudaError_t os_tile_smem(int hcap, int rows, int threads, size_t *smem, int *msm)
+cudaError_t os_tile_smem(const void *kernel, int hcap, int rows, int threads, size_t *smem, int *msm)
 {
     *smem = 0;
     *msm = 0;
@@ -942,15 +945,15 @@ cudaError_t os_tile_smem(int hcap, int rows, int threads, size_t *smem, int *msm
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
     cudaFuncAttributes fa{};
-    if ((e = cudaFuncGetAttributes(&fa, k_os_solve)) != cudaSuccess) return e;
+    if ((e = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return e;
     const size_t base = sizeof(float) * (3 * (size_t)hcap + 2 * (size_t)rows);
     const size_t full = base + sizeof(float) * 27 * (size_t)rows;
     if (base + fa.sharedSizeBytes > (size_t)optin) return cudaSuccess;
     const bool rows_too = full + fa.sharedSizeBytes <= (size_t)optin;
     const size_t want = rows_too ? full : base;
-    if ((e = cudaFuncSetAttribute(k_os_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want)) != cudaSuccess)
         return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_os_solve, threads, want)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, want)) != cudaSuccess) return e;
     if (per >= 1) {
         *smem = want;
         *msm = rows_too;
@@ -981,7 +984,8 @@ cudaError_t nn_os_solve(const NnOs &o, cudaStream_t st, double **x_out, int *kry
     const int n = o.nvox;
     if ((int64_t)o.n1 * o.n2 * o.n3 != (int64_t)n || n < 1) return cudaErrorInvalidValue;
     int nb = 0;
-    cudaError_t e = os_blocks(&nb);
+    const void *const kernel = o.own_rho ? (const void *)k_os_solve<true> : (const void *)k_os_solve<false>;
+    cudaError_t e = os_blocks(kernel, o.own_rho != 0, &nb);
     if (e != cudaSuccess) return e;
     Kv a{};
     a.n = n;
@@ -1017,7 +1021,6 @@ cudaError_t nn_os_solve(const NnOs &o, cudaStream_t st, double **x_out, int *kry
     a.kmax = std::max(1, o.kmax);
     a.jmax = std::max(1, o.jmax);
     a.stall = o.stall;
-    a.own_rho = o.own_rho;
     a.rows = (int)round4((N + nb - 1) / nb);
     // stencil reach in voxel index: n2 n3 + n3 + 1, and on the spherical grid also
     // the k neighbours across the phi seam (n3 - 1 away); across the cylindrical
@@ -1029,7 +1032,7 @@ cudaError_t nn_os_solve(const NnOs &o, cudaStream_t st, double **x_out, int *kry
     auto halo = [&](int64_t reach) {
         a.halo = (int)std::min<int64_t>(reach, N);
         a.hcap = (int)round4(std::min<int64_t>(N4, (int64_t)a.rows + 2 * (int64_t)a.halo + 8));
-        return os_tile_smem(a.hcap, a.rows, threads, &smem, &a.msm);
+        return os_tile_smem(kernel, a.hcap, a.rows, threads, &smem, &a.msm);
     };
     const int64_t n23 = (int64_t)o.n2 * o.n3;
     if ((e = halo(o.sph ? n23 + 2 * o.n3 : 2 * n23)) != cudaSuccess) return e;
@@ -1040,7 +1043,7 @@ cudaError_t nn_os_solve(const NnOs &o, cudaStream_t st, double **x_out, int *kry
     a.tile = smem > 0;
     if ((e = cudaMemsetAsync(a.ctl, 0, 8 * (size_t)(CTL_WORDS + 2 * PW * nb), st)) != cudaSuccess) return e;
     void *args[] = {&a};
-    if ((e = cudaLaunchCooperativeKernel((const void *)k_os_solve, dim3(nb), dim3(threads), args, smem, st)) != cudaSuccess)
+    if ((e = cudaLaunchCooperativeKernel(kernel, dim3(nb), dim3(threads), args, smem, st)) != cudaSuccess)
         return e;
     unsigned h[W_N];
     if ((e = cudaMemcpyAsync(h, a.ctl, sizeof(h), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
