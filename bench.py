@@ -388,7 +388,8 @@ def main():
     achieved = seg_per_launch * ALGO_BYTES_PER_SEGMENT / (march_avg_ms / 1e3) / 1e9
     achieved_design = seg_per_launch * bytes_per_seg / (march_avg_ms / 1e3) / 1e9
     peak, peak_src = hbm_peak()
-    traffic, traffic_src = ncu_traffic(seg_per_launch)
+    bundled = bytes_per_seg != 24.0  # 24 bytes a segment: the march in launch order, on grids where bundles do not pay
+    traffic, traffic_src = ncu_traffic(seg_per_launch) if bundled else (None, None)
     g.set_timing(1)  # every launch: march and gather shares of a step (informational window)
     k_info = max(2, args.steps // 4)
     ms_info = timed(g.ali_step, k_info)
@@ -513,15 +514,17 @@ def main():
                          "frac": achieved / peak, "traffic": traffic,
                          "traffic_over_algorithmic": (traffic / (ALGO_BYTES_PER_SEGMENT * seg_per_launch)
                                                       if traffic else None),
-                         "kernel": "k_march_bun (FP32 streamed-weight march of bundles of characteristics, J only)",
+                         "kernel": ("k_march_bun (FP32 streamed-weight march of bundles of characteristics, J only)"
+                                    if bundled else "k_march_sw (FP32 streamed-weight march in launch order, J only)"),
                          "algorithmic_bytes": "%d B per crossing segment (int32 voxel id + FP32 path length, the "
                                               "method's minimum stream)" % ALGO_BYTES_PER_SEGMENT,
                          "design_bytes": {"per_segment": bytes_per_seg, "achieved": achieved_design,
                                           "frac": achieved_design / peak,
                                           "what": "bytes this design streams per segment: four FP32 weights (E, alpha, "
-                                                  "beta, gamma, with the gather weight w l/L folded in), a u32 word "
-                                                  "(voxel and place in the bundle), and 8 bytes per unit and 4 per "
-                                                  "voxel of a bundle"},
+                                                  "beta, gamma, with the gather weight w l/L folded in) and "
+                                                  + ("a u32 word (voxel and place in the bundle), and 8 bytes per unit "
+                                                     "and 4 per voxel of a bundle" if bundled else
+                                                     "the segment's word and list place")},
                          "segments_per_launch": seg_per_launch, "avg_launch_ms": march_avg_ms,
                          "avg_launch_ms_events": march_event_ms,
                          "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs)" % peak_src if peak_src == "measured"

@@ -148,8 +148,9 @@ int rt_set_precision(rt_grid *g, int precision);
 
 /* Runtime tuning knobs (rt_tune).  RT_TUNE_MARCH_CHUNK: crossing segments per
  * warp bundle in the ray march, 64..16384 (default 512, which a grid too small to
- * give every SM 16 bundles halves down to 64 unless RT_TUNE_BUNDLES is 0); a bundle always holds whole
- * characteristics, so results do not depend on it beyond rounding. */
+ * give every SM 16 bundles halves down to 64 unless RT_TUNE_BUNDLES is 0); a
+ * bundle always holds whole characteristics, so results do not depend on it
+ * beyond rounding. */
 #define RT_TUNE_MARCH_CHUNK 1
 /* RT_TUNE_STREAMED_WEIGHTS (default 1): the J-only march of the ALI iteration
  * streams per-segment weights (E, alpha, beta, gamma) evaluated once per chi
