@@ -65,6 +65,14 @@ __device__ __forceinline__ double div64(double a, double q)
 __device__ __forceinline__ bool below_one(double x) { return (unsigned)__double2hiint(x) < 0x3ff00000u; }
 __device__ __forceinline__ bool below_half(double x) { return (unsigned)__double2hiint(x) < 0x3fe00000u; }
 
+// E below x = 1: 1 - e0, and from 1/2 on, where 1 - x is exact, x f1 + (1 - x); one FP64
+// instruction on operands chosen off that pipe.
+__device__ __forceinline__ double small_E(double x, double f1, double e0)
+{
+    const bool half = below_half(x);
+    return fma(half ? -1.0 : x, half ? e0 : f1, half ? 1.0 : 1.0 - x);
+}
+
 // h1(x) = (e^{-x} - 1 + x) / x^2 and h2(x) = f2(x) / x^2 (see below) on [0, 1]:
 // their values at 0 plus x times polynomials fitted to (h - h(0)) / x at Chebyshev
 // nodes (fit error 1e-18 of h, under FP64 rounding).
@@ -108,7 +116,7 @@ __device__ __forceinline__ double h2_small(double x)
 // f1 and f2 cancel catastrophically when evaluated from e0 at small x; below 1
 // they come from polynomials, above it from the exponential.  The three quotients
 // of the parabola share one.  The FP64 pipe bounds every kernel that
-// evaluates these: about 45 instructions of it for a small x and 44 for a large one
+// evaluates these: about 44 instructions of it for a small x and for a large one
 // (62 and 80 with the 19-term series, expm1 and divisions of Coef64Series).  Mean
 // errors of E, alpha, beta, gamma in half ulps of their terms, Coef64Series -> here:
 // below 0.5 0.27, 0.28, 0.49, 0.77 -> 0.27, 0.29, 0.50, 0.69; in [0.5, 1] 0.57, 0.74,
@@ -123,7 +131,7 @@ struct Coef64 {
             f1 = x * h1_small(x);
             f2 = (x * x) * h2_small(x);
             e0 = fma(-x, f1, x);
-            E = below_half(x) ? 1.0 - e0 : fma(x, f1, 1.0 - x);  // 1 - x is exact from 1/2 on
+            E = small_E(x, f1, e0);
         } else {
             E = exp(-x);
             e0 = 1.0 - E;
@@ -262,7 +270,7 @@ struct Coef64D {
             f1 = x * h1_small(x);
             f2 = (x * x) * h2_small(x);
             e0 = fma(-x, f1, x);
-            E = below_half(x) ? 1.0 - e0 : fma(x, f1, 1.0 - x);
+            E = small_E(x, f1, e0);
             g1 = k1;
             g2 = x * k2;
         } else {
